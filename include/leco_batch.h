@@ -105,8 +105,8 @@ leco_status leco_batch_encode(const void* const* d_vals, const uint64_t* n, cons
                               leco_column** out);
 
 /* Shape of the batched encode (a systems knob; the paper has no counterpart): values per pack item
- * (1024, 2048 or 4096: a run of consecutive short partitions of one column that the packer stages
- * with one copy and packs in one CTA) and fit CTAs per SM (2, 3 or 4: fewer keep more of each
+ * (1024, 2048 or 4096: the window of consecutive positions of one column that a warp of the packer
+ * takes at a time) and fit CTAs per SM (2, 3 or 4: fewer keep more of each
  * partition in L2 between the fit's two passes, more hide the exact solve's latency); ms is the
  * measured time of the chosen shape (leco_tune_batch_encode only). */
 typedef struct {
@@ -127,7 +127,7 @@ leco_status leco_tune_batch_encode(const void* const* d_vals, const uint64_t* n,
 
 /* A prepared batched encode replayed as one CUDA graph (§3.2.1 partitions, §3.1 fit, §3.3 packing,
  * as leco_batch_encode; the batching itself is this library's systems layer). Creation does the
- * host work once: the columns' tables and pack items go to the device, the plan reserves its device
+ * host work once: the columns' tables go to the device, the plan reserves its device
  * blocks (records, decode table, tile descriptors, fit scratch, and words for the widest stream each
  * column could have: 64 bits per value plus a polynomial coefficient block per partition that could
  * hold one), and the launches from the fit to the pack are captured in a CUDA graph in the encode

@@ -2,7 +2,6 @@
 // decode-table build and residual packing.
 #include "fit.cuh"
 #include "leco_internal.cuh"
-#include "tma.cuh"
 
 namespace leco {
 
@@ -19,121 +18,6 @@ __device__ __forceinline__ uint64_t part_begin(const uint64_t* starts, uint32_t 
   if (starts) return starts[p];
   const uint64_t s = p * (uint64_t)L;
   return s < n ? s : n;
-}
-
-// ------------------------------------------------------------------------------ staged partitions
-//
-// The fit and the packing read each partition's values twice or more, so a CTA stages the
-// partition in shared memory first: one 1-D bulk copy (TMA) of the 16-byte-aligned byte range
-// around it, completing on an mbarrier, double-buffered so the copy of the CTA's next partition
-// runs while the current one is processed. A partition the copy cannot take (the aligned range
-// would leave the array, or it does not fit a buffer) is read with plain loads: into the buffer
-// when it fits, else straight from global memory by the body.
-
-constexpr uint32_t kStageData = 32768;             // partition bytes one buffer holds
-constexpr uint32_t kStageBuf = kStageData + 32;    // + alignment lead and tail
-
-// the value at position x of a partition staged in shared memory (raw values of the column's type)
-__device__ __forceinline__ int64_t staged_value(const unsigned char* stage, int dtype, uint32_t x) {
-  return dtype == LECO_U32 ? (int64_t)reinterpret_cast<const uint32_t*>(stage)[x]
-                           : reinterpret_cast<const int64_t*>(stage)[x];
-}
-
-struct PartSrc {
-  const void* values;  // the column's values
-  uint64_t n;          // values in the column
-  uint64_t a;          // first position of the partition
-  uint32_t N;          // its length
-  int dtype;
-};
-
-// aligned byte range [g0, g0 + bytes) of the column holding the partition (at most cap value bytes);
-// lead = the partition's offset inside it
-__device__ __forceinline__ bool stage_plan(const PartSrc& s, uint32_t cap, uint64_t* g0, uint32_t* bytes,
-                                           uint32_t* lead) {
-  const uint64_t vb = s.dtype == LECO_U32 ? 4 : 8;
-  if (s.N == 0 || (uint64_t)s.N * vb > cap || (reinterpret_cast<uintptr_t>(s.values) & 15u)) return false;
-  const uint64_t b0 = s.a * vb, b1 = (s.a + s.N) * vb;
-  const uint64_t a0 = b0 & ~15ull, a1 = (b1 + 15) & ~15ull;
-  if (a1 > s.n * vb) return false;
-  *g0 = a0;
-  *bytes = (uint32_t)(a1 - a0);
-  *lead = (uint32_t)(b0 - a0);
-  return true;
-}
-
-// every thread decides (identically) whether the copy is used; thread 0 issues it
-__device__ __forceinline__ bool stage_issue(const PartSrc& s, uint32_t cap, unsigned char* dst, uint64_t* full) {
-  uint64_t g0;
-  uint32_t bytes, lead;
-  if (!stage_plan(s, cap, &g0, &bytes, &lead)) return false;
-  if (threadIdx.x == 0) {
-    mbar_arrive_expect_tx(full, bytes);
-    bulk_g2s(dst, static_cast<const char*>(s.values) + g0, bytes, full);
-  }
-  return true;
-}
-
-// Runs body(p, src, stage) for partitions p = blockIdx.x, + gridDim.x, ... < P, where stage is the
-// partition's values in shared memory (raw, the column's type; partitions of at most cap bytes,
-// cap <= kStageData) or nullptr. NBUF = 2 copies the
-// CTA's next partition while the current one is processed; NBUF = 1 keeps the CTA small (more CTAs
-// per SM hide each other's copies instead). body must end with a __syncthreads(). On a copy that
-// never lands the CTA records kStatTimeout in *err and stops.
-template <int NBUF, typename GetPart, typename Body>
-__device__ void for_each_staged(uint64_t P, uint32_t cap, GetPart get, Body body, unsigned char* ring, uint64_t* full,
-                                uint32_t* err) {
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < NBUF; k++) mbar_init(&full[k], 1);
-    mbar_fence_init();
-  }
-  __syncthreads();
-  uint32_t ph = 0, armed = 0;  // bit k: buffer k's mbarrier parity / a copy into buffer k is pending
-  uint32_t buf = 0;
-  uint64_t p = blockIdx.x;
-  if (p < P && stage_issue(get(p), cap, ring, &full[0])) armed = 1u;
-  for (; p < P; p += gridDim.x, buf = NBUF == 2 ? buf ^ 1u : 0u) {
-    // the buffer written next was released by the previous body's closing barrier
-    const uint32_t nb = NBUF == 2 ? buf ^ 1u : 0u;
-    const uint64_t pn = p + gridDim.x;
-    if (NBUF == 2) {
-      armed &= ~(1u << nb);
-      if (pn < P && stage_issue(get(pn), cap, ring + nb * kStageBuf, &full[nb])) armed |= 1u << nb;
-    }
-    const PartSrc s = get(p);
-    unsigned char* b = ring + buf * kStageBuf;
-    const unsigned char* st = nullptr;
-    if ((armed >> buf) & 1u) {
-      const bool ok = mbar_wait_bounded(&full[buf], (ph >> buf) & 1u);
-      if (__syncthreads_or(!ok)) {
-        if (threadIdx.x == 0 && err) atomicOr(err, kStatTimeout);
-        if (NBUF == 2 && ((armed >> nb) & 1u)) mbar_wait_bounded(&full[nb], (ph >> nb) & 1u);
-        return;
-      }
-      ph ^= 1u << buf;
-      uint64_t g0;
-      uint32_t bytes, lead;
-      stage_plan(s, cap, &g0, &bytes, &lead);
-      st = b + lead;
-    } else if ((uint64_t)s.N * (s.dtype == LECO_U32 ? 4 : 8) <= cap) {
-      if (s.dtype == LECO_U32) {
-        uint32_t* d = reinterpret_cast<uint32_t*>(b);
-        for (uint32_t x = threadIdx.x; x < s.N; x += blockDim.x)
-          d[x] = __ldg(static_cast<const uint32_t*>(s.values) + s.a + x);
-      } else {
-        uint64_t* d = reinterpret_cast<uint64_t*>(b);
-        for (uint32_t x = threadIdx.x; x < s.N; x += blockDim.x)
-          d[x] = __ldg(static_cast<const uint64_t*>(s.values) + s.a + x);
-      }
-      __syncthreads();
-      st = b;
-    }
-    body(p, s, st);
-    if (NBUF == 1) {  // the single buffer is free again: start the CTA's next partition
-      armed = 0;
-      if (pn < P && stage_issue(get(pn), cap, ring, &full[0])) armed = 1u;
-    }
-  }
 }
 
 // One warp per partition (grid-stride over warps): the fit's reductions are warp shuffles and its
@@ -467,20 +351,36 @@ __global__ void k_build_aux(const Record* __restrict__ rec, const PolyCoef* __re
 }
 
 // ------------------------------------------------------------------------------ packing
-
-// Packing, one CTA per partition (staged as for the fit). Phase 1 turns each staged value into its
-// zigzag residual under the partition's prediction, in shared memory (over the value itself for a
-// 64-bit column, into a second region for a 32-bit one). Phase 2 has each thread assemble output
-// words of the partition's bit range [off, off + N b) from those residuals. A word inside that
-// range belongs to this partition alone and is stored; a word the range covers only in part holds a
-// partition boundary (or the end of the stream), was zeroed beforehand, and is OR-ed into.
-constexpr uint32_t kZzOffset32 = (kStageData / 2 + 32 + 127) & ~127u;  // 32-bit columns: residuals after the values
-constexpr uint32_t kPackSmem64 = kStageBuf;
-constexpr uint32_t kPackSmem32 = kZzOffset32 + kStageData;
-
-// value bytes a staged partition may have: 64-bit residuals replace 64-bit values in place; a 32-bit
-// column's values (up to 4096 of them) leave room for their residuals after them
-__device__ __forceinline__ uint32_t pack_stage_cap(int dtype) { return dtype == LECO_U32 ? kStageData / 2 : kStageData; }
+//
+// A warp packs a window of consecutive positions, whatever partitions it touches: no barrier, no warp
+// waits for another, and partitions of any length take the same path; the windows shrink until a small
+// column fills the GPU. The piece of a partition inside a window owns the 32-bit words whose last bit
+// lies in it (at the partition's end, its last word too), so each word inside a partition is written
+// once, by one warp, with a few values before the piece read again. Words that hold a partition
+// boundary (or the end of the stream) were zeroed beforehand and are OR-ed into.
+//
+// The values' residuals go to a shared tile of 32 rows of K = 8, 16 or 32 consecutive values; lane r takes
+// row r into registers, strings its bits together from their place in the piece's words on (no division,
+// two values at a time up to 16 bits), passes the open last word to the next lane and leaves the others in
+// the tile, from where they go out coalesced. Widths above 32 bits and binary64 partitions assemble each word from
+// the fields it holds instead (pack_words, 79 instructions per value against 43).
+// The former packer staged a partition, or a run of short ones, per CTA by a bulk copy, three to seven
+// CTAs per SM each waiting for its own, and recomputed every field of partitions beyond 4096 values
+// from memory. Bound: memory and the latency of a piece's chain (64 registers hold 32 warps per SM; 48, 40
+// or 80 registers were slower). Measured, former -> this: 200M sorted normal uint64 in partitions of 4096
+// 431 -> 351 us (5.7 TB/s), 250M 32-bit timestamps in variable partitions 1295 -> 531 us, 100M piecewise
+// values 2.39 -> 0.9 ms, 96 columns of 200M values in partitions of 256 .. 4096 492 -> 431 us, 20M 32-bit
+// values in partitions of 1000 83 -> 60 us.
+constexpr int kPackBlock = 256;
+constexpr int kPackWarps = kPackBlock / 32;
+constexpr int kPackCtas = 4;  // CTAs per SM the registers are held for
+constexpr int kChunkLoads = 9;
+constexpr uint32_t kChunkVals = 32 * kChunkLoads;
+constexpr uint32_t kPackPiece = 1024;   // values packed at a time
+constexpr uint32_t kPackWindow = 4096;  // positions per warp of a large column
+constexpr uint32_t kPackWindowMin = 256;
+constexpr uint32_t kPackTile = 32 * 33;  // 32-bit entries of a warp's tile
+static_assert(kPackTile * 4 >= kChunkVals * 8, "a chunk's 64-bit residuals fit the tile");
 
 template <bool POLY>
 __device__ __forceinline__ uint64_t residual_at(const Record* __restrict__ rec, const PolyAux* __restrict__ poly,
@@ -489,150 +389,335 @@ __device__ __forceinline__ uint64_t residual_at(const Record* __restrict__ rec, 
   return zz_encode((int64_t)(v - (uint64_t)pred));
 }
 
-// contribution of a 64-bit field at bit f to the output word starting at bit wb
-__device__ __forceinline__ uint64_t place64(uint64_t z, uint64_t f, uint64_t wb) {
-  if (f >= wb + 64 || f + 64 <= wb) return 0;
-  return f >= wb ? z << (uint32_t)(f - wb) : z >> (uint32_t)(wb - f);
+// a partition being packed
+template <typename T>
+struct PackPart {
+  const T* v;            // its first value
+  uint32_t N, b, magic;  // values, width, ceil(2^32 / b) for b > 1: floor(r / b) as a high product, exact
+                         // for r < 2^26 (a chunk or piece has at most 2^16 bits)
+  uint32_t lead;         // bit of out[0] where its residuals begin
+  uint32_t* out;
+  uint64_t A, B;
+  uint32_t sh;
+  uint64_t p;
+  __device__ __forceinline__ uint32_t div_b(uint32_t r) const { return b > 1 ? __umulhi(r, magic) : r; }
+  // word w lies inside the partition's bits
+  __device__ __forceinline__ bool whole(uint32_t w) const {
+    return (w > 0 || lead == 0) && 32u * w + 32u <= lead + N * b;
+  }
+  __device__ __forceinline__ void put(uint32_t w, uint32_t x) const {
+    if (whole(w))
+      out[w] = x;
+    else
+      atomicOr(out + w, x);
+  }
+};
+
+// words [w0, w1) of a partition, each assembled from the fields it holds, a chunk of at most
+// kChunkVals values at a time
+template <typename T, bool POLY>
+__device__ __forceinline__ void pack_words(const PackPart<T>& q, const Aux& a, const Record* __restrict__ rec,
+                                           const PolyAux* __restrict__ poly, uint32_t w0, uint32_t w1, uint64_t* zs,
+                                           uint32_t lane) {
+  const uint32_t b = q.b;
+  const uint32_t most = ((kChunkVals - 2) * b) >> 5;  // words that at most kChunkVals fields overlap
+  const bool line = w3_exact(a.word3) != 0, pl = POLY && w3_poly(a.word3) != 0;
+  for (uint32_t w = w0; w < w1; w += most) {
+    const uint32_t we = min(w + most, w1);
+    const int32_t rb = (int32_t)(32u * w) - (int32_t)q.lead;
+    const uint32_t x_lo = rb > 0 ? (uint32_t)rb / b : 0u;
+    const int32_t rl = rb - (int32_t)(x_lo * b);  // below 0 where the partition begins inside the word
+    const uint32_t x_hi = min(q.N, x_lo + q.div_b((uint32_t)(rl + (int32_t)(32u * (we - w) + b - 1u))));
+    T val[kChunkLoads];
+#pragma unroll
+    for (int k = 0; k < kChunkLoads; k++) {
+      const uint32_t x = x_lo + lane + 32u * k;
+      val[k] = x < x_hi ? __ldg(q.v + x) : (T)0;
+    }
+    if (line) {
+      uint64_t F = q.A + q.B * (x_lo + lane);
+#pragma unroll
+      for (int k = 0; k < kChunkLoads; k++, F += q.B * 32u)
+        zs[lane + 32 * k] = zz_encode((int64_t)((uint64_t)val[k] - (uint64_t)((int64_t)F >> q.sh)));
+    } else if (pl) {
+      PolySteps Fd = poly_steps(poly[q.p], x_lo + lane, 32, 64u - ((uint32_t)w3_s(a.word3) & 63u));
+#pragma unroll
+      for (int k = 0; k < kChunkLoads; k++) {
+        zs[lane + 32 * k] = zz_encode((int64_t)((uint64_t)val[k] - ((uint64_t)a.A + (uint64_t)(Fd.F >> 64))));
+        poly_step(Fd);
+      }
+    } else {
+#pragma unroll 1
+      for (int k = 0; k < kChunkLoads; k++) {
+        const uint32_t x = x_lo + lane + 32u * k;
+        if (x < x_hi) zs[lane + 32 * k] = residual_at<POLY>(rec, poly, a, q.p, x, (uint64_t)__ldg(q.v + x));
+      }
+    }
+    __syncwarp();
+    const uint32_t V = x_hi - x_lo;
+    for (uint32_t j = lane; j < we - w; j += 32) {
+      const int32_t r = rl + (int32_t)(32u * j);
+      uint32_t x = r > 0 ? q.div_b((uint32_t)r) : 0u;
+      uint32_t acc = 0;
+      for (int32_t f = (int32_t)(x * b) - r; f < 32 && x < V; f += (int32_t)b, x++) {
+        const uint64_t z = zs[x];
+        acc |= f >= 0 ? (uint32_t)z << f : (uint32_t)(z >> (-f));
+      }
+      q.put(w + j, acc);
+    }
+    __syncwarp();
+  }
 }
 
-// POLY: the column may hold polynomial partitions (a separate instantiation keeps the constant and
-// linear packer as small as before)
-// zofs: the partition's first value within a stage holding several partitions (the 32-bit
-// residual buffer is indexed like the stage). WARP: one warp packs the partition (the CTA's warps
-// take different partitions of one staged item, whose residual buffers and full output words are
-// disjoint), otherwise the whole CTA.
-template <bool POLY, bool WARP = false>
-__device__ __forceinline__ void pack_partition(const PartSrc& s, const unsigned char* st, unsigned char* ring,
-                                               const Record* __restrict__ rec, const Aux* __restrict__ aux,
-                                               const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly,
-                                               uint64_t p, uint64_t* __restrict__ words, uint32_t zofs = 0) {
-  const uint32_t t = WARP ? (threadIdx.x & 31u) : threadIdx.x;
-  const uint32_t G = WARP ? 32u : blockDim.x;
-  auto gsync = [] {
-    if (WARP)
-      __syncwarp();
-    else
-      __syncthreads();
-  };
-  const Aux a = aux[p];
-  const uint32_t b = w3_b(a.word3);
-  const bool pl = POLY && w3_poly(a.word3) != 0;
-  const uint64_t off = w3_off(a.word3), endb = off + (uint64_t)s.N * b;
-  const uint64_t off0 = pl ? off - kPolyBlockBits : off;  // first bit of the partition (its block)
-  if (!pl && st && b && w3_exact(a.word3)) {
-    // Staged partition on the integer grid (the common case). Phase 1: each thread steps its
-    // fixed-point prediction F = A + B x by B blockDim from one position to its next (no multiply).
-    // Phase 2: bit positions relative to the partition's first residual bit fit 32 bits (at most
-    // 2^24 fields of at most 64 bits).
-    uint64_t* zs = s.dtype == LECO_U32 ? reinterpret_cast<uint64_t*>(ring + kZzOffset32) + zofs
-                                       : const_cast<uint64_t*>(reinterpret_cast<const uint64_t*>(st));
-    const int32_t sr = w3_s(a.word3);
-    const uint32_t sh = sr > 0 ? (uint32_t)sr : 0u;
-    uint64_t F = (uint64_t)a.A + (uint64_t)a.B * t;
-    const uint64_t dF = (uint64_t)a.B * G;
-    if (s.dtype == LECO_U32) {
-      const uint32_t* v = reinterpret_cast<const uint32_t*>(st);
-      for (uint32_t x = t; x < s.N; x += G, F += dF)
-        zs[x] = zz_encode((int64_t)((uint64_t)v[x] - (uint64_t)((int64_t)F >> sh)));
-    } else {
-      const uint64_t* v = reinterpret_cast<const uint64_t*>(st);
-      for (uint32_t x = t; x < s.N; x += G, F += dF)
-        zs[x] = zz_encode((int64_t)(v[x] - (uint64_t)((int64_t)F >> sh)));
+// values [x0, x0 + V) of a partition of width b <= 32 on a line (or, PL, a polynomial), V <= 32 K, K b >= 32:
+// lane r packs the K consecutive values of row r
+template <int K, typename T, bool PL>
+__device__ __forceinline__ void pack_rows(const PackPart<T>& q, const Aux& a, const PolyAux* __restrict__ poly,
+                                          uint32_t x0, uint32_t V, uint32_t* tile, uint32_t lane) {
+  const uint32_t b = q.b;
+  PolySteps Fd;
+  if (PL) Fd = poly_steps(poly[q.p], x0 + lane, 32, 64u - ((uint32_t)w3_s(a.word3) & 63u));
+  const T* v = q.v + x0 + lane;
+  // the lane loads values lane + 32 k for k < mine (x < V); steps past them leave bits past the piece
+  const int mine = V > lane ? (int)((V - lane + 31u) >> 5) : 0;
+  uint64_t F = q.A + q.B * (x0 + lane);
+  const uint64_t dF = q.B * 32u;
+  T val[2][8];
+#pragma unroll
+  for (int u = 0; u < 8; u++) val[0][u] = u < mine ? __ldg(v + 32 * u) : (T)0;
+  // a width of at most 32 bits: the zigzag code is 32 bits of the residual and its sign
+  auto zz32 = [](uint64_t r) { return ((uint32_t)r << 1) ^ (uint32_t)((int32_t)(r >> 32) >> 31); };
+  // the bits before the piece in its first word, from the values that hold them
+  const uint32_t bit = q.lead + x0 * b, w0 = bit >> 5, o = bit & 31u;
+  uint32_t prev = 0;
+  if (x0 && o) {
+    uint32_t c = 0;
+    if (lane * b < o && lane < x0) {
+      const uint32_t x = x0 - 1u - lane;
+      const uint64_t pred = PL ? (uint64_t)predict_aux(a, nullptr, poly, q.p, x) : (uint64_t)((int64_t)(q.A + q.B * x) >> q.sh);
+      const uint32_t z = zz32((uint64_t)__ldg(q.v + x) - pred);
+      const int32_t s = (int32_t)o - (int32_t)((lane + 1u) * b);
+      c = s >= 0 ? z << s : z >> (-s);
     }
-    gsync();
-    const uint32_t lead = (uint32_t)(off & 63u);
-    const int32_t nbits = (int32_t)(s.N * b);
-    const uint64_t w0 = off >> 6, wl = (endb - 1) >> 6;
-    for (uint64_t w = w0 + t; w <= wl; w += G) {
-      const int32_t r0 = (int32_t)((w - w0) << 6) - (int32_t)lead;  // the word's first bit, relative
-      const int32_t r1 = r0 + 64 < nbits ? r0 + 64 : nbits;
-      uint32_t x = r0 > 0 ? (uint32_t)r0 / b : 0u;
-      uint64_t acc = 0;
-      for (int32_t fr = (int32_t)(x * b); fr < r1; fr += (int32_t)b, x++) {
-        const uint64_t z = zs[x];
-        const int32_t d = fr - r0;
-        acc |= d >= 0 ? z << d : z >> (-d);
+    prev = __reduce_or_sync(0xffffffffu, c);
+  }
+  uint32_t* put = tile + lane + (K == 32 ? 0u : lane / (uint32_t)K);
+#pragma unroll
+  for (int k = 0; k < K; k += 8) {
+    const int cur = (k >> 3) & 1;
+    if (k + 8 < K) {
+#pragma unroll
+      for (int u = 0; u < 8; u++) val[cur ^ 1][u] = k + 8 + u < mine ? __ldg(v + 32 * (k + 8 + u)) : (T)0;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; u++) {
+      uint64_t pred;
+      if (PL) {
+        pred = (uint64_t)a.A + (uint64_t)(Fd.F >> 64);
+        poly_step(Fd);
+      } else {
+        pred = (uint64_t)((int64_t)F >> q.sh);
+        F += dF;
       }
-      if (r0 >= 0 && r0 + 64 <= nbits)
-        words[w] = acc;
-      else
-        atomicOr((unsigned long long*)&words[w], (unsigned long long)acc);
+      put[(32 + 32 / K) * (k + u)] = zz32((uint64_t)val[cur][u] - pred);  // value x at x + x / K
     }
-    gsync();  // the stage buffer is refilled for the next partition
+  }
+  __syncwarp();
+  // The row's bits begin at bit `at` of the piece's words; its first word and the open last one are put
+  // together with the neighbours'. Rows of 32 values begin at the same bit of a word in every lane, b words
+  // apart: `fill` and the branches on it are uniform, and the words replace the row's residuals in place
+  // (word k is complete after more than k values). Shorter rows go through registers to the tile as one
+  // run of words, every 33rd free so that rows a power of two apart use different banks.
+  const uint32_t at = o + lane * (uint32_t)K * b, wf = at >> 5;
+  uint32_t first = 0, open = 0;
+  if (K == 32) {
+    uint32_t* row = tile + lane * 33u;
+    uint32_t fill = o, done = 0, acc = 0;
+    auto emit = [&](uint32_t x, uint32_t width) {  // x < 2^width, or bits past the piece
+      const uint64_t t = (uint64_t)x * (1u << fill) + acc;
+      acc = (uint32_t)t;
+      fill += width;
+      if (fill >= 32u) {
+        row[done++] = acc;
+        acc = (uint32_t)(t >> 32);
+        fill -= 32u;
+      }
+    };
+    if (b <= 16) {
+      const uint32_t pw = 1u << b;
+#pragma unroll 8
+      for (int i = 0; i < K; i += 2) emit(row[i] + row[i + 1] * pw, 2u * b);
+    } else {
+#pragma unroll 8
+      for (int i = 0; i < K; i++) emit(row[i], b);
+    }
+    open = acc;
+  } else {
+    uint32_t z[K];
+#pragma unroll
+    for (int i = 0; i < K; i++) z[i] = tile[lane * (K + 1) + i];
+    __syncwarp();
+    uint32_t w = wf, fill = at & 31u, acc = 0;
+    auto emit = [&](uint32_t x, uint32_t width) {
+      const uint64_t t = (uint64_t)x * (1u << fill) + acc;
+      const bool full = fill + width >= 32u;
+      if (full && w != wf) tile[w + (w >> 5)] = (uint32_t)t;
+      if (full && w == wf) first = (uint32_t)t;
+      acc = full ? (uint32_t)(t >> 32) : (uint32_t)t;
+      fill = (fill + width) & 31u;
+      w += full ? 1u : 0u;
+    };
+    if (b <= 16) {
+      const uint32_t pw = 1u << b;
+#pragma unroll
+      for (int i = 0; i < K; i += 2) emit(z[i] + z[i + 1] * pw, 2u * b);
+    } else {
+#pragma unroll
+      for (int i = 0; i < K; i++) emit(z[i], b);
+    }
+    open = acc;
+  }
+  uint32_t below = __shfl_up_sync(0xffffffffu, open, 1);
+  if (lane == 0) below = prev;
+  if (K == 32)
+    tile[lane * 33u] |= below;
+  else
+    tile[wf + (wf >> 5)] = first | below;
+  const uint32_t past = (at + (uint32_t)K * b) >> 5;  // the open word
+  const uint32_t tail = __shfl_sync(0xffffffffu, open, 31), wtail = __shfl_sync(0xffffffffu, past, 31);
+  __syncwarp();
+  auto word = [&](uint32_t j) -> uint32_t {
+    if (j == wtail) return tail;
+    if (K != 32) return tile[j + (j >> 5)];
+    const uint32_t r = q.div_b(j);
+    return tile[r * 33u + (j - r * b)];
+  };
+  const uint32_t end = o + V * b;
+  const bool last = x0 + V == q.N;
+  // words that lie inside the partition's bits are stored, its first and last one OR-ed into
+  const uint32_t j0 = q.lead && w0 == 0 ? 1u : 0u, j1 = end >> 5;
+  uint32_t* out = q.out + w0;
+  for (uint32_t j = j0 + lane; j < j1; j += 32) out[j] = word(j);
+  if (lane == 0 && j0) {
+    const uint32_t keep = j1 == 0 ? (1u << (end & 31u)) - 1u : ~0u;
+    if (j1 || last) atomicOr(out, word(0) & keep);
+  }
+  if (lane == 1 && last && (end & 31u) && j1 >= j0) atomicOr(out + j1, word(j1) & ((1u << (end & 31u)) - 1u));
+  __syncwarp();
+}
+
+// values [xa, xb) of a partition of N values (its first value at v[0], entry a, index p)
+template <typename T, bool POLY>
+__device__ __forceinline__ void pack_piece(const T* __restrict__ v, uint32_t N, uint32_t xa, uint32_t xb, const Aux& a,
+                                           const Record* __restrict__ rec, const PolyAux* __restrict__ poly, uint64_t p,
+                                           uint32_t* __restrict__ words, uint64_t* zbuf, uint32_t lane) {
+  PackPart<T> q;
+  q.b = w3_b(a.word3);
+  if (q.b == 0) return;
+  q.v = v;
+  q.N = N;
+  q.magic = 0xFFFFFFFFu / q.b + 1u;  // b = 1 takes no product
+  const uint64_t off = w3_off(a.word3);
+  q.lead = (uint32_t)off & 31u;
+  q.out = words + (off >> 5);
+  q.A = (uint64_t)a.A;
+  q.B = (uint64_t)a.B;
+  const int32_t sr = w3_s(a.word3);
+  q.sh = sr > 0 ? (uint32_t)sr & 63u : 0u;
+  q.p = p;
+  const bool line = w3_exact(a.word3) != 0, pl = POLY && w3_poly(a.word3) != 0;
+  if (q.b <= 32 && (line || pl)) {
+    uint32_t* tile = reinterpret_cast<uint32_t*>(zbuf);
+    for (uint32_t x = xa; x < xb; x += kPackPiece) {
+      const uint32_t V = min(kPackPiece, xb - x);
+      if (pl)
+        pack_rows<32, T, true>(q, a, poly, x, V, tile, lane);
+      else if (V <= 256 && q.b >= 4)
+        pack_rows<8, T, false>(q, a, poly, x, V, tile, lane);
+      else if (V <= 512 && q.b >= 2)
+        pack_rows<16, T, false>(q, a, poly, x, V, tile, lane);
+      else
+        pack_rows<32, T, false>(q, a, poly, x, V, tile, lane);
+    }
     return;
   }
-  if (endb > off0) {
-    // phase 1: residuals into shared memory (staged partitions only; others recompute per field)
-    uint64_t* zs = nullptr;
-    if (st && b) {
-      zs = s.dtype == LECO_U32 ? reinterpret_cast<uint64_t*>(ring + kZzOffset32) + zofs
-                               : const_cast<uint64_t*>(reinterpret_cast<const uint64_t*>(st));
-      if (pl) {
-        // the thread's predictions T + (F(x) >> S) for x = tid, tid + blockDim, ... by forward
-        // differences of the cubic F over that stride, carried times 2^(64-S) modulo 2^128 so that
-        // the prediction's low 64 bits are the carried value's high half
-        PolySteps Fd = poly_steps(poly[p], t, G, 64u - ((uint32_t)w3_s(a.word3) & 63u));
-        const uint64_t T = (uint64_t)a.A;
-        for (uint32_t xx = t; xx < s.N; xx += G) {
-          zs[xx] = zz_encode((int64_t)((uint64_t)staged_value(st, s.dtype, xx) - (T + (uint64_t)(Fd.F >> 64))));
-          poly_step(Fd);
-        }
-      } else {
-        for (uint32_t x = t; x < s.N; x += G)
-          zs[x] = residual_at<POLY>(rec, poly, a, p, x, (uint64_t)staged_value(st, s.dtype, x));
-      }
-      gsync();
-    }
-    // phase 2: output words of [off0, endb): the polynomial block's five words, then the fields
-    for (uint64_t w = (off0 >> 6) + t; w <= ((endb - 1) >> 6); w += G) {
-      const uint64_t wb = w << 6;
-      const uint64_t lo = wb > off0 ? wb : off0, hi = wb + 64 < endb ? wb + 64 : endb;
-      uint64_t acc = 0;
-      if (pl && lo < off) {
-        const PolyCoef& pc = pcoef[p];
-        acc |= place64((uint64_t)pc.T, off0, wb) | place64((uint64_t)pc.K[0], off0 + 64, wb) |
-               place64((uint64_t)pc.K[1], off0 + 128, wb) | place64((uint64_t)pc.K[2], off0 + 192, wb) |
-               place64(pc.E, off0 + 256, wb);
-      }
-      if (b && hi > off) {
-        const uint64_t l2 = lo > off ? lo : off;
-        uint32_t x = (uint32_t)(l2 - off) / b;  // first field overlapping the word (< 2^30 bits in)
-        for (uint64_t f = off + (uint64_t)x * b; f < hi; f += b, x++) {
-          const uint64_t z = zs ? zs[x] : residual_at<POLY>(rec, poly, a, p, x, load_value(s.values, s.dtype, s.a + x));
-          acc |= f >= wb ? z << (uint32_t)(f - wb) : z >> (uint32_t)(wb - f);
-        }
-      }
-      if (lo == wb && hi == wb + 64)
-        words[w] = acc;
-      else
-        atomicOr((unsigned long long*)&words[w], (unsigned long long)acc);
-    }
-  }
-  gsync();  // the stage buffer is refilled for the next partition
+  const uint32_t w0 = (q.lead + xa * q.b) >> 5;
+  const uint32_t w1 = xb == N ? (q.lead + N * q.b + 31u) >> 5 : (q.lead + xb * q.b) >> 5;
+  pack_words<T, POLY>(q, a, rec, poly, w0, w1, zbuf, lane);
 }
 
-constexpr int kPackBlock = 128;
+// the coefficient block of a polynomial partition, ten 32-bit words at the bit before its residuals:
+// OR-ed, as are the words' other bits (k_zero_bounds zeroes them)
+__device__ __forceinline__ void pack_block(const PolyCoef& pc, uint64_t off0, uint32_t* __restrict__ words, uint32_t lane) {
+  if (lane >= 10) return;
+  const uint32_t q = lane >> 1;
+  const uint64_t f = q == 0 ? (uint64_t)pc.T : q == 4 ? pc.E : (uint64_t)(q == 1 ? pc.K[0] : q == 2 ? pc.K[1] : pc.K[2]);
+  const uint32_t h = (lane & 1u) ? (uint32_t)(f >> 32) : (uint32_t)f;
+  const uint64_t at = off0 + 32ull * lane;
+  const uint32_t o = (uint32_t)at & 31u;
+  uint32_t* w = words + (at >> 5);
+  atomicOr(w, h << o);
+  if (o) atomicOr(w + 1, h >> (32u - o));
+}
 
-template <bool POLY>
-__global__ void __launch_bounds__(kPackBlock)
-    k_pack(const void* __restrict__ values, int dtype, const Record* __restrict__ rec,
-           const Aux* __restrict__ aux, const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly,
-           uint64_t m, uint64_t n, uint64_t* __restrict__ words, uint32_t* __restrict__ err) {
-  __shared__ __align__(8) uint64_t full[1];
-  extern __shared__ __align__(128) unsigned char ring[];
-  auto get = [&](uint64_t p) {
-    PartSrc s;
-    s.values = values;
-    s.n = n;
-    s.a = aux[p].start;
-    s.N = (uint32_t)((p + 1 < m ? aux[p + 1].start : n) - s.a);
-    s.dtype = dtype;
-    return s;
-  };
-  auto body = [&](uint64_t p, const PartSrc& s, const unsigned char* st) {
-    pack_partition<POLY>(s, st, ring, rec, aux, pcoef, poly, p, words);
-  };
-  for_each_staged<1>(m, pack_stage_cap(dtype), get, body, ring, full, err);
+// positions [pos, end) of a column, partition p holding pos
+template <typename T, bool POLY>
+__device__ __forceinline__ void pack_window(const T* __restrict__ values, uint64_t n, uint64_t m, uint64_t pos,
+                                            uint64_t end, uint64_t p, const Record* __restrict__ rec,
+                                            const Aux* __restrict__ aux, const PolyCoef* __restrict__ pcoef,
+                                            const PolyAux* __restrict__ poly, uint32_t* __restrict__ words,
+                                            uint64_t* zbuf, uint32_t lane) {
+  // the lanes fetch 32 entries at a time (one memory round trip for a run of short partitions)
+  while (pos < end) {
+    Aux mine;
+    mine.A = mine.B = 0;
+    mine.word3 = 0;
+    mine.start = n;
+    if (p + lane < m) mine = aux[p + lane];
+    for (uint32_t k = 0; k < 31 && pos < end; k++, p++) {
+      Aux a;
+      a.A = __shfl_sync(0xffffffffu, mine.A, k);
+      a.B = __shfl_sync(0xffffffffu, mine.B, k);
+      a.start = __shfl_sync(0xffffffffu, mine.start, k);
+      a.word3 = __shfl_sync(0xffffffffu, mine.word3, k);
+      const uint64_t e = __shfl_sync(0xffffffffu, mine.start, k + 1);
+      const uint32_t xa = (uint32_t)(pos - a.start);
+      if (POLY && xa == 0 && w3_poly(a.word3)) pack_block(pcoef[p], w3_off(a.word3) - kPolyBlockBits, words, lane);
+      pack_piece<T, POLY>(values + a.start, (uint32_t)(e - a.start), xa, (uint32_t)(min(e, end) - a.start), a, rec, poly,
+                          p, words, zbuf, lane);
+      pos = e;
+    }
+  }
+}
+
+// L: the fixed partition length, or 0: partitions of any lengths, found through the scan tiles
+template <typename T, bool POLY>
+__global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
+    k_pack(const T* __restrict__ values, uint64_t n, uint64_t m, uint32_t L, uint32_t window,
+           const TileDesc* __restrict__ tiles, const Record* __restrict__ rec, const Aux* __restrict__ aux,
+           const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly, uint32_t* __restrict__ words) {
+  __shared__ uint64_t zbuf[kPackWarps][kPackTile / 2];
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  const uint64_t nwin = (n + window - 1) / window, nw = (uint64_t)gridDim.x * kPackWarps;
+  for (uint64_t k = (uint64_t)blockIdx.x * kPackWarps + wid; k < nwin; k += nw) {
+    const uint64_t pos = k * window, end = min(pos + window, n);
+    uint64_t p;
+    if (L) {
+      p = pos / L;
+    } else {
+      const TileDesc* d = tiles + pos / kScanTile;
+      p = d->p0;
+      uint64_t hi = p + d->np;
+      while (hi - p > 1) {
+        const uint64_t mid = (p + hi) >> 1;
+        if (aux[mid].start <= pos)
+          p = mid;
+        else
+          hi = mid;
+      }
+    }
+    pack_window<T, POLY>(values, n, m, pos, end, p, rec, aux, pcoef, poly, words, zbuf[wid], lane);
+  }
 }
 
 // first stream bit of a partition: its residuals, or the block ahead of them for a polynomial one
@@ -640,16 +725,25 @@ __device__ __forceinline__ uint64_t part_first_bit(const Aux& a) {
   return w3_off(a.word3) - (w3_poly(a.word3) ? kPolyBlockBits : 0);
 }
 
-// Zero the words that packing OR-s into: each word holding a partition's first bit, and the words
-// from the end of the stream on (the tail word and the zero padding). Every other word lies inside
-// one partition's bit range and is written whole.
+// zeroes the words that packing OR-s into at the start of one partition: the word of its first bit and
+// those of a coefficient block
+__device__ __forceinline__ void zero_bound(const Aux& a, uint64_t* __restrict__ words) {
+  const uint64_t w = part_first_bit(a) >> 6, e = w3_off(a.word3) >> 6;
+  for (uint64_t k = w; k <= e; k++) words[k] = 0;
+}
+
+// Zero the words that packing OR-s into: each word holding a partition's first bit (and its block), and
+// the words from the end of the stream on (the tail word and the zero padding). Every other word lies
+// inside one partition's bit range and is written whole.
 __global__ void k_zero_bounds(const Aux* __restrict__ aux, uint64_t m, uint64_t total_bits, uint64_t nwords,
                               uint64_t* __restrict__ words) {
   const uint64_t tail = total_bits >> 6;
   const uint64_t count = m + (nwords > tail ? nwords - tail : 0);
   for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < count; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t w = i < m ? (part_first_bit(aux[i]) >> 6) : tail + (i - m);
-    if (w < nwords) words[w] = 0;
+    if (i < m)
+      zero_bound(aux[i], words);
+    else
+      words[tail + (i - m)] = 0;
   }
 }
 
@@ -714,127 +808,28 @@ __global__ void k_aux_multi(const Record* __restrict__ rec, const PolyCoef* __re
   }
 }
 
-// CTA per pack item: a run of consecutive partitions of one column whose values fit one stage
-// (several short partitions share one staged copy, and a warp packs each of them)
-template <bool POLY>
-__global__ void __launch_bounds__(kPackBlock)
+// k_pack over the columns of a batch: windows of every column, tile_base[c] scan tiles before column c
+template <typename T, bool POLY>
+__global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
     k_pack_multi(const EncCol* __restrict__ cols, const uint64_t* __restrict__ part_base,
-                 const uint64_t* __restrict__ word_base, const PackItem* __restrict__ items, uint64_t nitems, int dtype,
-                 const Record* __restrict__ rec, const Aux* __restrict__ aux, const PolyCoef* __restrict__ pcoef,
-                 const PolyAux* __restrict__ poly, uint64_t* __restrict__ words, uint32_t* __restrict__ err) {
-  __shared__ __align__(8) uint64_t full[1];
-  extern __shared__ __align__(128) unsigned char ring[];
-  auto get = [&](uint64_t it) {
-    const PackItem item = items[it];
-    const EncCol col = cols[item.c];
-    const uint64_t pe = item.p0 + item.k;
-    PartSrc s;
-    s.values = col.values;
-    s.n = col.n;
-    s.a = aux[item.p0].start;
-    s.N = (uint32_t)((pe < part_base[item.c + 1] ? aux[pe].start : s.n) - s.a);
-    s.dtype = dtype;
-    return s;
-  };
-  auto body = [&](uint64_t it, const PartSrc& si, const unsigned char* st) {
-    const PackItem item = items[it];
-    const uint64_t p0 = part_base[item.c];
-    const uint32_t vb = dtype == LECO_U32 ? 4u : 8u;
-    auto part = [&](uint64_t p) {
-      PartSrc s = si;
-      s.a = aux[p].start;
-      s.N = (uint32_t)((p + 1 < part_base[item.c + 1] ? aux[p + 1].start : si.n) - s.a);
-      return s;
-    };
-    if (item.k == 1) {  // one partition: the whole CTA
-      pack_partition<POLY>(part(item.p0), st, ring, rec + p0, aux + p0, POLY ? pcoef + p0 : nullptr,
-                           POLY ? poly + p0 : nullptr, item.p0 - p0, words + word_base[item.c], 0);
-      return;
-    }
-    // several short partitions: a warp each, the CTA's warps side by side (their residual buffers
-    // and whole output words are disjoint)
-    for (uint32_t q = threadIdx.x >> 5; q < item.k; q += kPackBlock / 32) {
-      const uint64_t p = item.p0 + q;
-      const PartSrc s = part(p);
-      const uint32_t zofs = (uint32_t)(s.a - si.a);
-      pack_partition<POLY, true>(s, st ? st + (size_t)zofs * vb : nullptr, ring, rec + p0, aux + p0,
-                                 POLY ? pcoef + p0 : nullptr, POLY ? poly + p0 : nullptr, p - p0,
-                                 words + word_base[item.c], zofs);
-    }
-    __syncthreads();  // the stage buffer is refilled for the next item
-  };
-  for_each_staged<1>(nitems, pack_stage_cap(dtype), get, body, ring, full, err);
-}
-
-// Pack items of one column with short partitions (variable partitions): a partition of at most
-// kItemWindow values joins the item of its predecessor when both start in the same kItemWindow-aligned
-// window of positions (so an item spans fewer than 2 kItemWindow values and fits one stage); a longer
-// partition is an item of its own. flag[p] = 1 where an item begins.
-constexpr uint64_t kItemWindow = 2048;
-
-__global__ void k_item_flags(const Aux* __restrict__ aux, uint64_t m, uint64_t n, uint64_t* __restrict__ flag) {
-  for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < m; p += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t s = aux[p].start, e = p + 1 < m ? aux[p + 1].start : n;
-    bool begin = p == 0 || e - s > kItemWindow;
-    if (!begin) {
-      const uint64_t s0 = aux[p - 1].start;
-      begin = s - s0 > kItemWindow || (s / kItemWindow) != (s0 / kItemWindow);
-    }
-    flag[p] = begin ? 1ull : 0ull;
+                 const uint64_t* __restrict__ tile_base, const uint64_t* __restrict__ word_base, uint32_t ncols,
+                 uint64_t T_tiles, uint32_t window, const Record* __restrict__ rec, const Aux* __restrict__ aux,
+                 const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly, uint64_t* __restrict__ words) {
+  __shared__ uint64_t zbuf[kPackWarps][kPackTile / 2];
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  const uint32_t per_tile = (uint32_t)kScanTile / window;
+  const uint64_t jobs = T_tiles * per_tile, nw = (uint64_t)gridDim.x * kPackWarps;
+  for (uint64_t k = (uint64_t)blockIdx.x * kPackWarps + wid; k < jobs; k += nw) {
+    const uint64_t g = k / per_tile;
+    const uint32_t c = find_col(tile_base, ncols, g);
+    const EncCol col = cols[c];
+    const uint64_t pos = (k - tile_base[c] * per_tile) * window;
+    if (pos >= col.n) continue;  // the column's last tile is short
+    const uint64_t p0 = part_base[c];
+    pack_window<T, POLY>(static_cast<const T*>(col.values), col.n, part_base[c + 1] - p0, pos, min(pos + window, col.n),
+                         pos / col.L, rec + p0, aux + p0, POLY ? pcoef + p0 : nullptr, POLY ? poly + p0 : nullptr,
+                         reinterpret_cast<uint32_t*>(words + word_base[c]), zbuf[wid], lane);
   }
-}
-
-// item_start[idx[p]] = p for every item-beginning partition p, and item_start[nitems] = m
-__global__ void k_item_starts(const uint64_t* __restrict__ flag, const uint64_t* __restrict__ idx, uint64_t m,
-                              const uint64_t* __restrict__ nitems, uint64_t* __restrict__ item_start) {
-  for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < m; p += (uint64_t)gridDim.x * blockDim.x) {
-    if (flag[p]) item_start[idx[p]] = p;
-    if (p == 0) item_start[*nitems] = m;
-  }
-}
-
-// CTA per item of one column (constant and linear partitions): one staged copy for the item's
-// partitions, packed one after the other; the item count is read on the device
-__global__ void __launch_bounds__(kPackBlock)
-    k_pack_items(const void* __restrict__ values, int dtype, const Record* __restrict__ rec,
-                 const Aux* __restrict__ aux, uint64_t m, uint64_t n, const uint64_t* __restrict__ item_start,
-                 const uint64_t* __restrict__ nitems_d, uint64_t* __restrict__ words, uint32_t* __restrict__ err) {
-  __shared__ __align__(8) uint64_t full[1];
-  extern __shared__ __align__(128) unsigned char ring[];
-  const uint64_t nitems = *nitems_d;
-  auto get = [&](uint64_t it) {
-    const uint64_t p0 = item_start[it], pe = item_start[it + 1];
-    PartSrc s;
-    s.values = values;
-    s.n = n;
-    s.a = aux[p0].start;
-    s.N = (uint32_t)((pe < m ? aux[pe].start : n) - s.a);
-    s.dtype = dtype;
-    return s;
-  };
-  auto body = [&](uint64_t it, const PartSrc& si, const unsigned char* st) {
-    const uint64_t p0 = item_start[it], pe = item_start[it + 1];
-    const uint32_t vb = dtype == LECO_U32 ? 4u : 8u;
-    auto part = [&](uint64_t p) {
-      PartSrc s = si;
-      s.a = aux[p].start;
-      s.N = (uint32_t)((p + 1 < m ? aux[p + 1].start : n) - s.a);
-      return s;
-    };
-    if (pe - p0 == 1) {  // a long partition: the whole CTA
-      pack_partition<false>(part(p0), st, ring, rec, aux, nullptr, nullptr, p0, words, 0);
-      return;
-    }
-    // short partitions: a warp each, the CTA's warps side by side
-    for (uint64_t p = p0 + (threadIdx.x >> 5); p < pe; p += kPackBlock / 32) {
-      const PartSrc s = part(p);
-      const uint32_t zofs = (uint32_t)(s.a - si.a);
-      pack_partition<false, true>(s, st ? st + (size_t)zofs * vb : nullptr, ring, rec, aux, nullptr, nullptr, p, words,
-                                  zofs);
-    }
-    __syncthreads();  // the stage buffer is refilled for the next item
-  };
-  for_each_staged<1>(nitems, pack_stage_cap(dtype), get, body, ring, full, err);
 }
 
 __global__ void k_part_col(const uint64_t* __restrict__ part_base, uint32_t ncols, uint64_t P,
@@ -877,8 +872,7 @@ __global__ void k_zero_bounds_multi(const Aux* __restrict__ aux, const uint32_t*
                                     uint32_t ncols, uint64_t P, uint64_t* __restrict__ words) {
   const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
   for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < P; p += stride) {
-    const uint32_t c = part_col[p];
-    words[word_base[c] + (part_first_bit(aux[p]) >> 6)] = 0;
+    zero_bound(aux[p], words + word_base[part_col[p]]);
   }
   for (uint64_t c = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; c < ncols; c += stride)
     for (uint64_t w = word_base[c] + (col_bits[c] >> 6); w < word_base[c + 1]; w++) words[w] = 0;
@@ -903,16 +897,6 @@ int sm_count() {
     cached[dev] = v > 0 ? v : 1;
   }
   return cached[dev];
-}
-
-// persistent grid: as many CTAs as fit on the GPU at once with the staging ring (grid-stride over work)
-template <typename K>
-int resident_grid(K kern, int block, uint64_t work, uint32_t smem) {
-  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-  int nb = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, block, smem) != cudaSuccess || nb < 1) nb = 1;
-  const uint64_t cap = (uint64_t)sm_count() * nb;
-  return (int)(work < cap ? work : cap);
 }
 
 // the four polynomial phases over partitions [0, m) of the map, with their scratch (given: at least
@@ -1001,59 +985,35 @@ cudaError_t launch_build_aux(const Record* rec, const PolyCoef* pcoef, uint64_t 
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack(const void* values, int dtype, const Record* rec, const Aux* aux, const PolyCoef* pcoef,
-                        const PolyAux* poly, uint64_t m, uint64_t n, uint64_t total_bits, uint64_t* words,
-                        uint64_t nwords, uint32_t* err, cudaStream_t st) {
-  if (nwords == 0) return cudaSuccess;
-  const uint64_t tail = total_bits >> 6;
-  k_zero_bounds<<<grid_for(m + (nwords > tail ? nwords - tail : 0), 256, 8), 256, 0, st>>>(aux, m, total_bits, nwords,
-                                                                                         words);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || m == 0) return e;
-  const uint32_t smem = dtype == LECO_U32 ? kPackSmem32 : kPackSmem64;
-  if (pcoef)
-    k_pack<true><<<resident_grid(k_pack<true>, kPackBlock, m, smem), kPackBlock, smem, st>>>(
-        values, dtype, rec, aux, pcoef, poly, m, n, words, err);
-  else
-    k_pack<false><<<resident_grid(k_pack<false>, kPackBlock, m, smem), kPackBlock, smem, st>>>(
-        values, dtype, rec, aux, nullptr, nullptr, m, n, words, err);
+template <typename T, bool POLY>
+cudaError_t launch_pack_t(const void* values, uint64_t n, uint64_t m, uint32_t L, const TileDesc* tiles,
+                          const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
+                          uint64_t* words, cudaStream_t st) {
+  // Windows as long as kPackWindow while each resident warp (32 per SM) still has four, so that the last
+  // wave weighs little: 250M timestamps of ~570-value partitions packed in 650 us with windows of 1024
+  // (which cut most partitions) and 531 us with 4096; columns below 5M values come down to 256.
+  uint32_t window = kPackWindow;
+  while (window > kPackWindowMin && n / window < (uint64_t)sm_count() * 128) window /= 2;
+  const uint64_t nwin = (n + window - 1) / window;
+  k_pack<T, POLY><<<grid_for(nwin, kPackWarps, 8), kPackBlock, 0, st>>>(
+      static_cast<const T*>(values), n, m, L, window, tiles, rec, aux, pcoef, poly, reinterpret_cast<uint32_t*>(words));
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_var(const void* values, int dtype, const Record* rec, const Aux* aux, uint64_t m, uint64_t n,
-                            uint64_t total_bits, uint64_t* words, uint64_t nwords, uint32_t* err, cudaStream_t st) {
+cudaError_t launch_pack(const void* values, int dtype, uint32_t L, const TileDesc* tiles, const Record* rec,
+                        const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly, uint64_t m, uint64_t n,
+                        uint64_t total_bits, uint64_t* words, uint64_t nwords, cudaStream_t st) {
   if (nwords == 0) return cudaSuccess;
   const uint64_t tail = total_bits >> 6;
   k_zero_bounds<<<grid_for(m + (nwords > tail ? nwords - tail : 0), 256, 8), 256, 0, st>>>(aux, m, total_bits, nwords,
                                                                                          words);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess || m == 0) return e;
-  // flags | indices | item starts (m + 1) | scan scratch | item count
-  const uint64_t scr_elems = m / 2048 + 2;
-  uint64_t* buf = nullptr;
-  e = dev_alloc((void**)&buf, 8 * (3 * m + 1 + scr_elems + 2), st);
-  if (e != cudaSuccess) return e;
-  uint64_t* flag = buf;
-  uint64_t* idx = buf + m;
-  uint64_t* item_start = buf + 2 * m;
-  uint64_t* scr = item_start + m + 1;
-  uint64_t* nitems = scr + scr_elems + 1;
-  k_item_flags<<<grid_for(m, 256, 8), 256, 0, st>>>(aux, m, n, flag);
-  e = cudaGetLastError();
-  if (e == cudaSuccess) e = scan_u64(flag, m, idx, scr, nitems, st);
-  if (e == cudaSuccess) {
-    k_item_starts<<<grid_for(m, 256, 8), 256, 0, st>>>(flag, idx, m, nitems, item_start);
-    e = cudaGetLastError();
-  }
-  if (e == cudaSuccess) {
-    const uint32_t smem = dtype == LECO_U32 ? kPackSmem32 : kPackSmem64;
-    // every item holds at least one partition: m bounds the count the grid is sized for
-    k_pack_items<<<resident_grid(k_pack_items, kPackBlock, m, smem), kPackBlock, smem, st>>>(
-        values, dtype, rec, aux, m, n, item_start, nitems, words, err);
-    e = cudaGetLastError();
-  }
-  cudaFreeAsync(buf, st);
-  return e;
+  if (dtype == LECO_U32)
+    return pcoef ? launch_pack_t<uint32_t, true>(values, n, m, L, tiles, rec, aux, pcoef, poly, words, st)
+                 : launch_pack_t<uint32_t, false>(values, n, m, L, tiles, rec, aux, nullptr, nullptr, words, st);
+  return pcoef ? launch_pack_t<uint64_t, true>(values, n, m, L, tiles, rec, aux, pcoef, poly, words, st)
+               : launch_pack_t<uint64_t, false>(values, n, m, L, tiles, rec, aux, nullptr, nullptr, words, st);
 }
 
 cudaError_t launch_part_col(const uint64_t* part_base, uint32_t ncols, uint64_t P, uint32_t* part_col, cudaStream_t st) {
@@ -1104,31 +1064,42 @@ cudaError_t launch_aux_multi(const Record* rec, const PolyCoef* pcoef, const Enc
   return cudaGetLastError();
 }
 
-uint32_t pack_item_values() { return kStageData / 8; }
-
 cudaError_t launch_word_bases(const uint64_t* col_bits, uint32_t ncols, uint64_t* word_base, cudaStream_t st) {
   k_word_bases<<<1, kWordBaseBlock, 0, st>>>(col_bits, ncols, word_base);
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint32_t* part_col,
-                              const uint64_t* word_base, const uint64_t* col_bits, const PackItem* items,
-                              uint64_t nitems, uint32_t ncols, uint64_t P, uint64_t W, int dtype, const Record* rec,
-                              const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly, uint64_t* words,
-                              uint32_t* err, cudaStream_t st) {
+template <typename T, bool POLY>
+cudaError_t launch_pack_multi_t(const EncCol* cols, const uint64_t* part_base, const uint64_t* tile_base,
+                                const uint64_t* word_base, uint32_t ncols, uint64_t tiles, uint32_t window,
+                                const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
+                                uint64_t* words, cudaStream_t st) {
+  const uint64_t jobs = tiles * (kScanTile / window);
+  k_pack_multi<T, POLY><<<grid_for(jobs, kPackWarps, 8), kPackBlock, 0, st>>>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
+                                                     aux, pcoef, poly, words);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* tile_base,
+                              const uint32_t* part_col, const uint64_t* word_base, const uint64_t* col_bits,
+                              uint32_t ncols, uint64_t P, uint64_t tiles, uint64_t W, int dtype, uint32_t window,
+                              const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
+                              uint64_t* words, cudaStream_t st) {
   if (W == 0) return cudaSuccess;
   k_zero_bounds_multi<<<grid_for(P > ncols ? P : ncols, 256, 8), 256, 0, st>>>(aux, part_col, word_base, col_bits,
                                                                                 ncols, P, words);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess || nitems == 0) return e;
-  const uint32_t smem = dtype == LECO_U32 ? kPackSmem32 : kPackSmem64;
-  if (pcoef)
-    k_pack_multi<true><<<resident_grid(k_pack_multi<true>, kPackBlock, nitems, smem), kPackBlock, smem, st>>>(
-        cols, part_base, word_base, items, nitems, dtype, rec, aux, pcoef, poly, words, err);
-  else
-    k_pack_multi<false><<<resident_grid(k_pack_multi<false>, kPackBlock, nitems, smem), kPackBlock, smem, st>>>(
-        cols, part_base, word_base, items, nitems, dtype, rec, aux, nullptr, nullptr, words, err);
-  return cudaGetLastError();
+  if (e != cudaSuccess || tiles == 0) return e;
+  if (window < 1024 || window > kScanTile || kScanTile % window) window = (uint32_t)kScanTile;
+  if (dtype == LECO_U32)
+    return pcoef ? launch_pack_multi_t<uint32_t, true>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
+                                                       aux, pcoef, poly, words, st)
+                 : launch_pack_multi_t<uint32_t, false>(cols, part_base, tile_base, word_base, ncols, tiles, window,
+                                                        rec, aux, nullptr, nullptr, words, st);
+  return pcoef ? launch_pack_multi_t<uint64_t, true>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
+                                                     aux, pcoef, poly, words, st)
+               : launch_pack_multi_t<uint64_t, false>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
+                                                      aux, nullptr, nullptr, words, st);
 }
 
 }  // namespace leco

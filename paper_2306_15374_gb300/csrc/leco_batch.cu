@@ -299,7 +299,7 @@ bool encode_args_ok(const void* const* d_vals, const uint64_t* n, const leco_mod
   return true;
 }
 
-// Host tables of a batched encode (columns, first partition / scan tile of each column, pack items)
+// Host tables of a batched encode (columns, first partition / scan tile of each column)
 // and the layout of its device blocks:
 //   meta:    records | decode table | tile descriptors | status words | polynomial table
 //   scratch: lenbits | scan scratch | col_bits | max_b | polynomial blocks | part_col
@@ -309,12 +309,11 @@ struct EncBatch {
   bool any_poly = false;
   std::vector<EncCol> ec;
   std::vector<uint64_t> part_base, tile_base;
-  std::vector<PackItem> items;
   uint64_t P = 0, T = 0;
   uint64_t rec_b = 0, tiles_b = 0, stat_b = 0, poly_b = 0, pc_words = 0, pcol_words = 0, scr_words = 0;
 
   EncBatch(const void* const* d_vals, const uint64_t* n, const leco_model* models, const uint32_t* L, uint32_t k,
-           leco_dtype dt, EncodeConfig cfg)
+           leco_dtype dt)
       : ncols(k), dtype(dt), ec(k), part_base(k + 1), tile_base(k + 1) {
     for (uint32_t c = 0; c < ncols; c++) any_poly = any_poly || models[c] == LECO_MODEL_POLY;
     part_base[0] = tile_base[0] = 0;
@@ -325,16 +324,6 @@ struct EncBatch {
     }
     P = part_base[ncols];
     T = tile_base[ncols];
-    // pack items: runs of consecutive partitions of one column that fit one staged copy
-    items.reserve(P / 4 + ncols);
-    const uint64_t item_vals = cfg.item_values >= 1 && cfg.item_values <= pack_item_values() ? cfg.item_values
-                                                                                             : pack_item_values();
-    for (uint32_t c = 0; c < ncols; c++) {
-      const uint64_t mc = part_base[c + 1] - part_base[c];
-      const uint64_t g = models[c] == LECO_MODEL_POLY ? 1 : (L[c] >= item_vals ? 1 : item_vals / L[c]);
-      for (uint64_t q = 0; q < mc; q += g)
-        items.push_back(PackItem{part_base[c] + q, c, (uint32_t)(mc - q < g ? mc - q : g)});
-    }
     auto a256 = [](uint64_t x) { return (x + 255) & ~255ull; };
     rec_b = a256(32 * (P ? P : 1));
     tiles_b = a256(sizeof(TileDesc) * (T ? T : 1));
@@ -447,14 +436,13 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   cudaStream_t st = (cudaStream_t)stream;
   int dev = 0;
   cudaGetDevice(&dev);
-  const EncBatch B(d_vals, n, models, L, ncols, dtype, cfg);
-  const uint64_t P = B.P, T = B.T, nitems = B.items.size();
+  const EncBatch B(d_vals, n, models, L, ncols, dtype);
+  const uint64_t P = B.P, T = B.T;
   char* meta = nullptr;
   uint64_t* scr = nullptr;
   EncCol* d_ec = nullptr;
   uint64_t* d_bases = nullptr;  // part_base | tile_base | word_base
   ColumnView* d_views = nullptr;
-  PackItem* d_items = nullptr;
   uint64_t* words = nullptr;
   std::vector<uint64_t> col_bits(ncols), word_base(ncols + 1);
   std::vector<uint32_t> max_b(ncols);
@@ -464,7 +452,6 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   if (e == cudaSuccess) e = dev_alloc((void**)&d_ec, sizeof(EncCol) * ncols, st);
   if (e == cudaSuccess) e = dev_alloc((void**)&d_bases, 8 * 3 * (uint64_t)(ncols + 1), st);
   if (e == cudaSuccess) e = dev_alloc((void**)&d_views, sizeof(ColumnView) * ncols, st);
-  if (e == cudaSuccess) e = dev_alloc((void**)&d_items, sizeof(PackItem) * (nitems ? nitems : 1), st);
   const EncPtrs p = enc_ptrs(B, meta, scr);
   uint64_t* d_part = d_bases;
   uint64_t* d_tile = d_bases + (ncols + 1);
@@ -475,8 +462,6 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
     e = cudaMemcpyAsync(d_part, B.part_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(d_tile, B.tile_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && nitems)
-    e = cudaMemcpyAsync(d_items, B.items.data(), sizeof(PackItem) * nitems, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = launch_part_col(d_part, ncols, P, p.part_col, st);
   // fit every partition of every column, then column-relative offsets and per-column totals
   if (e == cudaSuccess)
@@ -504,14 +489,13 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, d_ec, d_part, p.part_col, P, p.aux, p.poly, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(d_views, d_tile, ncols, T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(d_ec, d_part, p.part_col, d_word, p.colbits, d_items, nitems, ncols, P, W, dtype, p.rec,
-                          p.aux, p.pcoef, p.poly, words, p.status, st);
+    e = launch_pack_multi(d_ec, d_part, d_tile, p.part_col, d_word, p.colbits, ncols, P, T, W, dtype, cfg.item_values,
+                          p.rec, p.aux, p.pcoef, p.poly, words, st);
   if (e == cudaSuccess) e = make_batch_columns(B, p, words, word_base, col_bits, max_b, models, L, dev, st, meta, out);
   cudaFreeAsync(scr, st);
   cudaFreeAsync(d_ec, st);
   cudaFreeAsync(d_bases, st);
   cudaFreeAsync(d_views, st);
-  cudaFreeAsync(d_items, st);
   if (e != cudaSuccess) {
     if (meta) cudaFreeAsync(meta, st);
     if (words) cudaFreeAsync(words, st);
@@ -540,7 +524,6 @@ struct leco_batch_encode_plan {
   EncCol* d_ec = nullptr;
   uint64_t* d_bases = nullptr;  // part_base | tile_base | word_base
   ColumnView* d_views = nullptr;
-  PackItem* d_items = nullptr;
   uint64_t* words = nullptr;
   uint64_t words_cap = 0;  // 64-bit words reserved for the packed streams
   uint64_t runs = 0;       // graph launches so far
@@ -557,7 +540,7 @@ void enc_plan_release(leco_batch_encode_plan* p) {
   if (p->graph) cudaGraphDestroy(p->graph);
   if (p->capture) cudaStreamDestroy(p->capture);
   for (void* b : {(void*)p->meta, (void*)p->scr, p->poly_scr, (void*)p->d_ec, (void*)p->d_bases, (void*)p->d_views,
-                  (void*)p->d_items, (void*)p->words})
+                  (void*)p->words})
     if (b) cudaFree(b);
   delete p->B;
   delete p;
@@ -580,8 +563,8 @@ cudaError_t enc_plan_launches(leco_batch_encode_plan* pl, cudaStream_t st) {
   if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, pl->d_ec, d_part, p.part_col, B.P, p.aux, p.poly, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(pl->d_views, d_tile, B.ncols, B.T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(pl->d_ec, d_part, p.part_col, d_word, p.colbits, pl->d_items, B.items.size(), B.ncols, B.P,
-                          pl->words_cap, B.dtype, p.rec, p.aux, p.pcoef, p.poly, pl->words, p.status, st);
+    e = launch_pack_multi(pl->d_ec, d_part, d_tile, p.part_col, d_word, p.colbits, B.ncols, B.P, B.T, pl->words_cap,
+                          B.dtype, pl->cfg.item_values, p.rec, p.aux, p.pcoef, p.poly, pl->words, st);
   return e;
 }
 
@@ -654,7 +637,7 @@ extern "C" leco_status leco_batch_encode_plan_create(const void* const* d_vals, 
   if (!pl) return LECO_ERR_OOM;
   pl->device = dev;
   pl->cfg = encode_config_lookup(dtype);
-  pl->B = new (std::nothrow) EncBatch(d_vals, n, models, L, ncols, dtype, pl->cfg);
+  pl->B = new (std::nothrow) EncBatch(d_vals, n, models, L, ncols, dtype);
   if (!pl->B) {
     enc_plan_release(pl);
     return LECO_ERR_OOM;
@@ -677,14 +660,12 @@ extern "C" leco_status leco_batch_encode_plan_create(const void* const* d_vals, 
     cap += stream_words(bits);
   }
   pl->words_cap = cap;
-  const uint64_t nitems = B.items.size();
   cudaError_t e = cudaMalloc((void**)&pl->meta, B.meta_bytes());
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->scr, 8 * B.scr_words);
   if (e == cudaSuccess && B.any_poly) e = cudaMalloc(&pl->poly_scr, poly_fit_scratch_bytes(B.P ? B.P : 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_ec, sizeof(EncCol) * ncols);
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_bases, 8 * 3 * (uint64_t)(ncols + 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_views, sizeof(ColumnView) * ncols);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_items, sizeof(PackItem) * (nitems ? nitems : 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->words, 8 * cap);
   const EncPtrs p = enc_ptrs(B, pl->meta, pl->scr);
   const std::vector<ColumnView> views = enc_views(B, p, n, L);
@@ -697,8 +678,6 @@ extern "C" leco_status leco_batch_encode_plan_create(const void* const* d_vals, 
     e = cudaMemcpyAsync(pl->d_bases, B.part_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, cst);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(pl->d_bases + (ncols + 1), B.tile_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, cst);
-  if (e == cudaSuccess && nitems)
-    e = cudaMemcpyAsync(pl->d_items, B.items.data(), sizeof(PackItem) * nitems, cudaMemcpyHostToDevice, cst);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(pl->d_views, views.data(), sizeof(ColumnView) * ncols, cudaMemcpyHostToDevice, cst);
   // the partition -> column table depends on the shapes only: filled once, outside the graph
@@ -772,8 +751,7 @@ extern "C" uint64_t leco_batch_encode_plan_reserved_bytes(const leco_batch_encod
   const EncBatch& B = *plan->B;
   const uint64_t nc = B.ncols;
   return B.meta_bytes() + 8 * B.scr_words + (B.any_poly ? poly_fit_scratch_bytes(B.P ? B.P : 1) : 0) +
-         sizeof(EncCol) * nc + 8 * 3 * (nc + 1) + sizeof(ColumnView) * nc +
-         sizeof(PackItem) * (B.items.empty() ? 1 : B.items.size()) + 8 * plan->words_cap;
+         sizeof(EncCol) * nc + 8 * 3 * (nc + 1) + sizeof(ColumnView) * nc + 8 * plan->words_cap;
 }
 
 extern "C" void leco_batch_encode_plan_free(leco_batch_encode_plan* plan) {

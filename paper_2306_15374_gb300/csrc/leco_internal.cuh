@@ -299,22 +299,15 @@ cudaError_t launch_offsets_multi(Record* rec, const uint64_t* lenbits, const uin
                                  uint64_t* col_bits, cudaStream_t st);
 cudaError_t launch_aux_multi(const Record* rec, const PolyCoef* pcoef, const EncCol* cols, const uint64_t* part_base,
                              const uint32_t* part_col, uint64_t P, Aux* aux, PolyAux* poly, cudaStream_t st);
-// A pack item: k consecutive partitions p0 .. p0 + k - 1 (global indices) of column c, packed by one
-// CTA from one staged copy; at most pack_item_values() values, one partition for polynomial columns.
-struct PackItem {
-  uint64_t p0;
-  uint32_t c;
-  uint32_t k;
-};
-uint32_t pack_item_values();
 // word_base[c] = sum of stream_words(col_bits[k]) over k < c, for c = 0 .. ncols, on the device (one
 // CTA): each column's packed stream placed right after the previous one
 cudaError_t launch_word_bases(const uint64_t* col_bits, uint32_t ncols, uint64_t* word_base, cudaStream_t st);
-cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint32_t* part_col,
-                              const uint64_t* word_base, const uint64_t* col_bits, const PackItem* items,
-                              uint64_t nitems, uint32_t ncols, uint64_t P, uint64_t W, int dtype, const Record* rec,
-                              const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly, uint64_t* words,
-                              uint32_t* err, cudaStream_t st);
+// window: positions a warp packs (1024, 2048 or 4096); tiles: scan tiles of all columns
+cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* tile_base,
+                              const uint32_t* part_col, const uint64_t* word_base, const uint64_t* col_bits,
+                              uint32_t ncols, uint64_t P, uint64_t tiles, uint64_t W, int dtype, uint32_t window,
+                              const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
+                              uint64_t* words, cudaStream_t st);
 // poly: some column has a polynomial table (its tiles then get the exact polynomial bounds)
 cudaError_t launch_tile_desc_multi(const ColumnView* views, const uint64_t* tile_base, uint32_t ncols, uint64_t T,
                                    bool poly, TileDesc* tiles, cudaStream_t st);
@@ -332,8 +325,8 @@ __device__ __forceinline__ uint32_t find_col(const uint64_t* __restrict__ base, 
   return lo;
 }
 
-// Shape of the batched encode: values per pack item (a run of short partitions staged by one copy:
-// 1024, 2048 or 4096) and fit CTAs per SM (2, 3 or 4; fewer keep more of each partition in L2 for
+// Shape of the batched encode: values per pack item (a warp's window of positions: 1024, 2048 or 4096)
+// and fit CTAs per SM (2, 3 or 4; fewer keep more of each partition in L2 for
 // the fit's second pass). Tuned per value width by leco_tune_batch_encode.
 struct EncodeConfig {
   uint32_t item_values;
@@ -358,13 +351,10 @@ cudaError_t launch_offsets(Record* rec, const uint64_t* lenbits, uint64_t m, uin
 uint64_t offsets_scratch_elems(uint64_t m);
 cudaError_t launch_build_aux(const Record* rec, const PolyCoef* pcoef, uint64_t m, uint64_t n, Aux* aux,
                              PolyAux* poly, uint32_t* status, cudaStream_t st);
-cudaError_t launch_pack(const void* values, int dtype, const Record* rec, const Aux* aux, const PolyCoef* pcoef,
-                        const PolyAux* poly, uint64_t m, uint64_t n, uint64_t total_bits, uint64_t* words,
-                        uint64_t nwords, uint32_t* err, cudaStream_t st);
-// the same for a column of constant and linear partitions of any lengths (variable partitions):
-// short partitions that start in one 2048-position window share one staged copy
-cudaError_t launch_pack_var(const void* values, int dtype, const Record* rec, const Aux* aux, uint64_t m, uint64_t n,
-                            uint64_t total_bits, uint64_t* words, uint64_t nwords, uint32_t* err, cudaStream_t st);
+// L: the fixed partition length, or 0 with the column's tile descriptors for partitions of any lengths
+cudaError_t launch_pack(const void* values, int dtype, uint32_t L, const TileDesc* tiles, const Record* rec,
+                        const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly, uint64_t m, uint64_t n,
+                        uint64_t total_bits, uint64_t* words, uint64_t nwords, cudaStream_t st);
 
 // scans (k_scan.cu) and lookups (k_decode.cu)
 cudaError_t launch_tile_desc(const ColumnView& c, TileDesc* tiles, cudaStream_t st);

@@ -87,8 +87,8 @@ extern "C" leco_status leco_encode_fixed_noalloc(const void* d_values, uint64_t 
   if (nwords > words_cap) return LECO_ERR_INVALID_ARG;  // *nwords_out tells the size needed
   e = launch_build_aux(rec, nullptr, m, n, aux, nullptr, nullptr, st);
   if (e == cudaSuccess)
-    e = launch_pack(d_values, dtype, rec, aux, nullptr, nullptr, m, n, total, static_cast<uint64_t*>(d_words), nwords,
-                    err, st);
+    e = launch_pack(d_values, dtype, L, nullptr, rec, aux, nullptr, nullptr, m, n, total,
+                    static_cast<uint64_t*>(d_words), nwords, st);
   // A staging copy that gave up leaves part of the stream unwritten, and this call has no column
   // whose status word could carry the flag to a later leco_sync: read it back here, before the
   // next call's clear can erase it.
