@@ -211,10 +211,14 @@ __host__ __device__ FitParams solve_params(i128 S, int64_t mx, int64_t mn, uint3
       v = recip_of(dn);
 #endif
       const u128 t = a6 + (d - 1);
-      if (t >> (128 - sh)) return fallback_params(mx, mn);  // the quotient exceeds 64 bits
-      const u128 tn = t << sh;
-      if ((uint64_t)(tn >> 64) >= dn) return fallback_params(mx, mn);
-      Q = div_recip((uint64_t)(tn >> 64), (uint64_t)tn, dn, v);
+      if ((uint64_t)(t >> 64) == 0) {
+        Q = div_recip((uint64_t)t >> (64 - sh), (uint64_t)t << sh, dn, v);
+      } else {
+        if (t >> (128 - sh)) return fallback_params(mx, mn);  // the quotient exceeds 64 bits
+        const u128 tn = t << sh;
+        if ((uint64_t)(tn >> 64) >= dn) return fallback_params(mx, mn);
+        Q = div_recip((uint64_t)(tn >> 64), (uint64_t)tn, dn, v);
+      }
     } else {
       D = (i128)((u128)(uint64_t)N * ((uint64_t)N * N - 1));
       const i128 q = floordiv_i128((i128)a6 + D - 1, D);
@@ -236,9 +240,16 @@ __host__ __device__ FitParams solve_params(i128 S, int64_t mx, int64_t mn, uint3
   } else if (lin && fast && s >= 0) {
     // floor((2 a + D) / 2D) for q >= 0, -floor((2 a + D - 1) / 2D) below 0, with a = |6S| 2^s; the
     // result is below 2^53, so the dividend's high word is below the divisor's
-    const u128 t = ((a6 << s) << 1) + (u128)D - (neg ? 1u : 0u);
-    const u128 tn = t << (sh - 1);  // 2D normalised is D normalised
-    const uint64_t q = div_recip((uint64_t)(tn >> 64), (uint64_t)tn, dn, v);
+    // (2D normalised is D normalised: one place less)
+    uint64_t q;
+    if ((uint64_t)(a6 >> 64) == 0 && ((uint64_t)a6 >> (62 - s)) == 0) {
+      const uint64_t t = ((uint64_t)a6 << (s + 1)) + (uint64_t)D - (neg ? 1u : 0u);  // D < 2^63
+      q = div_recip((t >> 1) >> (64 - sh), t << (sh - 1), dn, v);
+    } else {
+      const u128 t = ((a6 << s) << 1) + (u128)D - (neg ? 1u : 0u);
+      const u128 tn = t << (sh - 1);
+      q = div_recip((uint64_t)(tn >> 64), (uint64_t)tn, dn, v);
+    }
     B = neg ? -(int64_t)q : (int64_t)q;
   } else if (lin) {
     const i128 sixS = neg ? -(i128)a6 : (i128)a6;

@@ -34,7 +34,6 @@ cudaError_t scan_u64(const uint64_t* in, uint64_t count, uint64_t* out, uint64_t
 namespace {
 
 constexpr uint64_t kChunk = 1ull << 16;
-constexpr uint64_t kNone = ~0ull;  // no merged size (pair longer than the cap)
 
 // ----------------------------------------------------------------------------------------- split
 //
@@ -590,201 +589,534 @@ int grid_for(uint64_t items, int per_block, int max_blocks_per_sm) {
 
 // ----------------------------------------------------------------------------------------- merge
 //
-// The moments of a span's values (w = the value as two's complement int64, x = the local index):
-// T0 = sum w, T1 = sum x w, and min and max of w. Two adjacent spans' moments combine exactly (the
-// right span's x shifts by the left span's length: T1 gains N_left T0_right), and they give the
-// least-squares moment S = sum (2x - (N-1)) w = 2 T1 - (N-1) T0 of the fit and its bounds, so a
-// refit needs one pass over the values: the residual range under the snapped line (none for the
-// constant model, whose residuals are the values themselves). The moments move with the partitions
-// when a round compacts them (a merged pair's are combined then), and the final partitions' fits
-// are taken once, from their moments, at the end.
-// a pair too long for one warp: its residual range is reduced over pieces of kPiece values
-struct LongPair {
-  uint64_t j;  // pair index
-  uint64_t k;  // slot of its left partition
-  uint64_t a;  // first position
-  FitParams P;
-  uint32_t N;
-  uint32_t pad;
-};
-
+// A partition is its start, its width b (a byte; its size is S_M + len b) and, beyond kStatVals values,
+// its values' moments (SpanStats, span_fit.cuh). The moments sit in a table by start / 32, where partitions
+// of more than 32 values never collide: they stay in place when partitions merge, so a round moves ten
+// bytes per partition. Shorter partitions' moments are taken from their values whenever they are needed,
+// which reads less than storing them would. A pair is its left partition's merged width mb, or
+//   kDirty  not fitted since one of its partitions changed,
+//   kNo     no gain (a pair that does not gain never merges and never keeps a neighbour from merging: its
+//           width does not matter) or longer than the cap.
+// While most pairs change (dense rounds) a round is: k_fit_spans (a lane fits a pair of up to kLaneVals
+// values by itself, from values the warp staged; longer pairs get their line there, from combined moments),
+// k_span_range (a warp takes a longer pair's residual range and stops as soon as the range rules out a
+// gain), k_select, a scan of the tiles' counts, k_compact. Once few pairs merge (sparse rounds), partitions
+// stay in their slots, linked left and right, and a round touches only the pairs that can merge and those
+// that changed.
+// Measured, 100M piecewise uint64 (45 rounds) and 250M 32-bit timestamps (62 rounds), against 16-byte sizes
+// and 48-byte moments moved every round, one kernel of 78 registers for fits of all lengths, and ten
+// launches and a host round trip per round to the end: whole passes 28.05 -> 20.46 ms and 18.37 -> 11.59 ms.
 constexpr uint32_t kTinySpan = 256;    // size search: a thread per sampled partition up to this size
-constexpr uint32_t kWarpSpan = 4096;   // a warp fits longer pairs up to this long (split partitions: any)
-constexpr uint32_t kPiece = 2048;      // values per piece of a longer pair
-constexpr int kGroupBlock = 256;       // 8 warps, each taking 32 spans at a time
-constexpr uint32_t kStageBytes = 4096; // per warp: a group's values are staged when they fit
+constexpr uint32_t kLaneVals = 64;     // a lane fits spans up to this long on its own
+constexpr uint32_t kStatVals = 32;     // longer partitions carry their moments (at most kLaneVals; the table's stride)
+constexpr uint32_t kPieceVals = 4096;  // a warp takes the residual range of a span up to this long; pieces above
+constexpr int kSpanBlock = 128;        // k_fit_spans: 4 warps, each taking 32 spans at a time
+constexpr uint32_t kSpanStage = 1088;  // staged differences per warp
+constexpr uint32_t kTileVals = 512;    // spans up to this long take eight lanes, four at a time, longer ones a warp
+constexpr uint8_t kNo = 0xFF, kDirty = 0xFE, kDead = 0xFD;
+constexpr uint32_t kSlotEnd = 0xFFFFFFFFu;
+// sparse rounds begin below one merge in kSparseShare partitions, or at kSparseBelow partitions, where a dense
+// round's launches and host round trip cost more than its work
+constexpr uint64_t kSparseShare = 16, kSparseBelow = 32768;
 
-struct MergeWork {
-  LongPair* longs;
-  uint64_t* pieces;
-  unsigned long long* counters;  // [long pairs, pieces]
-  long long* lo;                 // per long pair
-  long long* hi;
-  unsigned long long* zmax;
+// a longer span and its line (fallback: B is the shift); bmax: widths above it bring no gain
+struct SpanJob {
+  uint64_t a;
+  int64_t B;
+  uint64_t j;
+  uint32_t N;
+  int8_t s;
+  uint8_t fallback;
+  uint8_t bmax;
+  uint8_t narrow;  // values within 2^30 of each other, line within 2^30 (span_fit.cuh)
+};
+static_assert(sizeof(SpanJob) == 32, "span job layout");
+
+// piece q of np of a job beyond kPieceVals, whose range is gathered in slot mi
+struct SpanPiece {
+  uint32_t e, mi, q, np;
 };
 
-// Full fits of spans. MODE 1: every partition of the split (its moments from a pass over its
-// values, into stats[j]; size S_M + len * b into size_out[j]). MODE 2: the dirty adjacent pairs
-// [st[j], st[j + 2)) (moments combined from stats[j] and stats[j + 1]; merged size into
-// size_out[j]). MODE 3: the final partitions (moments stats[j]; record into rec[j], as the
-// encoder's fit writes it). A warp takes 32 consecutive spans; when their values cover at most
-// kStageBytes it first stages them in shared memory with coalesced loads. A lane then fits its own
-// span when it is at most kLaneSpan long, tiles of eight lanes fit spans up to kTileSpan, the warp
-// fits longer ones together, and spans longer than
-// kWarpSpan (modes 2 and 3, not staged) go to the piece list, where many warps share their residual
-// pass (k_pair_pieces, then k_pair_finish).
+struct SpanWork {
+  SpanJob* jobs;
+  SpanPiece* pieces;
+  long long *lo, *hi;  // per slot
+  unsigned long long* zmax;
+  uint32_t* done;
+  unsigned long long* cnt;  // jobs, pieces, slots
+};
+
+// a span's job (and pieces) at place e of the list
+__device__ __forceinline__ void put_job(const SpanWork& w, uint64_t e, uint64_t a, uint32_t N, uint64_t j,
+                                        const FitParams& P, uint32_t bmax, bool narrow, bool pieces) {
+  SpanJob q;
+  q.a = a;
+  q.B = P.fallback ? P.fb_shift : P.B;
+  q.j = j;
+  q.N = N;
+  q.s = (int8_t)P.s;
+  q.fallback = (uint8_t)P.fallback;
+  q.bmax = (uint8_t)bmax;
+  q.narrow = narrow ? 1 : 0;
+  w.jobs[e] = q;
+  if (!pieces || N <= kPieceVals) return;
+  const uint32_t np = (N + kPieceVals - 1) / kPieceVals;
+  const unsigned long long mi = atomicAdd(&w.cnt[2], 1ull), pb = atomicAdd(&w.cnt[1], (unsigned long long)np);
+  w.lo[mi] = INT64_MAX;
+  w.hi[mi] = INT64_MIN;
+  w.zmax[mi] = 0;
+  w.done[mi] = 0;
+  for (uint32_t k = 0; k < np; k++) w.pieces[pb + k] = SpanPiece{(uint32_t)e, (uint32_t)mi, k, np};
+}
+
+// the largest width that gains when partitions of N1 and N2 values and widths b1 and b2 merge:
+// S_M + N b < 2 S_M + N1 b1 + N2 b2
+__device__ __forceinline__ uint32_t gain_width(uint32_t N1, uint32_t b1, uint32_t N2, uint32_t b2) {
+  return min(((uint32_t)kSmBits + N1 * b1 + N2 * b2 - 1u) / (N1 + N2), 64u);  // lengths below 2^25, widths up to 64
+}
+
+__device__ __forceinline__ Record span_record(uint64_t a, const FitResult& R) {
+  Record r;
+  r.theta0 = R.theta0;
+  r.theta1 = R.theta1;
+  r.start = a;
+  r.word3 = make_w3(0, R.b, R.s, 1);
+  return r;
+}
+
+// the moments of a partition: from the table, or from its values when it is short
+template <typename T>
+__device__ __forceinline__ SpanStats part_stats(const T* __restrict__ v, uint64_t a, uint32_t N,
+                                                const SpanStats* __restrict__ stats) {
+  return N > kStatVals ? stats[a / kStatVals] : lane_stats(v + a, N);
+}
+
+template <typename T>
+struct SpanArgs {
+  const T* v;
+  uint32_t cap;
+  int model;
+  SpanStats* stats;
+  SpanWork w;
+};
+
+// Fits of the spans [st[j], st[j + W]), j < count, a lane each. MODE 1: the split's partitions (b[j];
+// moments of those beyond kStatVals into the table; those beyond kLaneVals are listed for k_fit_long).
+// MODE 2: the dirty pairs (W = 2; mb[j]). MODE 3: the final partitions (rec[j]). Spans beyond kLaneVals get
+// their line from their moments and go to the job list. The warp stages the values of its short spans as
+// 32-bit differences from the first one, which leaves both passes over them in 32 bits; values too far
+// apart are read from memory in 64 bits instead.
 template <typename T, int MODE>
-__global__ void __launch_bounds__(kGroupBlock, 3)
-    k_span_groups(const T* __restrict__ v, const uint64_t* __restrict__ st, uint64_t count, uint32_t cap, int model,
-                  const uint8_t* __restrict__ dirty, SpanStats* __restrict__ stats, uint64_t* __restrict__ size_out,
-                  Record* __restrict__ rec, MergeWork mw) {
+__global__ void __launch_bounds__(kSpanBlock, 8)
+    k_fit_spans(const SpanArgs<T> A, const uint64_t* __restrict__ st, uint64_t count, uint8_t* __restrict__ b,
+                uint8_t* __restrict__ mb, Record* __restrict__ rec) {
   constexpr int W = MODE == 2 ? 2 : 1;
-  __shared__ __align__(16) unsigned char stage_raw[kGroupBlock / 32][kStageBytes];
-  constexpr uint64_t kStageVals = kStageBytes / sizeof(T);
+  __shared__ int32_t raw[kSpanBlock / 32][kSpanStage];
   const uint32_t lane = threadIdx.x & 31u, wib = threadIdx.x >> 5;
-  T* stage = reinterpret_cast<T*>(stage_raw[wib]);
-  const uint64_t ngroups = (count + 31) / 32;
-  const uint64_t gw = (uint64_t)gridDim.x * (kGroupBlock / 32);
-  for (uint64_t g = (uint64_t)blockIdx.x * (kGroupBlock / 32) + wib; g < ngroups; g += gw) {
+  int32_t* stage = raw[wib];
+  const uint64_t groups = (count + 31) / 32, gw = (uint64_t)gridDim.x * (kSpanBlock / 32);
+  for (uint64_t g = (uint64_t)blockIdx.x * (kSpanBlock / 32) + wib; g < groups; g += gw) {
     const uint64_t j = g * 32 + lane;
-    bool act = j < count && (MODE != 2 || dirty[j]);
+    bool act = j < count && (MODE != 2 || mb[j] == kDirty);
     if (!__any_sync(kFull, act)) continue;
-    uint64_t a = 0, c = 0;
+    uint64_t a = 0, mid = 0, c = 0;
+    uint32_t bmax = 64;
     if (act) {
       a = st[j];
       c = st[j + W];
-      if (W == 2 && c - a > cap) {  // pairs beyond the cap never merge
-        size_out[j] = kNone;
-        act = false;
+      if (W == 2) {
+        mid = st[j + 1];
+        if (c - a > A.cap) {
+          mb[j] = kNo;
+          act = false;
+        } else {
+          bmax = gain_width((uint32_t)(mid - a), b[j], (uint32_t)(c - mid), b[j + 1]);
+        }
       }
     }
     const uint32_t N = act ? (uint32_t)(c - a) : 0u;
-    const uint64_t ga = xw_min_u(act ? a : ~0ull), gc = xw_max_u(act ? c : 0ull);
-    const bool staged = ga != ~0ull && gc - ga <= kStageVals;
-    if (staged) {
-      for (uint64_t t = lane; t < gc - ga; t += 32) stage[t] = __ldg(v + ga + t);
-      __syncwarp();
+    const bool small = act && N <= kLaneVals;
+    const uint32_t smalls = __ballot_sync(kFull, small);
+    uint64_t ga = 0;
+    int64_t ref = 0;
+    bool narrow = false;
+    if (smalls) {  // their values, from the first one's start to the last one's end
+      ga = __shfl_sync(kFull, a, __ffs((int)smalls) - 1);
+      const uint64_t gc = __shfl_sync(kFull, c, 31 - __clz((int)smalls));
+      if (gc - ga <= kSpanStage) {
+        const uint32_t len = (uint32_t)(gc - ga);
+        ref = (int64_t)__ldg(A.v + ga);
+        bool ok = narrow_ref(ref);
+#pragma unroll 4
+        for (uint32_t t = lane; t < len; t += 32) {
+          const int64_t d = (int64_t)__ldg(A.v + ga + t) - ref;
+          ok = ok && narrow_diff(d);
+          stage[t] = (int32_t)d;
+        }
+        narrow = __all_sync(kFull, ok);
+        __syncwarp();
+      }
     }
-    const T* src = staged ? stage + (a - ga) : v + a;
-    // moments
+    const bool lin = A.model == LECO_MODEL_LINEAR && N >= 2;
+    const int32_t* dp = stage + (uint32_t)(a - ga);
     SpanStats S;
+    i128 moment = 0;
     S.T0 = S.T1 = 0;
     S.mn = S.mx = 0;
-    if (MODE == 1) {
-      if (act && N <= kLaneSpan) S = stats_part(src, 0, N, 1);
-      coop_stats<8>(__ballot_sync(kFull, act && N > kLaneSpan && N <= kTileSpan), src, N, S);
-      coop_stats<32>(__ballot_sync(kFull, act && N > kTileSpan), src, N, S);
-    } else if (MODE == 2 && act) {
-      S = combine_stats(stats[j], st[j + 1] - a, stats[j + 1]);
-    } else if (act) {
-      S = stats[j];
+    if (small && narrow) {
+      int64_t sum = 0, Sd = 0;
+      int32_t mn = INT32_MAX, mx = INT32_MIN, u = 1 - (int32_t)N;  // u = 2 x - (N - 1)
+#pragma unroll 4
+      for (uint32_t x = 0; x < N; x++, u += 2) {
+        const int32_t d = dp[x];
+        mn = min(mn, d);
+        mx = max(mx, d);
+        sum += (int64_t)u * d;
+        if (W == 1) Sd += d;
+      }
+      S.mn = ref + mn;
+      S.mx = ref + mx;
+      moment = sum;
+      if (MODE == 1 && N > kStatVals) A.stats[a / kStatVals] = stats_from(ref, N, Sd, sum, mn, mx);
+    } else if (small) {
+      S = lane_stats(A.v + a, N);
+      moment = line_moment(S, N);
+      if (MODE == 1 && N > kStatVals) A.stats[a / kStatVals] = S;
+    } else if (act && MODE != 1) {
+      if (W == 2)
+        S = combine_stats(part_stats(A.v, a, (uint32_t)(mid - a), A.stats), mid - a,
+                          part_stats(A.v, mid, (uint32_t)(c - mid), A.stats));
+      else
+        S = A.stats[a / kStatVals];
+      moment = line_moment(S, N);
     }
-    // parameters (fit.cuh steps 1-3)
-    const bool lin = model == LECO_MODEL_LINEAR && N >= 2;
     FitParams P;
     P.B = 0;
     P.fb_shift = 0;
     P.s = 0;
     P.fallback = 0;
-    if (act) P = solve_params(lin ? 2 * S.T1 - mul_i128_u64(S.T0, N - 1) : (i128)0, S.mx, S.mn, N, lin);
-    // residual range (step 4)
-    int64_t lo = INT64_MAX, hi = INT64_MIN;
+    if (act && (small || MODE != 1)) P = solve_params(lin ? moment : (i128)0, S.mx, S.mn, N, lin);
+    // the residual range; the constant model's residuals on its grid are the values themselves
+    int64_t lo = S.mn, hi = S.mx;
     uint64_t zmax = 0;
-    const bool need = act && (lin || P.fallback);
-    if (act && !need) {  // constant model on its grid: the residuals are the values
-      lo = S.mn;
-      hi = S.mx;
-    }
-    const bool by_lane = need && N <= kLaneSpan;
-    const bool by_warp = need && N > kLaneSpan && (MODE == 1 || staged || N <= kWarpSpan);
-    const bool by_pieces = need && !by_lane && !by_warp;
-    if (by_lane) resid_part(src, 0, N, 1, P, lo, hi, zmax);
-    coop_resid<8>(__ballot_sync(kFull, by_warp && N <= kTileSpan), src, N, P, lo, hi, zmax);
-    coop_resid<32>(__ballot_sync(kFull, by_warp && N > kTileSpan), src, N, P, lo, hi, zmax);
-    if (by_pieces) {
-      const uint32_t np = (N + kPiece - 1) / kPiece;
-      const unsigned long long li = atomicAdd(&mw.counters[0], 1ull);
-      const unsigned long long pb = atomicAdd(&mw.counters[1], (unsigned long long)np);
-      LongPair lp;
-      lp.j = j;
-      lp.k = 0;
-      lp.a = a;
-      lp.P = P;
-      lp.N = N;
-      lp.pad = 0;
-      mw.longs[li] = lp;
-      mw.lo[li] = INT64_MAX;
-      mw.hi[li] = INT64_MIN;
-      mw.zmax[li] = 0;
-      for (uint32_t q = 0; q < np; q++) mw.pieces[pb + q] = ((uint64_t)li << 16) | q;
-    }
-    if (act && !by_pieces) {  // steps 5-6
-      if (MODE == 3) {
-        const FitResult R = finish_fit(P, lo, hi, zmax);
-        Record r;
-        r.theta0 = R.theta0;
-        r.theta1 = R.theta1;
-        r.start = a;
-        r.word3 = make_w3(0, R.b, R.s, 1);
-        rec[j] = r;
+    const bool need = lin || P.fallback;
+    const bool flat = act && narrow_line(P, N);
+    if (small && need) {
+      lo = INT64_MAX;
+      hi = INT64_MIN;
+      if (narrow && flat) {
+        const NarrowLine line(P.B, P.s);
+        int32_t l = INT32_MAX, h = INT32_MIN;
+        uint64_t G = 0;
+#pragma unroll 4
+        for (uint32_t x = 0; x < N; x++, G += line.B) {
+          const int32_t r = dp[x] - line.at(G);
+          l = min(l, r);
+          h = max(h, r);
+        }
+        lo = ref + l;
+        hi = ref + h;
       } else {
-        size_out[j] = kSmBits + (uint64_t)N * finish_width(P, lo, hi, zmax);
+        resid_part(A.v + a, 0, N, 1, P, lo, hi, zmax);
       }
-      if (MODE == 1) stats[j] = S;
+    }
+    const bool job = act && !small && (MODE == 1 || need);
+    if (act && !job) {
+      if (MODE == 3) {
+        rec[j] = span_record(a, finish_fit(P, lo, hi, zmax));
+      } else {
+        const uint32_t w = finish_width(P, lo, hi, zmax);
+        if (MODE == 1)
+          b[j] = (uint8_t)w;
+        else
+          mb[j] = w <= bmax ? (uint8_t)w : kNo;
+      }
+    }
+    const uint32_t jobs = __ballot_sync(kFull, job);
+    if (jobs) {
+      unsigned long long e = 0;
+      if (lane == 0) e = atomicAdd(&A.w.cnt[0], (unsigned long long)__popc(jobs));
+      e = __shfl_sync(kFull, e, 0) + __popc(jobs & ((1u << lane) - 1u));
+      if (job) {
+        const bool near = flat && narrow_ref(S.mn) && narrow_diff(S.mx - S.mn);
+        put_job(A.w, e, a, N, j, P, bmax, near, MODE != 1);
+        if (MODE == 1 && N > kPieceVals) A.w.pieces[atomicAdd(&A.w.cnt[1], 1ull)] = SpanPiece{(uint32_t)e, 0, 0, 1};
+      }
     }
     __syncwarp();  // the stage is reused by the next group
   }
 }
 
-// residual range of one piece of a long pair per warp, folded into the pair's range by atomics
-template <typename T>
-__global__ void __launch_bounds__(256) k_pair_pieces(const T* __restrict__ v, MergeWork mw) {
-  const uint64_t np = *(volatile unsigned long long*)&mw.counters[1];
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t nw = ((uint64_t)gridDim.x * blockDim.x) >> 5;
-  for (uint64_t pi = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5; pi < np; pi += nw) {
-    const uint64_t e = mw.pieces[pi];
-    const uint64_t li = e >> 16;
-    const uint32_t q = (uint32_t)(e & 0xFFFFu);
-    const LongPair L = mw.longs[li];
-    const uint32_t x0 = q * kPiece, x1 = min(x0 + kPiece, L.N);
-    int64_t lo = INT64_MAX, hi = INT64_MIN;
-    uint64_t z = 0;
-    resid_part(v + L.a, x0 + lane, x1, 32, L.P, lo, hi, z);
-    lo = warp_min_i64(lo);
-    hi = warp_max_i64(hi);
-    z = warp_max_u64(z);
-    if (lane == 0) {
-      atomicMin(&mw.lo[li], (long long)lo);
-      atomicMax(&mw.hi[li], (long long)hi);
-      atomicMax(&mw.zmax[li], (unsigned long long)z);
-    }
+// One listed partition of the split by a tile of TILE lanes (N = 0: the tile only takes part in the
+// warp's steps): moments into the table, line, residual range, width
+template <int TILE, typename T>
+__device__ __forceinline__ void fit_listed(const SpanArgs<T>& A, uint64_t a, uint32_t N, uint64_t j, uint8_t* __restrict__ b,
+                                           uint32_t r) {
+  const T* p = A.v + a;
+  const bool lin = A.model == LECO_MODEL_LINEAR;
+  const int64_t ref = N ? (int64_t)__ldg(p) : 0;
+  bool ok = narrow_ref(ref);
+  int64_t sum = 0, Sd = 0;
+  int32_t mn = INT32_MAX, mx = INT32_MIN;
+  const int32_t nm1 = (int32_t)N - 1;
+#pragma unroll 4
+  for (uint32_t x = r; x < N; x += TILE) {
+    const int64_t d = (int64_t)__ldg(p + x) - ref;
+    ok = ok && narrow_diff(d);
+    const int32_t e = (int32_t)d;
+    mn = min(mn, e);
+    mx = max(mx, e);
+    Sd += e;
+    sum += (int64_t)(2 * (int32_t)x - nm1) * e;
   }
-}
-
-// steps 5-6 of the long spans: their merged size (msz) or their record (rec)
-__global__ void k_pair_finish(MergeWork mw, uint64_t* __restrict__ msz, Record* __restrict__ rec) {
-  const uint64_t nl = *(volatile unsigned long long*)&mw.counters[0];
-  for (uint64_t li = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; li < nl; li += (uint64_t)gridDim.x * blockDim.x) {
-    const LongPair L = mw.longs[li];
-    if (rec) {
-      const FitResult R = finish_fit(L.P, (int64_t)mw.lo[li], (int64_t)mw.hi[li], (uint64_t)mw.zmax[li]);
-      Record r;
-      r.theta0 = R.theta0;
-      r.theta1 = R.theta1;
-      r.start = L.a;
-      r.word3 = make_w3(0, R.b, R.s, 1);
-      rec[L.j] = r;
+  SpanStats S;
+  i128 moment;
+  const bool near = __all_sync(kFull, ok);
+  if (near) {
+    mn = tile_min<TILE>(mn);
+    mx = tile_max<TILE>(mx);
+    Sd = tile_sum<TILE>(Sd);
+    sum = tile_sum<TILE>(sum);
+    S = stats_from(ref, N, Sd, sum, mn, mx);
+    moment = sum;
+  } else {
+    S = group_stats<TILE>(p, r, N, (uint32_t)TILE);
+    moment = line_moment(S, N);
+  }
+  if (N && r == 0) A.stats[a / kStatVals] = S;
+  FitParams P;
+  P.B = 0;
+  P.fb_shift = 0;
+  P.s = 0;
+  P.fallback = 0;
+  if (N) P = solve_params(lin ? moment : (i128)0, S.mx, S.mn, N, lin);
+  int64_t lo = S.mn, hi = S.mx;
+  uint64_t zmax = 0;
+  if (__any_sync(kFull, N && (lin || P.fallback))) {
+    if (__all_sync(kFull, !N || (near && narrow_line(P, N)))) {
+      const NarrowLine line(P.B, P.s);
+      int32_t l = INT32_MAX, h = INT32_MIN;
+      uint64_t G = line.B * r;
+      const uint64_t dG = line.B * (uint64_t)TILE;
+#pragma unroll 4
+      for (uint32_t x = r; x < N; x += TILE, G += dG) {
+        const int32_t e = (int32_t)((uint32_t)__ldg(p + x) - (uint32_t)ref) - line.at(G);
+        l = min(l, e);
+        h = max(h, e);
+      }
+      lo = ref + tile_min<TILE>(l);
+      hi = ref + tile_max<TILE>(h);
     } else {
-      msz[L.j] = kSmBits + (uint64_t)L.N * finish_width(L.P, (int64_t)mw.lo[li], (int64_t)mw.hi[li], (uint64_t)mw.zmax[li]);
+      lo = INT64_MAX;
+      hi = INT64_MIN;
+      resid_part(p, r, N, (uint32_t)TILE, P, lo, hi, zmax);
+      lo = tile_min<TILE>(lo);
+      hi = tile_max<TILE>(hi);
+      zmax = tile_max<TILE>(zmax);
+    }
+  }
+  if (N && r == 0) b[j] = (uint8_t)finish_width(P, lo, hi, zmax);
+}
+
+// the listed partitions of the split up to kPieceVals values: four at a time, those beyond kTileVals one
+// after another
+template <typename T>
+__global__ void __launch_bounds__(256) k_fit_long(const SpanArgs<T> A, uint8_t* __restrict__ b) {
+  const uint64_t nj = *(volatile unsigned long long*)&A.w.cnt[0];
+  const uint32_t lane = threadIdx.x & 31u, r = lane & 7u;
+  for (uint64_t e0 = ((uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5)) * 4; e0 < nj; e0 += (uint64_t)gridDim.x * 32) {
+    const uint64_t e = e0 + (lane >> 3);
+    SpanJob q = {};
+    if (e < nj) q = A.w.jobs[e];
+    fit_listed<8>(A, q.a, q.N <= kTileVals ? q.N : 0u, q.j, b, r);
+    uint32_t big = __ballot_sync(kFull, r == 0 && q.N > kTileVals && q.N <= kPieceVals);
+    while (big) {
+      const int src = __ffs((int)big) - 1;
+      big &= big - 1;
+      fit_listed<32>(A, __shfl_sync(kFull, q.a, src), __shfl_sync(kFull, q.N, src), __shfl_sync(kFull, q.j, src), b, lane);
     }
   }
 }
 
-__device__ __forceinline__ bool pair_gain(const uint64_t* sz, const uint64_t* msz, uint64_t j, int64_t* g) {
-  if (msz[j] == kNone) return false;
-  *g = (int64_t)(sz[j] + sz[j + 1]) - (int64_t)msz[j];
-  return true;
+// ... and those beyond, a CTA each (at most 2^16 values: a split's partition ends with its chunk)
+template <typename T>
+__global__ void __launch_bounds__(256) k_fit_longest(const SpanArgs<T> A, uint8_t* __restrict__ b) {
+  __shared__ SpanStats part[8];
+  __shared__ int64_t plo[8], phi[8];
+  __shared__ uint64_t pz[8];
+  const uint64_t np = *(volatile unsigned long long*)&A.w.cnt[1];
+  const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
+  for (uint64_t k = blockIdx.x; k < np; k += gridDim.x) {
+    const SpanJob q = A.w.jobs[A.w.pieces[k].e];
+    const T* p = A.v + q.a;
+    SpanStats S = group_stats<32>(p, threadIdx.x, q.N, 256);
+    if (lane == 0) part[wid] = S;
+    __syncthreads();
+    S = part[0];
+    for (int w = 1; w < 8; w++) {
+      S.T0 += part[w].T0;
+      S.T1 += part[w].T1;
+      S.mn = min(S.mn, part[w].mn);
+      S.mx = max(S.mx, part[w].mx);
+    }
+    if (threadIdx.x == 0) A.stats[q.a / kStatVals] = S;
+    const bool lin = A.model == LECO_MODEL_LINEAR;
+    const FitParams P = solve_params(lin ? line_moment(S, q.N) : (i128)0, S.mx, S.mn, q.N, lin);
+    int64_t lo = S.mn, hi = S.mx;
+    uint64_t zmax = 0;
+    if (lin || P.fallback) {
+      lo = INT64_MAX;
+      hi = INT64_MIN;
+      resid_part(p, threadIdx.x, q.N, 256, P, lo, hi, zmax);
+      lo = tile_min<32>(lo);
+      hi = tile_max<32>(hi);
+      zmax = tile_max<32>(zmax);
+      if (lane == 0) {
+        plo[wid] = lo;
+        phi[wid] = hi;
+        pz[wid] = zmax;
+      }
+      __syncthreads();
+      for (int w = 0; w < 8; w++) {
+        lo = min(lo, plo[w]);
+        hi = max(hi, phi[w]);
+        zmax = max(zmax, pz[w]);
+      }
+    }
+    if (threadIdx.x == 0) b[q.j] = (uint8_t)finish_width(P, lo, hi, zmax);
+    __syncthreads();  // the shared parts are reused
+  }
+}
+
+__device__ __forceinline__ FitParams job_line(const SpanJob& q) {
+  FitParams P;
+  P.s = q.s;
+  P.fallback = q.fallback;
+  P.B = q.fallback ? 0 : q.B;
+  P.fb_shift = q.fallback ? q.B : 0;
+  return P;
+}
+
+// Residual range of values x0 + r, + TILE, ... < x1 of a listed span, reduced over the tile. narrow: every
+// tile of the warp has a narrow span. CHECK (a warp per span): stops once the range alone needs more than
+// bmax bits, first at 32 values spread over a long span (which settles most pairs that do not belong together).
+template <int TILE, bool CHECK, typename T>
+__device__ __forceinline__ void job_range(const T* __restrict__ p, const SpanJob& q, uint32_t x0, uint32_t x1, uint32_t r,
+                                          bool narrow, int64_t& lo, int64_t& hi, uint64_t& zmax) {
+  if (narrow) {
+    const NarrowLine line(q.B, q.s);
+    const uint32_t ref = x0 < x1 ? (uint32_t)__ldg(p) : 0u;
+    int32_t l = INT32_MAX, h = INT32_MIN;
+    auto pass = [&](uint32_t xa, uint32_t xb, uint32_t step) {
+      uint64_t G = line.B * xa;
+      const uint64_t dG = line.B * (uint64_t)step;
+#pragma unroll 4
+      for (uint32_t x = xa; x < xb; x += step, G += dG) {
+        const int32_t e = (int32_t)((uint32_t)__ldg(p + x) - ref) - line.at(G);
+        l = min(l, e);
+        h = max(h, e);
+      }
+    };
+    if (CHECK && q.bmax < 31) {
+      bool over = false;
+      if (x1 - x0 >= 1024) {
+        const uint32_t x = x0 + r * ((x1 - x0) >> 5);
+        pass(x, x + 1, 1);
+        over = ((uint32_t)tile_max<TILE>(h) - (uint32_t)tile_min<TILE>(l)) >> q.bmax != 0;
+      }
+      for (uint32_t x = x0; x < x1 && !over; x += 1024) {
+        pass(x + r, min(x + 1024u, x1), TILE);
+        if (x + 1024 < x1) over = __any_sync(kFull, l <= h && ((uint32_t)h - (uint32_t)l) >> q.bmax != 0);
+      }
+    } else {
+      pass(x0 + r, x1, TILE);
+    }
+    // 32-bit differences from the span's first value: whole again by its 64 bits
+    const int64_t ref64 = x0 < x1 ? (int64_t)__ldg(p) : 0;
+    lo = ref64 + tile_min<TILE>(l);
+    hi = ref64 + tile_max<TILE>(h);
+    zmax = 0;
+    return;
+  }
+  const FitParams P = job_line(q);
+  lo = INT64_MAX;
+  hi = INT64_MIN;
+  zmax = 0;
+  if (CHECK && q.bmax < 63 && !P.fallback) {
+    bool over = false;
+    for (uint32_t x = x0; x < x1 && !over; x += 1024) {
+      resid_part(p, x + r, min(x + 1024u, x1), (uint32_t)TILE, P, lo, hi, zmax);
+      if (x + 1024 < x1) over = __any_sync(kFull, lo <= hi && ((uint64_t)hi - (uint64_t)lo) >> q.bmax != 0);
+    }
+  } else {
+    resid_part(p, x0 + r, x1, (uint32_t)TILE, P, lo, hi, zmax);
+  }
+  lo = tile_min<TILE>(lo);
+  hi = tile_max<TILE>(hi);
+  zmax = tile_max<TILE>(zmax);
+}
+
+__device__ __forceinline__ void finish_job(const SpanJob& q, int64_t lo, int64_t hi, uint64_t zmax, uint8_t* __restrict__ mb,
+                                           Record* __restrict__ rec) {
+  const FitParams P = job_line(q);
+  if (rec) {
+    rec[q.j] = span_record(q.a, finish_fit(P, lo, hi, zmax));
+  } else {
+    const uint32_t w = finish_width(P, lo, hi, zmax);
+    mb[q.j] = w <= q.bmax ? (uint8_t)w : kNo;
+  }
+}
+
+// Residual ranges of the listed spans under their lines, then the width (mb) or the record (rec): four spans
+// of up to kTileVals values per warp at a time, longer ones a warp each, pieces of those beyond kPieceVals. A
+// range that rules out a gain may be cut short: the width is at least bitlen(hi - lo) whatever the intercept.
+template <typename T>
+__global__ void __launch_bounds__(256) k_span_range(const SpanArgs<T> A, uint8_t* __restrict__ mb, Record* __restrict__ rec) {
+  const uint64_t nj = *(volatile unsigned long long*)&A.w.cnt[0], np = *(volatile unsigned long long*)&A.w.cnt[1];
+  const uint32_t lane = threadIdx.x & 31u, r = lane & 7u;
+  const uint64_t gw = (uint64_t)blockIdx.x * 8 + (threadIdx.x >> 5), nw = (uint64_t)gridDim.x * 8;
+  for (uint64_t e0 = gw * 4; e0 < nj; e0 += nw * 4) {
+    const uint64_t e = e0 + (lane >> 3);
+    SpanJob q = {};
+    if (e < nj) q = A.w.jobs[e];
+    const bool tiled = q.N && q.N <= kTileVals;
+    int64_t lo, hi;
+    uint64_t zmax;
+    if (__any_sync(kFull, tiled)) {
+      job_range<8, false>(A.v + q.a, q, 0, tiled ? q.N : 0u, r, __all_sync(kFull, !tiled || q.narrow), lo, hi, zmax);
+      if (tiled && r == 0) finish_job(q, lo, hi, zmax, mb, rec);
+    }
+    uint32_t big = __ballot_sync(kFull, r == 0 && q.N > kTileVals && q.N <= kPieceVals);
+    while (big) {
+      const int src = __ffs((int)big) - 1;
+      big &= big - 1;
+      const SpanJob one = A.w.jobs[e0 + (uint64_t)(src >> 3)];
+      job_range<32, true>(A.v + one.a, one, 0, one.N, lane, one.narrow != 0, lo, hi, zmax);
+      if (lane == 0) finish_job(one, lo, hi, zmax, mb, rec);
+    }
+  }
+  for (uint64_t t = gw; t < np; t += nw) {
+    const SpanPiece pc = A.w.pieces[t];
+    const SpanJob q = A.w.jobs[pc.e];
+    const uint32_t x0 = pc.q * kPieceVals, x1 = min(x0 + kPieceVals, q.N);
+    int64_t lo, hi;
+    uint64_t zmax;
+    job_range<32, true>(A.v + q.a, q, x0, x1, lane, q.narrow != 0, lo, hi, zmax);
+    if (lane != 0) continue;
+    atomicMin(&A.w.lo[pc.mi], (long long)lo);
+    atomicMax(&A.w.hi[pc.mi], (long long)hi);
+    atomicMax(&A.w.zmax[pc.mi], (unsigned long long)zmax);
+    __threadfence();
+    if (atomicAdd(&A.w.done[pc.mi], 1u) + 1u < pc.np) continue;  // the last of the pieces has the whole range
+    __threadfence();
+    finish_job(q, *(volatile long long*)&A.w.lo[pc.mi], *(volatile long long*)&A.w.hi[pc.mi],
+               *(volatile unsigned long long*)&A.w.zmax[pc.mi], mb, rec);
+  }
+}
+
+// gain of a pair of widths and lengths that merges at width w
+__device__ __forceinline__ int64_t gain_of(uint64_t N1, uint32_t b1, uint64_t N2, uint32_t b2, uint32_t w) {
+  return (int64_t)(kSmBits + N1 * b1 + N2 * b2) - (int64_t)((N1 + N2) * w);
 }
 
 // priority order of two pairs: gain, then the hash of the start, then the smaller start
@@ -795,70 +1127,285 @@ __device__ __forceinline__ bool beats(int64_t g1, uint64_t s1, int64_t g2, uint6
   return s1 < s2;
 }
 
-// sel[j]: pair j merges this round; keep[p]: partition p survives (it was not merged into its left
-// neighbour); *nsel counts the merging pairs
-__global__ void k_select(const uint64_t* __restrict__ st, const uint64_t* __restrict__ sz,
-                         const uint64_t* __restrict__ msz, uint64_t m, uint8_t* __restrict__ sel,
-                         uint64_t* __restrict__ keep, unsigned long long* __restrict__ nsel) {
+// Dense rounds: tiles of kMergeTile partitions. k_select: bit j of sel is set when pair j merges (it gains
+// and beats both neighbours); the tile's count into cnt.
+constexpr uint32_t kMergeTile = 1024;
+
+__global__ void __launch_bounds__(256)
+    k_select(const uint64_t* __restrict__ st, const uint8_t* __restrict__ b, const uint8_t* __restrict__ mb, uint64_t m,
+             uint32_t* __restrict__ sel, uint64_t* __restrict__ cnt) {
+  // [i] belongs to pair base - 1 + i. A pair's gain fits 32 bits (at most 2^24 values of 64 bits); kLoses:
+  // it does not merge. Gains tie in most pairs of the first rounds, so each pair's hash is taken once too.
+  constexpr int32_t kLoses = INT32_MIN;
+  __shared__ uint64_t s_st[kMergeTile + 2], s_hash[kMergeTile + 2];
+  __shared__ int32_t s_gain[kMergeTile + 2];
+  __shared__ uint32_t ws[8];
+  const uint64_t base = (uint64_t)blockIdx.x * kMergeTile;
+  for (uint32_t i = threadIdx.x; i < kMergeTile + 2; i += 256) {
+    const int64_t p = (int64_t)(base + i) - 1;
+    int32_t g = kLoses;
+    uint64_t a = 0;
+    if (p >= 0 && (uint64_t)p + 1 < m) {
+      const uint32_t w = mb[p];
+      a = st[p];
+      if (w <= 64) {
+        const uint64_t mid = st[p + 1];
+        g = (int32_t)gain_of(mid - a, b[p], st[p + 2] - mid, b[p + 1], w);
+      }
+    }
+    s_gain[i] = g;
+    s_st[i] = a;
+    s_hash[i] = splitmix64(a);
+  }
+  __syncthreads();
   uint32_t local = 0;
-  for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < m; j += (uint64_t)gridDim.x * blockDim.x) {
-    bool ok = false;
-    if (j + 1 < m) {
-      int64_t g;
-      ok = pair_gain(sz, msz, j, &g) && g > 0;
-      if (ok && j > 0) {
-        int64_t gl;
-        if (pair_gain(sz, msz, j - 1, &gl) && !beats(g, st[j], gl, st[j - 1])) ok = false;
-      }
-      if (ok && j + 2 < m) {
-        int64_t gr;
-        if (pair_gain(sz, msz, j + 1, &gr) && !beats(g, st[j], gr, st[j + 1])) ok = false;
-      }
+  for (uint32_t u = threadIdx.x; u < kMergeTile; u += 256) {
+    const uint32_t i = u + 1;
+    const int32_t g = s_gain[i];
+    auto over = [&](uint32_t k) {  // pair i beats pair k
+      if (g != s_gain[k]) return g > s_gain[k];
+      return s_hash[i] != s_hash[k] ? s_hash[i] > s_hash[k] : s_st[i] < s_st[k];
+    };
+    const bool ok = g != kLoses && over(i - 1) && over(i + 1);
+    const uint32_t w = __ballot_sync(kFull, ok);
+    if ((threadIdx.x & 31u) == 0) {
+      sel[(base + u) >> 5] = w;
+      local += (uint32_t)__popc(w);
     }
-    sel[j] = ok ? 1 : 0;
-    local += ok ? 1u : 0u;
-    // partition j + 1 is absorbed when pair j merges; partition 0 always survives
-    if (j + 1 < m) keep[j + 1] = ok ? 0ull : 1ull;
-    if (j == 0) keep[0] = 1ull;
   }
-  local = (uint32_t)warp_sum_u64(local);
-  if ((threadIdx.x & 31u) == 0 && local) atomicAdd(nsel, (unsigned long long)local);
+  if ((threadIdx.x & 31u) == 0) ws[threadIdx.x >> 5] = local;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int k = 1; k < 8; k++) local += ws[k];
+    cnt[blockIdx.x] = local;
+  }
 }
 
-// the next round's arrays; a merged pair's moments are combined. Every load a partition needs is
-// issued before the first branch, so the loads of one thread overlap.
-__global__ void k_compact(const uint64_t* __restrict__ st, const uint64_t* __restrict__ sz,
-                          const uint64_t* __restrict__ msz, const uint8_t* __restrict__ sel,
-                          const uint64_t* __restrict__ newidx, const SpanStats* __restrict__ stats, uint64_t m,
-                          uint64_t n, uint64_t new_m, uint64_t* __restrict__ nst, uint64_t* __restrict__ nsz,
-                          uint64_t* __restrict__ nmsz, uint8_t* __restrict__ ndirty, SpanStats* __restrict__ nstats) {
-  for (uint64_t p = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; p < m;
-       p += (uint64_t)gridDim.x * blockDim.x) {
-    const bool absorbed = p > 0 && sel[p - 1];  // merged into p - 1
-    const bool mp = p + 1 < m && sel[p];
-    const bool mq2 = p + 3 < m && sel[p + 2];  // the next survivor's pair when p merges
-    const bool mq1 = p + 2 < m && sel[p + 1];  // ... when it does not
-    const uint64_t k = newidx[p];
-    const uint64_t s0 = st[p];
-    const uint64_t szp = sz[p];
-    const uint64_t mszp = p + 1 < m ? msz[p] : 0;
-    const uint64_t s1 = p + 1 < m ? st[p + 1] : n;
+// the moments of two partitions [a, mid), [mid, c) that merge, where the result carries them
+template <typename T>
+__device__ __forceinline__ void merge_stats(const T* __restrict__ v, SpanStats* __restrict__ stats, uint64_t a,
+                                            uint64_t mid, uint64_t c) {
+  if (c - a <= kStatVals) return;
+  stats[a / kStatVals] = combine_stats(part_stats(v, a, (uint32_t)(mid - a), stats), mid - a,
+                                       part_stats(v, mid, (uint32_t)(c - mid), stats));
+}
+
+// The next round's partitions. Partition p survives unless pair p - 1 merges; its rank is p less the pairs
+// that merge before pair p - 1.
+template <typename T>
+__global__ void __launch_bounds__(256)
+    k_compact(const T* __restrict__ v, const uint64_t* __restrict__ st, const uint8_t* __restrict__ b,
+              const uint8_t* __restrict__ mb, uint64_t m, const uint32_t* __restrict__ sel,
+              const uint64_t* __restrict__ before, const uint64_t* __restrict__ total, SpanStats* __restrict__ stats,
+              uint64_t* __restrict__ nst, uint8_t* __restrict__ nb, uint8_t* __restrict__ nmb) {
+  __shared__ uint32_t bits[kMergeTile / 32 + 2];  // word i: pairs base - 32 + 32 i ..
+  __shared__ uint32_t pre[kMergeTile / 32];       // pairs of the tile that merge before word i
+  const uint64_t base = (uint64_t)blockIdx.x * kMergeTile, words = (m + 31) / 32;
+  const uint32_t t = threadIdx.x;
+  if (t < kMergeTile / 32 + 2) {
+    const int64_t w = (int64_t)(base >> 5) - 1 + (int64_t)t;
+    bits[t] = w >= 0 && (uint64_t)w < words ? sel[w] : 0u;
+  }
+  __syncthreads();
+  if (t < 32) {
+    const uint32_t c = (uint32_t)__popc(bits[t + 1]);
+    uint32_t inc = c;
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, inc, o);
+      if (t >= o) inc += y;
+    }
+    pre[t] = inc - c;
+  }
+  __syncthreads();
+  auto merges = [&](uint32_t i) -> bool {  // pair base - 32 + i
+    return (bits[i >> 5] >> (i & 31u)) & 1u;
+  };
+  const uint64_t merged = before[blockIdx.x];
+  for (uint32_t u = t; u < kMergeTile; u += 256) {
+    const uint64_t p = base + u;
+    if (p >= m) break;
+    const uint32_t i = u + 32u;
+    const bool absorbed = merges(i - 1u);
     if (absorbed) continue;
-    const SpanStats sp = stats[p];
-    nst[k] = s0;
-    nsz[k] = mp ? mszp : szp;
-    nstats[k] = mp ? combine_stats(sp, s1 - s0, stats[p + 1]) : sp;
-    const uint64_t q = mp ? p + 2 : p + 1;  // next surviving partition
-    if (q < m) {
-      const bool d = mp || (mp ? mq2 : mq1);
-      ndirty[k] = d ? 1 : 0;
-      if (!d) nmsz[k] = mszp;
-    }
-    if (k == 0) nst[new_m] = n;
+    const uint64_t k = p - (merged + pre[u >> 5] + (uint32_t)__popc(bits[i >> 5] & ((1u << (u & 31u)) - 1u)));
+    const bool mp = merges(i);
+    const uint32_t w = mb[p];
+    const uint64_t a = st[p];
+    nst[k] = a;
+    nb[k] = mp ? (uint8_t)w : b[p];
+    // the next survivor is q; the pair of the two is new when either of them is
+    const uint32_t qi = i + (mp ? 2u : 1u);
+    const uint64_t q = p + (mp ? 2 : 1);
+    if (q < m) nmb[k] = mp || merges(qi) ? kDirty : (uint8_t)w;
+    if (mp) merge_stats(v, stats, a, st[p + 1], st[p + 2]);
+    if (p == 0) nst[m - *total] = st[m];
   }
 }
 
+// ------------------------------------------------------------------------------ sparse rounds
+//
+// The partitions keep their slots (the indexes at the switch); left / right link the live ones. A round:
+// k_sparse_select takes the candidate pairs (left partitions whose pair gains; once each, by `seen`),
+// lists the ones that beat both neighbours and keeps the others as candidates; k_sparse_apply merges
+// them; k_sparse_plan fits the pairs that changed (short ones at once, the others through the job list) and
+// adds them to the candidates; k_span_range ends the fits. Every list's length stays on the device, in
+// a counter per round.
+struct Sparse {
+  uint64_t n;
+  const uint64_t* st;
+  uint8_t *b, *mb;
+  uint32_t *left, *right, *seen, *merged;
+  uint32_t* chosen;
+};
+struct SparseRound {
+  unsigned long long cands, chosen, jobs, pieces, slots;
+};
 
+__global__ void k_sparse_init(Sparse S, uint64_t m, uint32_t* __restrict__ cand, SparseRound* __restrict__ r) {
+  for (uint64_t j = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; j < m; j += (uint64_t)gridDim.x * blockDim.x) {
+    S.left[j] = j ? (uint32_t)(j - 1) : kSlotEnd;
+    S.right[j] = j + 1 < m ? (uint32_t)(j + 1) : kSlotEnd;
+    S.seen[j] = 0;
+    S.merged[j] = 0;
+    if (j + 1 == m) S.mb[j] = kNo;
+    if (j + 1 < m && S.mb[j] <= 64) cand[atomicAdd(&r->cands, 1ull)] = (uint32_t)j;
+  }
+}
+
+__device__ __forceinline__ uint64_t slot_end(const Sparse& S, uint32_t j) {
+  const uint32_t r = S.right[j];
+  return r == kSlotEnd ? S.n : S.st[r];
+}
+
+// gain of the pair of slot j and its right neighbour (mb[j] <= 64)
+__device__ __forceinline__ int64_t slot_gain(const Sparse& S, uint32_t j) {
+  const uint32_t r = S.right[j];
+  const uint64_t mid = S.st[r];
+  return gain_of(mid - S.st[j], S.b[j], slot_end(S, r) - mid, S.b[r], S.mb[j]);
+}
+
+__global__ void k_sparse_select(Sparse S, uint32_t round, const uint32_t* __restrict__ cand, SparseRound* __restrict__ r,
+                                uint32_t* __restrict__ next, SparseRound* __restrict__ rn) {
+  const uint64_t nc = r->cands;
+  for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < nc; t += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t j = cand[t];
+    if (S.mb[j] > 64 || atomicExch(&S.seen[j], round) == round) continue;
+    const uint64_t a = S.st[j];
+    const int64_t g = slot_gain(S, j);
+    const uint32_t l = S.left[j], rt = S.right[j];
+    bool ok = l == kSlotEnd || S.mb[l] > 64 || beats(g, a, slot_gain(S, l), S.st[l]);
+    if (ok && S.mb[rt] <= 64) ok = beats(g, a, slot_gain(S, rt), S.st[rt]);
+    if (ok)
+      S.chosen[atomicAdd(&r->chosen, 1ull)] = j;
+    else
+      next[atomicAdd(&rn->cands, 1ull)] = j;
+  }
+}
+
+template <typename T>
+__global__ void k_sparse_apply(Sparse S, const T* __restrict__ v, SpanStats* __restrict__ stats, uint32_t round,
+                               const SparseRound* __restrict__ r) {
+  const uint64_t nc = r->chosen;
+  for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < nc; t += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t j = S.chosen[t], q = S.right[j], qq = S.right[q];
+    merge_stats(v, stats, S.st[j], S.st[q], qq == kSlotEnd ? S.n : S.st[qq]);
+    S.b[j] = S.mb[j];
+    S.right[j] = qq;
+    if (qq != kSlotEnd) S.left[qq] = j;
+    S.mb[q] = kDead;
+    S.merged[j] = round;
+  }
+}
+
+// the two pairs of every partition merged this round (the left one is its left neighbour's own when that
+// merged too)
+template <typename T>
+__global__ void k_sparse_plan(Sparse S, const SpanArgs<T> A, uint32_t round, const SparseRound* __restrict__ r,
+                              uint32_t* __restrict__ next, SparseRound* __restrict__ rn) {
+  const uint64_t nc = 2 * r->chosen;
+  for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < nc; t += (uint64_t)gridDim.x * blockDim.x) {
+    uint32_t j = S.chosen[t >> 1];
+    if (t & 1) {
+      j = S.left[j];
+      if (j == kSlotEnd || S.merged[j] == round) continue;
+    }
+    const uint32_t q = S.right[j];
+    if (q == kSlotEnd) {
+      S.mb[j] = kNo;
+      continue;
+    }
+    const uint64_t a = S.st[j], mid = S.st[q], c = slot_end(S, q);
+    if (c - a > A.cap) {
+      S.mb[j] = kNo;
+      continue;
+    }
+    const uint32_t N = (uint32_t)(c - a);
+    const bool lin = A.model == LECO_MODEL_LINEAR;
+    const SpanStats M = combine_stats(part_stats(A.v, a, (uint32_t)(mid - a), A.stats), mid - a,
+                                      part_stats(A.v, mid, (uint32_t)(c - mid), A.stats));
+    const FitParams P = solve_params(lin ? line_moment(M, N) : (i128)0, M.mx, M.mn, N, lin);
+    const uint32_t bmax = gain_width((uint32_t)(mid - a), S.b[j], (uint32_t)(c - mid), S.b[q]);
+    if (N > kLaneVals && (lin || P.fallback)) {
+      const bool near = narrow_line(P, N) && narrow_ref(M.mn) && narrow_diff(M.mx - M.mn);
+      put_job(A.w, atomicAdd(&A.w.cnt[0], 1ull), a, N, j, P, bmax, near, true);
+    } else {
+      int64_t lo = M.mn, hi = M.mx;
+      uint64_t zmax = 0;
+      if (lin || P.fallback) {
+        lo = INT64_MAX;
+        hi = INT64_MIN;
+        resid_part(A.v + a, 0, N, 1, P, lo, hi, zmax);
+      }
+      const uint32_t w = finish_width(P, lo, hi, zmax);
+      S.mb[j] = w <= bmax ? (uint8_t)w : kNo;
+    }
+    next[atomicAdd(&rn->cands, 1ull)] = j;
+  }
+}
+
+// live slots as bits, and their number per tile; then the surviving starts side by side
+__global__ void __launch_bounds__(256) k_live(const uint8_t* __restrict__ mb, uint64_t m, uint32_t* __restrict__ live,
+                                              uint64_t* __restrict__ cnt) {
+  __shared__ uint32_t total;
+  if (threadIdx.x == 0) total = 0;
+  __syncthreads();
+  const uint64_t base = (uint64_t)blockIdx.x * kMergeTile;
+  for (uint32_t u = threadIdx.x; u < kMergeTile; u += 256) {
+    const uint64_t p = base + u;
+    const uint32_t w = __ballot_sync(kFull, p < m && mb[p] != kDead);
+    if ((threadIdx.x & 31u) == 0) {
+      live[p >> 5] = w;
+      atomicAdd(&total, (uint32_t)__popc(w));
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) cnt[blockIdx.x] = total;
+}
+
+__global__ void __launch_bounds__(256)
+    k_gather_live(const uint64_t* __restrict__ st, uint64_t m, uint64_t n, const uint32_t* __restrict__ live,
+                  const uint64_t* __restrict__ before, const uint64_t* __restrict__ total, uint64_t* __restrict__ nst) {
+  __shared__ uint32_t pre[kMergeTile / 32];
+  const uint64_t base = (uint64_t)blockIdx.x * kMergeTile;
+  const uint32_t t = threadIdx.x;
+  if (t < 32) {
+    const uint32_t c = (uint32_t)__popc(live[(base >> 5) + t]);
+    uint32_t inc = c;
+    for (uint32_t o = 1; o < 32; o <<= 1) {
+      const uint32_t y = __shfl_up_sync(kFull, inc, o);
+      if (t >= o) inc += y;
+    }
+    pre[t] = inc - c;
+  }
+  __syncthreads();
+  for (uint32_t u = t; u < kMergeTile; u += 256) {
+    const uint64_t p = base + u;
+    if (p >= m) break;
+    const uint32_t w = live[p >> 5];
+    if ((w >> (u & 31u)) & 1u) nst[before[blockIdx.x] + pre[u >> 5] + (uint32_t)__popc(w & ((1u << (u & 31u)) - 1u))] = st[p];
+    if (p == 0) nst[*total] = n;
+  }
+}
 
 template <typename T>
 cudaError_t dalloc(T** p, uint64_t elems, cudaStream_t st) {
@@ -878,36 +1425,177 @@ cudaError_t launch_split(const T* v, uint64_t n, uint64_t nchunks, uint32_t cap,
   return cudaGetLastError();
 }
 
-int group_grid(uint64_t count) {
-  const uint64_t groups = (count + 31) / 32;
-  return grid_for((groups + kGroupBlock / 32 - 1) / (kGroupBlock / 32), 1, 3);
-}
+// one allocation handed out in 256-byte steps: sized by a first pass over the same calls with no base
+struct Arena {
+  char* base = nullptr;
+  uint64_t used = 0;
+  template <typename U>
+  U* take(uint64_t elems) {
+    U* p = base ? reinterpret_cast<U*>(base + used) : nullptr;
+    used += (elems * sizeof(U) + 255) & ~255ull;
+    return p;
+  }
+};
 
-// one mode of k_span_groups over count spans, then (modes 2 and 3) the pieces of the long ones
+constexpr uint32_t kSparseRounds = 6;  // sparse rounds between two looks at the count of merges
+
+// the merge from the split's m partitions in starts_out: rounds until none merges; m starts (and n) in
+// starts_out, and the records of their fits when rec_out is given
 template <typename T>
-cudaError_t span_groups(const void* values, int mode, const uint64_t* st, uint64_t count, uint32_t cap, int model,
-                        const uint8_t* dirty, SpanStats* stats, uint64_t* size_out, Record* rec, const MergeWork& mw,
-                        cudaStream_t s) {
-  if (count == 0) return cudaSuccess;
-  const T* v = static_cast<const T*>(values);
-  if (mode != 1) {
-    const cudaError_t e = cudaMemsetAsync(mw.counters, 0, 2 * sizeof(unsigned long long), s);
-    if (e != cudaSuccess) return e;
+cudaError_t merge_rounds(const T* v, uint64_t n, uint32_t cap, int model, uint64_t* starts_out, uint64_t m,
+                         uint64_t* m_out, Record** rec_out, cudaStream_t s) {
+  const uint64_t tiles = (m + kMergeTile - 1) / kMergeTile, spans = 2 * n / kPieceVals + 2;
+  SpanArgs<T> A;
+  A.v = v;
+  A.cap = cap;
+  A.model = model;
+  uint64_t *st_b, *cnt, *before, *scan, *total;
+  uint8_t *b_a, *b_b, *mb_a, *mb_b;
+  uint32_t* sel;
+  auto layout = [&](Arena& ar) {
+    A.stats = ar.take<SpanStats>(n / kStatVals + 1);
+    st_b = ar.take<uint64_t>(m + 1);
+    b_a = ar.take<uint8_t>(m);
+    b_b = ar.take<uint8_t>(m);
+    mb_a = ar.take<uint8_t>(m);
+    mb_b = ar.take<uint8_t>(m);
+    sel = ar.take<uint32_t>(tiles * (kMergeTile / 32));
+    cnt = ar.take<uint64_t>(tiles);
+    before = ar.take<uint64_t>(tiles);
+    scan = ar.take<uint64_t>(tiles / 2048 + 3);
+    total = ar.take<uint64_t>(1);
+    A.w.jobs = ar.take<SpanJob>(2 * n / kLaneVals + 2);  // spans beyond kLaneVals in pairs cover n twice at most
+    A.w.pieces = ar.take<SpanPiece>(2 * spans);
+    A.w.lo = ar.take<long long>(spans);
+    A.w.hi = ar.take<long long>(spans);
+    A.w.zmax = ar.take<unsigned long long>(spans);
+    A.w.done = ar.take<uint32_t>(spans);
+    A.w.cnt = ar.take<unsigned long long>(3);
+  };
+  Arena ar;
+  layout(ar);
+  cudaError_t e = dev_alloc((void**)&ar.base, ar.used, s);
+  if (e != cudaSuccess) return e;
+  ar.used = 0;
+  layout(ar);
+  char *arena = ar.base, *sparse_arena = nullptr;
+  const int wide = sm_count() * 8;
+  auto span_grid = [&](uint64_t count) { return grid_for((count + 31) / 32, kSpanBlock / 32, 8); };
+  auto clear = [&]() { return cudaMemsetAsync(A.w.cnt, 0, 3 * sizeof(unsigned long long), s); };
+  uint64_t *cur = starts_out, *nxt = st_b;
+  e = clear();
+  if (e == cudaSuccess) {
+    k_fit_spans<T, 1><<<span_grid(m), kSpanBlock, 0, s>>>(A, cur, m, b_a, nullptr, nullptr);
+    k_fit_long<T><<<wide, 256, 0, s>>>(A, b_a);
+    k_fit_longest<T><<<sm_count() * 2, 256, 0, s>>>(A, b_a);
+    e = cudaMemsetAsync(mb_a, kDirty, m, s);
   }
-  if (mode == 1)
-    k_span_groups<T, 1><<<group_grid(count), kGroupBlock, 0, s>>>(v, st, count, cap, model, dirty, stats, size_out,
-                                                                  rec, mw);
-  else if (mode == 2)
-    k_span_groups<T, 2><<<group_grid(count), kGroupBlock, 0, s>>>(v, st, count, cap, model, dirty, stats, size_out,
-                                                                  rec, mw);
-  else
-    k_span_groups<T, 3><<<group_grid(count), kGroupBlock, 0, s>>>(v, st, count, cap, model, dirty, stats, size_out,
-                                                                  rec, mw);
-  if (mode != 1) {
-    k_pair_pieces<T><<<sm_count() * 8, 256, 0, s>>>(v, mw);
-    k_pair_finish<<<sm_count() * 2, 256, 0, s>>>(mw, size_out, mode == 3 ? rec : nullptr);
+  bool sparse = false;
+  while (e == cudaSuccess && m > 1) {
+    e = clear();
+    if (e != cudaSuccess) break;
+    k_fit_spans<T, 2><<<span_grid(m - 1), kSpanBlock, 0, s>>>(A, cur, m - 1, b_a, mb_a, nullptr);
+    k_span_range<T><<<wide, 256, 0, s>>>(A, mb_a, nullptr);
+    e = cudaGetLastError();
+    sparse = sparse || m <= kSparseBelow;
+    if (e != cudaSuccess || sparse) break;
+    const uint64_t nt = (m + kMergeTile - 1) / kMergeTile;
+    k_select<<<(unsigned)nt, 256, 0, s>>>(cur, b_a, mb_a, m, sel, cnt);
+    e = scan_u64(cnt, nt, before, scan, total, s);
+    uint64_t merges = 0;
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&merges, total, 8, cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    if (e != cudaSuccess || merges == 0) break;
+    k_compact<T><<<(unsigned)nt, 256, 0, s>>>(v, cur, b_a, mb_a, m, sel, before, total, A.stats, nxt, b_b, mb_b);
+    e = cudaGetLastError();
+    std::swap(cur, nxt);
+    std::swap(b_a, b_b);
+    std::swap(mb_a, mb_b);
+    sparse = merges * kSparseShare < m && m < kSlotEnd;
+    m -= merges;
   }
-  return cudaGetLastError();
+  if (e == cudaSuccess && sparse) {
+    Sparse S;
+    S.n = n;
+    S.st = cur;
+    S.b = b_a;
+    S.mb = mb_a;
+    uint32_t *cand[2];
+    SparseRound* rounds[2];
+    auto slots = [&](Arena& a2) {
+      S.left = a2.take<uint32_t>(m);
+      S.right = a2.take<uint32_t>(m);
+      S.seen = a2.take<uint32_t>(m);
+      S.merged = a2.take<uint32_t>(m);
+      S.chosen = a2.take<uint32_t>(m);
+      cand[0] = a2.take<uint32_t>(2 * m);  // a slot enters at most once from each of two kernels
+      cand[1] = a2.take<uint32_t>(2 * m);
+      rounds[0] = a2.take<SparseRound>(kSparseRounds + 1);
+      rounds[1] = a2.take<SparseRound>(kSparseRounds + 1);
+    };
+    Arena a2;
+    slots(a2);
+    e = dev_alloc((void**)&a2.base, a2.used, s);
+    a2.used = 0;
+    slots(a2);
+    sparse_arena = a2.base;
+    const uint64_t round_bytes = sizeof(SparseRound) * (kSparseRounds + 1);
+    const int grid = grid_for(m, 256, 2);
+    if (e == cudaSuccess) e = cudaMemsetAsync(rounds[0], 0, round_bytes, s);
+    if (e == cudaSuccess) k_sparse_init<<<grid_for(m, 256, 8), 256, 0, s>>>(S, m, cand[0], rounds[0]);
+    uint32_t round = 1;
+    int side = 0;
+    for (unsigned long long merges = 1; e == cudaSuccess && merges; side ^= 1) {
+      SparseRound* r = rounds[side];
+      for (uint32_t k = 0; k < kSparseRounds; k++, round++) {
+        uint32_t *c = cand[round & 1u ? 0 : 1], *next = cand[round & 1u ? 1 : 0];
+        SpanArgs<T> B = A;
+        B.w.cnt = &r[k].jobs;
+        k_sparse_select<<<grid, 256, 0, s>>>(S, round, c, r + k, next, r + k + 1);
+        k_sparse_apply<T><<<grid, 256, 0, s>>>(S, v, A.stats, round, r + k);
+        k_sparse_plan<T><<<grid, 256, 0, s>>>(S, B, round, r + k, next, r + k + 1);
+        k_span_range<T><<<sm_count() * 4, 256, 0, s>>>(B, S.mb, nullptr);
+      }
+      e = cudaGetLastError();
+      if (e == cudaSuccess) e = cudaMemcpyAsync(&merges, &r[kSparseRounds - 1].chosen, 8, cudaMemcpyDeviceToHost, s);
+      SparseRound* rn = rounds[side ^ 1];
+      if (e == cudaSuccess) e = cudaMemsetAsync(rn, 0, round_bytes, s);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(&rn->cands, &r[kSparseRounds].cands, 8, cudaMemcpyDeviceToDevice, s);
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    }
+    if (e == cudaSuccess) {  // the live slots' starts side by side
+      const uint64_t nt = (m + kMergeTile - 1) / kMergeTile;
+      k_live<<<(unsigned)nt, 256, 0, s>>>(mb_a, m, sel, cnt);
+      e = scan_u64(cnt, nt, before, scan, total, s);
+      if (e == cudaSuccess) {
+        k_gather_live<<<(unsigned)nt, 256, 0, s>>>(cur, m, n, sel, before, total, nxt);
+        e = cudaMemcpyAsync(&m, total, 8, cudaMemcpyDeviceToHost, s);
+      }
+      if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+      std::swap(cur, nxt);
+    }
+  }
+  if (e == cudaSuccess && rec_out) {
+    e = dalloc(rec_out, m, s);  // the final partitions' fits
+    if (e == cudaSuccess) e = clear();
+    if (e == cudaSuccess) {
+      k_fit_spans<T, 3><<<span_grid(m), kSpanBlock, 0, s>>>(A, cur, m, nullptr, nullptr, *rec_out);
+      k_span_range<T><<<wide, 256, 0, s>>>(A, nullptr, *rec_out);
+      e = cudaGetLastError();
+    }
+  }
+  if (e == cudaSuccess && cur != starts_out)
+    e = cudaMemcpyAsync(starts_out, cur, (m + 1) * 8, cudaMemcpyDeviceToDevice, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  cudaFreeAsync(arena, s);
+  if (sparse_arena) cudaFreeAsync(sparse_arena, s);
+  if (e != cudaSuccess && rec_out && *rec_out) {
+    cudaFreeAsync(*rec_out, s);
+    *rec_out = nullptr;
+  }
+  if (e == cudaSuccess) *m_out = m;
+  return e;
 }
 
 }  // namespace
@@ -1060,95 +1748,8 @@ cudaError_t var_partition_fit(const void* values, int dtype, uint64_t n, double 
   }
   if (e != cudaSuccess) return e;
 
-  // merge state
-  const uint64_t m0 = m;
-  SpanStats *stats = nullptr, *stats_b = nullptr;
-  uint64_t *st_b = nullptr, *sz_a = nullptr, *sz_b = nullptr;
-  uint64_t *msz_a = nullptr, *msz_b = nullptr, *keep = nullptr, *newidx = nullptr, *scr = nullptr, *d_total = nullptr;
-  uint8_t *dirty_a = nullptr, *dirty_b = nullptr, *sel = nullptr;
-  unsigned long long* d_nsel = nullptr;
-  MergeWork mw;
-  mw.longs = nullptr;
-  mw.pieces = nullptr;
-  mw.counters = nullptr;
-  mw.lo = nullptr;
-  mw.hi = nullptr;
-  mw.zmax = nullptr;
-  const uint64_t long_cap = 2 * n / kWarpSpan + 2;
-  const uint64_t piece_cap = 2 * n / kPiece + long_cap + 2;
-  const uint64_t scr_elems = m0 / 2048 + 2;
-  if (e == cudaSuccess) e = dalloc(&stats, m0, st);
-  if (e == cudaSuccess) e = dalloc(&stats_b, m0, st);
-  if (e == cudaSuccess) e = dalloc(&st_b, m0 + 1, st);
-  if (e == cudaSuccess) e = dalloc(&sz_a, m0, st);
-  if (e == cudaSuccess) e = dalloc(&sz_b, m0, st);
-  if (e == cudaSuccess) e = dalloc(&msz_a, m0, st);
-  if (e == cudaSuccess) e = dalloc(&msz_b, m0, st);
-  if (e == cudaSuccess) e = dalloc(&keep, m0, st);
-  if (e == cudaSuccess) e = dalloc(&newidx, m0, st);
-  if (e == cudaSuccess) e = dalloc(&scr, scr_elems + 1, st);
-  if (e == cudaSuccess) e = dalloc(&d_total, 1, st);
-  if (e == cudaSuccess) e = dalloc(&dirty_a, m0, st);
-  if (e == cudaSuccess) e = dalloc(&dirty_b, m0, st);
-  if (e == cudaSuccess) e = dalloc(&sel, m0, st);
-  if (e == cudaSuccess) e = dalloc(&d_nsel, 1, st);
-  if (e == cudaSuccess) e = dalloc(&mw.longs, long_cap, st);
-  if (e == cudaSuccess) e = dalloc(&mw.pieces, piece_cap, st);
-  if (e == cudaSuccess) e = dalloc(&mw.counters, 2, st);
-  if (e == cudaSuccess) e = dalloc(&mw.lo, long_cap, st);
-  if (e == cudaSuccess) e = dalloc(&mw.hi, long_cap, st);
-  if (e == cudaSuccess) e = dalloc(&mw.zmax, long_cap, st);
-  uint64_t* cur_st = starts_out;
-  uint64_t* nxt_st = st_b;
-  // every split partition's moments, fit and size
-  if (e == cudaSuccess)
-    e = u32 ? span_groups<uint32_t>(values, 1, cur_st, m, cap, model, nullptr, stats, sz_a, nullptr, mw, st)
-            : span_groups<uint64_t>(values, 1, cur_st, m, cap, model, nullptr, stats, sz_a, nullptr, mw, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(dirty_a, 1, m, st);
-  while (e == cudaSuccess && m > 1) {
-    e = u32 ? span_groups<uint32_t>(values, 2, cur_st, m - 1, cap, model, dirty_a, stats, msz_a, nullptr, mw, st)
-            : span_groups<uint64_t>(values, 2, cur_st, m - 1, cap, model, dirty_a, stats, msz_a, nullptr, mw, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d_nsel, 0, 8, st);
-    if (e != cudaSuccess) break;
-    k_select<<<grid_for(m, 256, 8), 256, 0, st>>>(cur_st, sz_a, msz_a, m, sel, keep, d_nsel);
-    unsigned long long nsel = 0;
-    e = cudaMemcpyAsync(&nsel, d_nsel, 8, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess || nsel == 0) break;
-    e = scan_u64(keep, m, newidx, scr, d_total, st);
-    if (e != cudaSuccess) break;
-    const uint64_t new_m = m - nsel;
-    k_compact<<<grid_for(m, 256, 8), 256, 0, st>>>(cur_st, sz_a, msz_a, sel, newidx, stats, m, n, new_m, nxt_st,
-                                                   sz_b, msz_b, dirty_b, stats_b);
-    e = cudaGetLastError();
-    std::swap(cur_st, nxt_st);
-    std::swap(sz_a, sz_b);
-    std::swap(msz_a, msz_b);
-    std::swap(dirty_a, dirty_b);
-    std::swap(stats, stats_b);
-    m = new_m;
-  }
-  if (e == cudaSuccess && rec_out) {
-    e = dalloc(rec_out, m, st);  // the final partitions' fits from their moments
-    if (e == cudaSuccess)
-      e = u32 ? span_groups<uint32_t>(values, 3, cur_st, m, cap, model, nullptr, stats, nullptr, *rec_out, mw, st)
-              : span_groups<uint64_t>(values, 3, cur_st, m, cap, model, nullptr, stats, nullptr, *rec_out, mw, st);
-  }
-  if (e == cudaSuccess && cur_st != starts_out)
-    e = cudaMemcpyAsync(starts_out, cur_st, (m + 1) * 8, cudaMemcpyDeviceToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  cudaFreeAsync(cur_st == starts_out ? nxt_st : cur_st, st);  // st_b, wherever it ended up
-  for (void* p : {(void*)stats, (void*)stats_b, (void*)sz_a,
-                  (void*)sz_b, (void*)msz_a, (void*)msz_b, (void*)keep, (void*)newidx, (void*)scr, (void*)d_total,
-                  (void*)dirty_a, (void*)dirty_b, (void*)sel, (void*)d_nsel, (void*)mw.longs, (void*)mw.pieces,
-                  (void*)mw.counters, (void*)mw.lo, (void*)mw.hi, (void*)mw.zmax})
-    if (p) cudaFreeAsync(p, st);
-  if (e != cudaSuccess && rec_out && *rec_out) {
-    cudaFreeAsync(*rec_out, st);
-    *rec_out = nullptr;
-  }
-  if (e == cudaSuccess) *m_out = m;
-  return e;
+  return u32 ? merge_rounds(static_cast<const uint32_t*>(values), n, cap, model, starts_out, m, m_out, rec_out, st)
+             : merge_rounds(static_cast<const uint64_t*>(values), n, cap, model, starts_out, m, m_out, rec_out, st);
 }
 
 cudaError_t var_partition(const void* values, int dtype, uint64_t n, double tau, uint32_t cap, int model, bool seeded,

@@ -1,5 +1,5 @@
 // Span fits of the variable partitioner (§3.1 Regressor over the spans of §3.2.2): the moments of a
-// span's values and the cooperative passes that let several lanes work on one span.
+// span's values by one thread or a group, and the residual range under a span's line.
 //
 // Moments of a span (w = the value as two's complement int64, x = the local index): T0 = sum w,
 // T1 = sum x w, and min and max of w. The fit's least-squares moment is S = sum (2x - (N-1)) w =
@@ -31,57 +31,132 @@ __device__ __forceinline__ SpanStats combine_stats(const SpanStats& l, uint64_t 
   return c;
 }
 
-// reductions over aligned tiles of TILE lanes (32: the warp) whose result every lane of the tile
-// receives
-template <int TILE = 32>
-__device__ __forceinline__ int64_t xw_min(int64_t v) {
+// the fit's least-squares moment of a span of N values
+__device__ __forceinline__ i128 line_moment(const SpanStats& s, uint32_t N) {
+  return 2 * s.T1 - mul_i128_u64(s.T0, N - 1);
+}
+
+// minimum, maximum and sum over aligned tiles of TILE lanes (32: the warp), in every lane
+template <int TILE>
+__device__ __forceinline__ int32_t tile_min(int32_t v) {
+  if constexpr (TILE == 32) {
+    v = __reduce_min_sync(kFull, v);
+  } else {
+    for (int o = TILE / 2; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(kFull, v, o));
+  }
+  return v;
+}
+template <int TILE>
+__device__ __forceinline__ int32_t tile_max(int32_t v) {
+  if constexpr (TILE == 32) {
+    v = __reduce_max_sync(kFull, v);
+  } else {
+    for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(kFull, v, o));
+  }
+  return v;
+}
+template <int TILE>
+__device__ __forceinline__ int64_t tile_min(int64_t v) {
   for (int o = TILE / 2; o > 0; o >>= 1) v = min(v, (int64_t)__shfl_xor_sync(kFull, v, o));
   return v;
 }
-template <int TILE = 32>
-__device__ __forceinline__ int64_t xw_max(int64_t v) {
+template <int TILE>
+__device__ __forceinline__ int64_t tile_max(int64_t v) {
   for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, (int64_t)__shfl_xor_sync(kFull, v, o));
   return v;
 }
-__device__ __forceinline__ uint64_t xw_min_u(uint64_t v) {
-  for (int o = 16; o > 0; o >>= 1) v = min(v, (uint64_t)__shfl_xor_sync(kFull, v, o));
-  return v;
-}
-template <int TILE = 32>
-__device__ __forceinline__ uint64_t xw_max_u(uint64_t v) {
+template <int TILE>
+__device__ __forceinline__ uint64_t tile_max(uint64_t v) {
   for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, (uint64_t)__shfl_xor_sync(kFull, v, o));
   return v;
 }
-template <int TILE = 32>
-__device__ __forceinline__ i128 xw_sum(i128 v) {
-  uint64_t lo = (uint64_t)v, hi = (uint64_t)((u128)v >> 64);
-  for (int o = TILE / 2; o > 0; o >>= 1) {
-    const uint64_t l2 = __shfl_xor_sync(kFull, lo, o);
-    const uint64_t h2 = __shfl_xor_sync(kFull, hi, o);
-    const uint64_t nl = lo + l2;
-    hi = hi + h2 + (nl < lo ? 1ull : 0ull);
-    lo = nl;
-  }
-  return (i128)(((u128)hi << 64) | lo);
+template <int TILE>
+__device__ __forceinline__ int64_t tile_sum(int64_t v) {
+  for (int o = TILE / 2; o > 0; o >>= 1) v += (int64_t)__shfl_xor_sync(kFull, v, o);
+  return v;
 }
 
-// moments of the positions x, x + step, ... < N of the span whose first value is p[0]
-template <typename T>
-__device__ __forceinline__ SpanStats stats_part(const T* p, uint32_t x, uint32_t N, uint32_t step) {
-  SpanStats s;
-  s.T0 = 0;
-  s.T1 = 0;
-  s.mn = INT64_MAX;
-  s.mx = INT64_MIN;
-#pragma unroll 8
-  for (; x < N; x += step) {
-    const int64_t w = (int64_t)p[x];
-    s.mn = min(s.mn, w);
-    s.mx = max(s.mx, w);
-    s.T0 += (i128)w;
-    s.T1 += mul_s64(w, (int64_t)x);
+// Narrow spans: values within 2^30 of a reference in (-2^62, 2^62), so that their differences d from it fit
+// 32 bits (a difference that wraps in 64 bits is above 2^61 in magnitude, so the test sees it), and a line
+// that stays within 2^30 over the span. Extremes are then 32-bit, products 32 x 32 -> 64-bit, and the line
+// needs no 64-bit shift: G = B x 2^(32-s) (or B x, for s > 32) is carried and its high half read.
+constexpr int64_t kNarrow = (int64_t)1 << 30;
+constexpr int64_t kNarrowRef = (int64_t)1 << 62;
+__device__ __forceinline__ bool narrow_ref(int64_t ref) { return ref > -kNarrowRef && ref < kNarrowRef; }
+__device__ __forceinline__ bool narrow_diff(int64_t d) { return d > -kNarrow && d < kNarrow; }
+__device__ __forceinline__ bool narrow_line(const FitParams& P, uint32_t N) {
+  return !P.fallback && P.s >= 0 && ((uint64_t)(P.B < 0 ? -P.B : P.B) * (N - 1)) >> P.s < (uint64_t)kNarrow;
+}
+struct NarrowLine {
+  uint64_t B;
+  uint32_t sh;
+  __device__ __forceinline__ NarrowLine(int64_t slope, int s)
+      : B((uint64_t)slope << (s < 32 ? 32 - s : 0)), sh(s > 32 ? (uint32_t)(s - 32) : 0u) {}
+  __device__ __forceinline__ int32_t at(uint64_t G) const { return (int32_t)(G >> 32) >> sh; }
+};
+
+// Sums of w and x w as high and low halves of w (the high half signed), each below 2^62 in magnitude
+// while a thread adds at most 2^11 values at positions x < 2^17.
+struct HalfSums {
+  int64_t h0 = 0, l0 = 0, h1 = 0, l1 = 0;
+  int64_t mn = INT64_MAX, mx = INT64_MIN;
+  template <typename T>
+  __device__ __forceinline__ void add(T value, uint32_t x) {
+    const int64_t w = (int64_t)value;
+    mn = min(mn, w);
+    mx = max(mx, w);
+    l0 += (int64_t)(uint32_t)w;
+    l1 += (int64_t)((uint64_t)(uint32_t)w * x);
+    if (sizeof(T) == 8) {
+      h0 += (int64_t)(int32_t)(w >> 32);
+      h1 += (int64_t)(int32_t)(w >> 32) * (int64_t)x;
+    }
   }
+  __device__ __forceinline__ SpanStats stats() const {
+    SpanStats s;
+    s.T0 = (i128)h0 * ((i128)1 << 32) + (i128)l0;
+    s.T1 = (i128)h1 * ((i128)1 << 32) + (i128)l1;
+    s.mn = mn;
+    s.mx = mx;
+    return s;
+  }
+};
+
+// a span's moments from those of its differences from ref: Sd = sum d and its least-squares moment S
+__device__ __forceinline__ SpanStats stats_from(int64_t ref, uint32_t N, int64_t Sd, int64_t S, int32_t mn, int32_t mx) {
+  SpanStats s;
+  s.T0 = mul_s64(ref, (int64_t)N) + (i128)Sd;
+  s.T1 = ((i128)S + mul_i128_u64(s.T0, N - 1)) >> 1;  // S = 2 T1 - (N - 1) T0
+  s.mn = ref + mn;
+  s.mx = ref + mx;
   return s;
+}
+
+// moments of a short span by one thread
+template <typename T>
+__device__ __forceinline__ SpanStats lane_stats(const T* p, uint32_t N) {
+  HalfSums h;
+#pragma unroll 4
+  for (uint32_t x = 0; x < N; x++) h.add(p[x], x);
+  return h.stats();
+}
+
+// moments of the positions rank, rank + step, ... of a span of up to 2^16 values, summed over the tile
+// (every lane has the sum)
+template <int TILE, typename T>
+__device__ __forceinline__ SpanStats group_stats(const T* p, uint32_t rank, uint32_t N, uint32_t step) {
+  HalfSums h;
+#pragma unroll 8
+  for (uint32_t x = rank; x < N; x += step) h.add(p[x], x);
+  h.l0 = tile_sum<TILE>(h.l0);
+  h.l1 = tile_sum<TILE>(h.l1);
+  if (sizeof(T) == 8) {
+    h.h0 = tile_sum<TILE>(h.h0);
+    h.h1 = tile_sum<TILE>(h.h1);
+  }
+  h.mn = tile_min<TILE>(h.mn);
+  h.mx = tile_max<TILE>(h.mx);
+  return h.stats();
 }
 
 // residual range at the positions x, x + step, ... < N under the parameters P (fit.cuh, steps 4
@@ -112,87 +187,6 @@ __device__ __forceinline__ void resid_part(const T* p, uint32_t x, uint32_t N, u
     }
   }
 }
-
-__device__ __forceinline__ FitParams shfl_params(const FitParams& P, int src) {
-  FitParams q;
-  q.B = (int64_t)__shfl_sync(kFull, (unsigned long long)P.B, src);
-  q.fb_shift = (int64_t)__shfl_sync(kFull, (unsigned long long)P.fb_shift, src);
-  q.s = __shfl_sync(kFull, P.s, src);
-  q.fallback = __shfl_sync(kFull, P.fallback, src);
-  return q;
-}
-
-// Spans fitted cooperatively: the spans of the lanes set in mask, TILE lanes each (32 / TILE spans
-// at a time, in the order of their lanes). Each call hands every owning lane the reduced result of
-// its own span. p, N, P: the calling lane's span (a pointer to its first value, in global or shared
-// memory, its length and its parameters).
-template <int TILE, typename T>
-__device__ __forceinline__ void coop_stats(uint32_t mask, const T* p, uint32_t N, SpanStats& S) {
-  constexpr int NT = 32 / TILE;
-  const int lane = (int)(threadIdx.x & 31u), tile = lane / TILE, r = lane % TILE;
-  const int total = __popc(mask);
-  const bool mine = (mask >> lane) & 1u;
-  const int rank = __popc(mask & ((1u << lane) - 1u));
-  for (int it = 0; it * NT < total; it++) {
-    const int k = it * NT + tile;
-    const int sl = k < total ? (int)__fns(mask, 0, k + 1) : lane;
-    const T* ps = reinterpret_cast<const T*>(__shfl_sync(kFull, (unsigned long long)p, sl));
-    const uint32_t Ns = __shfl_sync(kFull, N, sl);
-    SpanStats q = stats_part(ps, (uint32_t)r, k < total ? Ns : 0u, (uint32_t)TILE);
-    q.T0 = xw_sum<TILE>(q.T0);
-    q.T1 = xw_sum<TILE>(q.T1);
-    q.mn = xw_min<TILE>(q.mn);
-    q.mx = xw_max<TILE>(q.mx);
-    const bool take = mine && rank / NT == it;
-    const int src = take ? (rank % NT) * TILE : lane;
-    const uint64_t t0l = __shfl_sync(kFull, (uint64_t)q.T0, src), t0h = __shfl_sync(kFull, (uint64_t)((u128)q.T0 >> 64), src);
-    const uint64_t t1l = __shfl_sync(kFull, (uint64_t)q.T1, src), t1h = __shfl_sync(kFull, (uint64_t)((u128)q.T1 >> 64), src);
-    const int64_t mn = __shfl_sync(kFull, q.mn, src), mx = __shfl_sync(kFull, q.mx, src);
-    if (take) {
-      S.T0 = (i128)(((u128)t0h << 64) | t0l);
-      S.T1 = (i128)(((u128)t1h << 64) | t1l);
-      S.mn = mn;
-      S.mx = mx;
-    }
-  }
-}
-
-template <int TILE, typename T>
-__device__ __forceinline__ void coop_resid(uint32_t mask, const T* p, uint32_t N, const FitParams& P, int64_t& lo,
-                                           int64_t& hi, uint64_t& zmax) {
-  constexpr int NT = 32 / TILE;
-  const int lane = (int)(threadIdx.x & 31u), tile = lane / TILE, r = lane % TILE;
-  const int total = __popc(mask);
-  const bool mine = (mask >> lane) & 1u;
-  const int rank = __popc(mask & ((1u << lane) - 1u));
-  for (int it = 0; it * NT < total; it++) {
-    const int k = it * NT + tile;
-    const int sl = k < total ? (int)__fns(mask, 0, k + 1) : lane;
-    const T* ps = reinterpret_cast<const T*>(__shfl_sync(kFull, (unsigned long long)p, sl));
-    const uint32_t Ns = __shfl_sync(kFull, N, sl);
-    const FitParams Ps = shfl_params(P, sl);
-    int64_t l = INT64_MAX, h = INT64_MIN;
-    uint64_t z = 0;
-    resid_part(ps, (uint32_t)r, k < total ? Ns : 0u, (uint32_t)TILE, Ps, l, h, z);
-    l = xw_min<TILE>(l);
-    h = xw_max<TILE>(h);
-    z = xw_max_u<TILE>(z);
-    const bool take = mine && rank / NT == it;
-    const int src = take ? (rank % NT) * TILE : lane;
-    l = __shfl_sync(kFull, l, src);
-    h = __shfl_sync(kFull, h, src);
-    z = __shfl_sync(kFull, z, src);
-    if (take) {
-      lo = l;
-      hi = h;
-      zmax = z;
-    }
-  }
-}
-
-
-constexpr uint32_t kLaneSpan = 64;     // a lane fits spans up to this long on its own
-constexpr uint32_t kTileSpan = 1024;   // eight lanes fit longer spans up to this long, four at a time
 
 }  // namespace
 }  // namespace leco
