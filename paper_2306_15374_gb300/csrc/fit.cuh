@@ -93,7 +93,8 @@ struct FitParams {
   int64_t B;
   int64_t fb_shift;  // fallback: theta0 as an integer (multiple of 2^11)
   int32_t s;
-  int32_t fallback;
+  int16_t fallback;
+  int16_t narrow;    // fit_range: the second pass fits 32 bits
 };
 
 struct FitResult {
@@ -171,6 +172,7 @@ __host__ __device__ __forceinline__ FitParams fallback_params(int64_t mx, int64_
   P.s = -11;
   P.B = 0;
   P.fb_shift = (t >> 11) * 2048;
+  P.narrow = 0;
   return P;
 }
 
@@ -261,6 +263,7 @@ __host__ __device__ FitParams solve_params(i128 S, int64_t mx, int64_t mn, uint3
   P.s = s;
   P.B = B;
   P.fb_shift = 0;
+  P.narrow = 0;
   return P;
 }
 
@@ -300,6 +303,25 @@ __device__ FitResult finish_fit(const FitParams& P, int64_t lo, int64_t hi, uint
 }
 
 
+// Narrow spans: values within 2^30 of a reference in (-2^62, 2^62), so that their differences d from it fit
+// 32 bits (a difference that wraps in 64 bits is above 2^61 in magnitude, so the test sees it), and a line
+// that stays within 2^30 over the span. Extremes are then 32-bit, products 32 x 32 -> 64-bit, and the line
+// needs no 64-bit shift: G = B x 2^(32-s) (or B x, for s > 32) is carried and its high half read.
+constexpr int64_t kNarrow = (int64_t)1 << 30;
+constexpr int64_t kNarrowRef = (int64_t)1 << 62;
+__device__ __forceinline__ bool narrow_ref(int64_t ref) { return ref > -kNarrowRef && ref < kNarrowRef; }
+__device__ __forceinline__ bool narrow_diff(int64_t d) { return d > -kNarrow && d < kNarrow; }
+__device__ __forceinline__ bool narrow_line(const FitParams& P, uint32_t N) {
+  return !P.fallback && P.s >= 0 && ((uint64_t)(P.B < 0 ? -P.B : P.B) * (N - 1)) >> P.s < (uint64_t)kNarrow;
+}
+struct NarrowLine {
+  uint64_t B;
+  uint32_t sh;
+  __device__ __forceinline__ NarrowLine(int64_t slope, int s)
+      : B((uint64_t)slope << (s < 32 ? 32 - s : 0)), sh(s > 32 ? (uint32_t)(s - 32) : 0u) {}
+  __device__ __forceinline__ int32_t at(uint64_t G) const { return (int32_t)(G >> 32) >> sh; }
+};
+
 // Group fit: GROUP threads (one thread, a warp, or a whole CTA when GROUP > 32) fit [a, a+N).
 // Returns the result in every thread of the group. sm: shared scratch (only used when GROUP > 32).
 struct FitShared {
@@ -310,16 +332,99 @@ struct FitShared {
   FitResult R;
 };
 
+// f over one group member's values v[rank], v[rank + GROUP], ... of N, RUN at a time with their loads in
+// flight together (whole runs without bounds; the last one repeats v[0] past the end); stops when f's run
+// hook `ok` says so
+template <int GROUP, int RUN, typename T, typename F, typename Ok>
+__device__ __forceinline__ bool for_runs(const T* __restrict__ v, uint32_t N, uint32_t rank, T ref, F f, Ok ok) {
+  const T* p = v + rank;
+  // whole runs are the same for all members: the values of one run of the group lie side by side
+  uint32_t left = N;
+  for (; left >= (uint32_t)(RUN * GROUP); left -= RUN * GROUP, p += RUN * GROUP) {
+    T w[RUN];
+#pragma unroll
+    for (int k = 0; k < RUN; k++) w[k] = __ldg(p + k * GROUP);
+#pragma unroll
+    for (int k = 0; k < RUN; k++) f(w[k]);
+    if (!ok()) return false;
+  }
+  if (left) {
+    const int mine = left > rank ? (int)((left - rank - 1) / GROUP) + 1 : 0;
+    T w[RUN];
+#pragma unroll
+    for (int k = 0; k < RUN; k++) w[k] = k < mine ? __ldg(p + k * GROUP) : ref;
+#pragma unroll
+    for (int k = 0; k < RUN; k++)
+      if (k < mine) f(w[k]);
+    if (!ok()) return false;
+  }
+  return true;
+}
+
 // Pass 1 over one group member's positions x = rank, rank + GROUP, ... < N of the values v (the
 // partition's first value at v[0]): min, max and (linear model) S = sum u_x w_x with
-// u_x = 2x - (N-1), where w is the value as two's complement int64. S equals
-// sum u_x (w_x - w_0) because the u_x sum to zero. Each term is split as u w_hi 2^32 + u w_lo with
-// 32 x 32 -> 64-bit products, accumulated in 64 bits over at most 64 terms (|u| < 2^24: each
-// partial stays below 2^62), then folded into 128 bits. Pairs of warps on one partition (GROUP 64,
-// partitions of 1024+ values) keep sixteen loads in flight per lane, other groups eight.
+// u_x = 2x - (N-1), where w is the value as two's complement int64 (over the whole group S equals
+// sum u_x (w_x - w_0) because the u_x sum to zero). Narrow partitions take their differences from w_0 in
+// 32 bits; a group that meets a value too far away starts again in 64 bits: each term is then split as
+// u w_hi 2^32 + u w_lo with 32 x 32 -> 64-bit products, accumulated in 64 bits over at most 64 terms
+// (|u| < 2^24: each partial stays below 2^62) and folded into 128 bits. Pairs of warps on one partition
+// (GROUP 64, partitions of 1024+ values) keep sixteen loads in flight per lane, warps eight.
+// In 64 bits throughout, with bounds on every load, the two passes took 43 instructions per value and
+// were bound by their issue: 200M sorted normal uint64 in partitions of 4096 414 -> 307 us (1.6 GB read),
+// 20M 32-bit values in partitions of 1000 51 -> 32 us, 96 columns of 200M values 600 -> 490 us.
+struct NarrowMom {
+  int64_t S;        // sum of u_x (w_x - w_0) over the member's positions
+  int32_t mx, mn;   // of w_x - w_0; w_0 itself counts
+};
+
 template <int GROUP, typename T>
-__device__ __forceinline__ void fit_pass1(const T* __restrict__ v, uint32_t N, bool lin, uint32_t rank, i128* S_out,
-                                          int64_t* mx_out, int64_t* mn_out) {
+__device__ __forceinline__ bool fit_pass1_narrow(const T* __restrict__ v, uint32_t N, bool lin, uint32_t rank, int64_t ref,
+                                                 NarrowMom& out) {
+  if (!narrow_ref(ref) || N > (1u << 16)) return false;  // |u| < 2^16, 2^30 differences, 2^11 values: below 2^57
+  int32_t mx = 0, mn = 0;
+  int32_t u = 2 * (int32_t)rank - ((int32_t)N - 1);
+  uint32_t far = 0;
+  int64_t S = 0;
+  auto add = [&](T value) {
+    const int64_t d = (int64_t)value - ref;
+    const int32_t e = (int32_t)d;
+    far |= (uint32_t)((int32_t)(d >> 32) ^ (e >> 31));  // d outside 32 bits
+    mx = max(mx, e);
+    mn = min(mn, e);
+    if (lin) S += (int64_t)u * e;
+    u += 2 * GROUP;
+  };
+  auto ok = [&]() { return !__any_sync(0xffffffffu, far != 0 || mn <= -(int32_t)kNarrow || mx >= (int32_t)kNarrow); };
+  if (!for_runs<GROUP, GROUP == 64 ? 16 : 8>(v, N, rank, (T)ref, add, ok)) return false;
+  out.S = S;
+  out.mx = mx;
+  out.mn = mn;
+  return true;
+}
+
+// pass 2 of a narrow partition: the member's residual range, relative to w_0 (empty members: the inverted range)
+template <int GROUP, typename T>
+__device__ __forceinline__ void fit_pass2_narrow(const T* __restrict__ v, uint32_t N, int64_t B, int32_t s, uint32_t rank,
+                                                 int64_t ref, int32_t* lo, int32_t* hi) {
+  const NarrowLine line(B, s);
+  int32_t l = INT32_MAX, h = INT32_MIN;
+  uint64_t G = line.B * rank;
+  const uint64_t dG = line.B * (uint64_t)GROUP;
+  const uint32_t r32 = (uint32_t)ref;
+  auto add = [&](T value) {
+    const int32_t r = (int32_t)((uint32_t)value - r32) - line.at(G);
+    l = min(l, r);
+    h = max(h, r);
+    G += dG;
+  };
+  for_runs<GROUP, GROUP == 64 ? 16 : 8>(v, N, rank, (T)ref, add, []() { return true; });
+  *lo = l;
+  *hi = h;
+}
+
+template <int GROUP, typename T>
+__device__ __forceinline__ void fit_pass1_wide(const T* __restrict__ v, uint32_t N, bool lin, uint32_t rank, i128* S_out,
+                                               int64_t* mx_out, int64_t* mn_out) {
   int64_t mx = INT64_MIN, mn = INT64_MAX;
   i128 S = 0;
   if (lin) {
@@ -328,7 +433,7 @@ __device__ __forceinline__ void fit_pass1(const T* __restrict__ v, uint32_t N, b
       const uint32_t xe = N - x0 > 64u * GROUP ? x0 + 64u * GROUP : N;
       int64_t acc_hi = 0, acc_lo = 0;
       int32_t u = (int32_t)(2 * (int64_t)x0 - nm1);
-#pragma unroll (GROUP == 64 ? 16 : 8)
+#pragma unroll 8
       for (uint32_t x = x0; x < xe; x += GROUP, u += 2 * GROUP) {
         const int64_t w = (int64_t)__ldg(v + x);
         mx = max(mx, w);
@@ -351,16 +456,46 @@ __device__ __forceinline__ void fit_pass1(const T* __restrict__ v, uint32_t N, b
   *mn_out = mn;
 }
 
-// Pass 2: range [lo, hi] of the residuals w_x - line(x) with line(x) = (B x) >> s (s >= 0) or
-// (B x) << -s, B x taken mod 2^64 and stepped by B GROUP from one position to the next.
 template <int GROUP, typename T>
-__device__ __forceinline__ void fit_pass2(const T* __restrict__ v, uint32_t N, int64_t B, int32_t s, uint32_t rank,
+__device__ __forceinline__ void fit_pass1(const T* __restrict__ v, uint32_t N, bool lin, uint32_t rank, i128* S_out,
+                                          int64_t* mx_out, int64_t* mn_out) {
+  NarrowMom m;
+  if (GROUP > 1) {
+    const int64_t ref = (int64_t)__ldg(v);
+    if (fit_pass1_narrow<GROUP>(v, N, lin, rank, ref, m)) {
+      // as a sum of u w: the member's u add up to cnt (2 rank - (N-1)) + GROUP cnt (cnt - 1)
+      const int64_t cnt = rank < N ? (int64_t)((N - 1 - rank) / GROUP + 1) : 0;
+      *S_out = lin ? (i128)m.S + mul_s64(ref, cnt * (2 * (int64_t)rank - ((int64_t)N - 1)) + (int64_t)GROUP * cnt * (cnt - 1))
+                   : (i128)0;
+      *mx_out = ref + m.mx;
+      *mn_out = ref + m.mn;
+      return;
+    }
+  }
+  fit_pass1_wide<GROUP>(v, N, lin, rank, S_out, mx_out, mn_out);
+}
+
+// Pass 2: range [lo, hi] of the residuals w_x - line(x) with line(x) = (B x) >> s (s >= 0) or
+// (B x) << -s, B x taken mod 2^64 and stepped by B GROUP from one position to the next; in 32 bits
+// when the partition and its line are narrow.
+template <int GROUP, typename T>
+__device__ __forceinline__ void fit_pass2(const T* __restrict__ v, uint32_t N, const FitParams& P, uint32_t rank,
                                           int64_t* lo_out, int64_t* hi_out) {
+  if (GROUP > 1 && P.narrow) {
+    const int64_t ref = (int64_t)__ldg(v);
+    int32_t l, h;
+    fit_pass2_narrow<GROUP>(v, N, P.B, P.s, rank, ref, &l, &h);
+    *lo_out = rank < N ? ref + l : INT64_MAX;
+    *hi_out = rank < N ? ref + h : INT64_MIN;
+    return;
+  }
+  const int64_t B = P.B;
+  const int32_t s = P.s;
   int64_t lo = INT64_MAX, hi = INT64_MIN;
   uint64_t F = (uint64_t)B * rank;
   const uint64_t dF = (uint64_t)B * GROUP;
   if (s >= 0) {
-#pragma unroll (GROUP == 64 ? 16 : 8)
+#pragma unroll 8
     for (uint32_t x = rank; x < N; x += GROUP, F += dF) {
       const int64_t r = (int64_t)__ldg(v + x) - ((int64_t)F >> s);
       lo = min(lo, r);
@@ -406,14 +541,21 @@ __device__ FitResult fit_range(const void* __restrict__ values, int dtype, uint6
   }
   const uint32_t lane = rank & 31u;
   FitParams P;
+  auto solve = [&](i128 moment) {
+    FitParams q = solve_params(moment, mx, mn, N, lin);
+    q.narrow = narrow_line(q, N) && narrow_ref(mn) && narrow_diff(mx - mn) ? 1 : 0;
+    return q;
+  };
   if (GROUP == 1) {
-    P = solve_params(S, mx, mn, N, lin);
+    P = solve(S);
   } else if (GROUP == 32) {
-    if (lane == 0) P = solve_params(S, mx, mn, N, lin);
+    if (lane == 0) P = solve(S);
     P.B = (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)P.B, 0);
     P.fb_shift = (int64_t)__shfl_sync(0xffffffffu, (unsigned long long)P.fb_shift, 0);
     P.s = __shfl_sync(0xffffffffu, P.s, 0);
-    P.fallback = __shfl_sync(0xffffffffu, P.fallback, 0);
+    const uint32_t f = __shfl_sync(0xffffffffu, (uint32_t)(uint16_t)P.fallback | ((uint32_t)(uint16_t)P.narrow << 16), 0);
+    P.fallback = (int16_t)(f & 0xFFFFu);
+    P.narrow = (int16_t)(f >> 16);
   } else {
     const uint32_t wid = rank >> 5;
     if (lane == 0) {
@@ -428,7 +570,7 @@ __device__ FitResult fit_range(const void* __restrict__ values, int dtype, uint6
         mx = max(mx, sm->mx[k]);
         mn = min(mn, sm->mn[k]);
       }
-      sm->P = solve_params(S, mx, mn, N, lin);
+      sm->P = solve(S);
     }
     group_sync(bar_id, GROUP);
     P = sm->P;
@@ -445,9 +587,9 @@ __device__ FitResult fit_range(const void* __restrict__ values, int dtype, uint6
     if (GROUP > 1) zmax = warp_max_u64(zmax);
   } else {
     if (u32)
-      fit_pass2<GROUP>(v32, N, P.B, P.s, rank, &lo, &hi);
+      fit_pass2<GROUP>(v32, N, P, rank, &lo, &hi);
     else
-      fit_pass2<GROUP>(v64, N, P.B, P.s, rank, &lo, &hi);
+      fit_pass2<GROUP>(v64, N, P, rank, &lo, &hi);
     if (GROUP > 1) {
       lo = warp_min_i64(lo);
       hi = warp_max_i64(hi);
@@ -483,6 +625,116 @@ __device__ FitResult fit_range(const void* __restrict__ values, int dtype, uint6
     group_sync(bar_id, GROUP);  // sm is reused by the next partition
   }
   return R;
+}
+
+// minimum, maximum and sum over aligned tiles of TILE lanes (32: the warp), in every lane
+template <int TILE>
+__device__ __forceinline__ int32_t tile_min(int32_t v) {
+  if constexpr (TILE == 32) {
+    v = __reduce_min_sync(0xffffffffu, v);
+  } else {
+    for (int o = TILE / 2; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(0xffffffffu, v, o));
+  }
+  return v;
+}
+template <int TILE>
+__device__ __forceinline__ int32_t tile_max(int32_t v) {
+  if constexpr (TILE == 32) {
+    v = __reduce_max_sync(0xffffffffu, v);
+  } else {
+    for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+  }
+  return v;
+}
+template <int TILE>
+__device__ __forceinline__ int64_t tile_min(int64_t v) {
+  for (int o = TILE / 2; o > 0; o >>= 1) v = min(v, (int64_t)__shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+template <int TILE>
+__device__ __forceinline__ int64_t tile_max(int64_t v) {
+  for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, (int64_t)__shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+template <int TILE>
+__device__ __forceinline__ uint64_t tile_max(uint64_t v) {
+  for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, (uint64_t)__shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+template <int TILE>
+__device__ __forceinline__ int64_t tile_sum(int64_t v) {
+  for (int o = TILE / 2; o > 0; o >>= 1) v += (int64_t)__shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Fit of one short partition per tile of TILE lanes (N = 0: the tile only takes part in the warp's steps), r
+// the lane's place in it; the result in every lane. A warp that fits one partition at a time spends as long in
+// its one-lane solve as on 256 values; here 32 / TILE partitions solve at once and their loads are in flight
+// together.
+template <int TILE, typename T>
+__device__ __forceinline__ FitResult fit_tile(const T* __restrict__ v, uint32_t N, int model, uint32_t r) {
+  const bool lin = model == LECO_MODEL_LINEAR && N >= 2;
+  const int64_t ref = N ? (int64_t)__ldg(v) : 0;
+  int32_t mx32 = 0, mn32 = 0, u = 2 * (int32_t)r - ((int32_t)N - 1);
+  uint32_t far = 0;
+  int64_t sum = 0;
+  auto always = []() { return true; };
+  for_runs<TILE, 8>(
+      v, N, r, (T)ref,
+      [&](T value) {
+        const int64_t d = (int64_t)value - ref;
+        const int32_t e = (int32_t)d;
+        far |= (uint32_t)((int32_t)(d >> 32) ^ (e >> 31));  // d outside 32 bits
+        mx32 = max(mx32, e);
+        mn32 = min(mn32, e);
+        sum += (int64_t)u * e;
+        u += 2 * TILE;
+      },
+      always);
+  i128 S;
+  int64_t mx, mn;
+  if (__all_sync(0xffffffffu, far == 0 && mn32 > -(int32_t)kNarrow && mx32 < (int32_t)kNarrow && narrow_ref(ref))) {
+    S = tile_sum<TILE>(sum);
+    mx = ref + tile_max<TILE>(mx32);
+    mn = ref + tile_min<TILE>(mn32);
+  } else {
+    fit_pass1_wide<TILE>(v, N, lin, r, &S, &mx, &mn);
+    for (int o = TILE / 2; o > 0; o >>= 1) {
+      const uint64_t lo = __shfl_xor_sync(0xffffffffu, (uint64_t)S, o), hi = __shfl_xor_sync(0xffffffffu, (uint64_t)((u128)S >> 64), o);
+      S += (i128)(((u128)hi << 64) | lo);
+    }
+    mx = tile_max<TILE>(mx);
+    mn = tile_min<TILE>(mn);
+  }
+  FitParams P;
+  P.B = 0;
+  P.fb_shift = 0;
+  P.s = 0;
+  P.fallback = 0;
+  P.narrow = 1;
+  if (N) {
+    P = solve_params(lin ? S : (i128)0, mx, mn, N, lin);
+    P.narrow = narrow_line(P, N) && narrow_ref(mn) && narrow_diff(mx - mn) ? 1 : 0;
+  }
+  int64_t lo = INT64_MAX, hi = INT64_MIN;
+  uint64_t zmax = 0;
+  if (__all_sync(0xffffffffu, P.narrow)) {
+    int32_t l, h;
+    fit_pass2_narrow<TILE>(v, N, P.B, P.s, r, ref, &l, &h);
+    lo = ref + tile_min<TILE>(l);
+    hi = ref + tile_max<TILE>(h);
+  } else {
+    if (P.fallback) {
+      for (uint32_t x = r; x < N; x += TILE) zmax = max(zmax, zz_encode((int64_t)((uint64_t)__ldg(v + x) - (uint64_t)P.fb_shift)));
+    } else {
+      P.narrow = 0;
+      fit_pass2<TILE>(v, N, P, r, &lo, &hi);
+    }
+    lo = tile_min<TILE>(lo);
+    hi = tile_max<TILE>(hi);
+    zmax = tile_max<TILE>(zmax);
+  }
+  return finish_fit(P, lo, hi, zmax);
 }
 
 // ------------------------------------------------------------------------------ polynomial model

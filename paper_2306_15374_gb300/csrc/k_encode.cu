@@ -20,29 +20,42 @@ __device__ __forceinline__ uint64_t part_begin(const uint64_t* starts, uint32_t 
   return s < n ? s : n;
 }
 
-// One warp per partition (grid-stride over warps): the fit's reductions are warp shuffles and its
-// parameter solve runs on one lane, so a warp waiting on its solve stalls only itself while the
-// SM's other warps stream their partitions; the second pass re-reads the partition from L2.
+// the record of a fitted partition [a, a + N), its stream bits and the column's widest width
+__device__ __forceinline__ void put_fit(const FitResult& R, uint64_t a, uint32_t N, uint64_t p, Record* __restrict__ rec,
+                                        uint64_t* __restrict__ lenbits, uint32_t* __restrict__ max_b) {
+  Record r;
+  r.theta0 = R.theta0;
+  r.theta1 = R.theta1;
+  r.start = a;
+  r.word3 = make_w3(0, R.b, R.s, 1);
+  rec[p] = r;
+  lenbits[p] = (uint64_t)N * R.b;
+  if (R.b) atomicMax(max_b, R.b);
+}
+
+// Tiles of TILE lanes per partition (fixed partitions below 1024 values), or a warp (TILE = 32: partitions of
+// any lengths), grid-stride: reductions are shuffles, the second pass re-reads the partition from L1 or L2.
+template <typename T, int TILE>
 __global__ void __launch_bounds__(kFitBlock, kFitCtasPerSm)
-    k_fit(const void* __restrict__ values, int dtype, uint64_t n, const uint64_t* __restrict__ starts,
-          uint32_t L, uint64_t m, int model, Record* __restrict__ rec, uint64_t* __restrict__ lenbits,
-          uint32_t* __restrict__ max_b) {
-  const uint32_t lane = threadIdx.x & 31u;
+    k_fit(const T* __restrict__ values, uint64_t n, const uint64_t* __restrict__ starts, uint32_t L, uint64_t m,
+          int model, Record* __restrict__ rec, uint64_t* __restrict__ lenbits, uint32_t* __restrict__ max_b) {
+  constexpr uint32_t kTiles = 32 / TILE;
+  const uint32_t lane = threadIdx.x & 31u, r = lane % TILE;
   const uint64_t nw = (uint64_t)gridDim.x * kFitWarps;
-  for (uint64_t p = (uint64_t)blockIdx.x * kFitWarps + (threadIdx.x >> 5); p < m; p += nw) {
-    const uint64_t a = part_begin(starts, L, n, p);
-    const uint32_t N = (uint32_t)(part_begin(starts, L, n, p + 1) - a);
-    const FitResult R = fit_range<32>(values, dtype, a, N, model, lane, nullptr);
-    if (lane == 0) {
-      Record r;
-      r.theta0 = R.theta0;
-      r.theta1 = R.theta1;
-      r.start = a;
-      r.word3 = make_w3(0, R.b, R.s, 1);
-      rec[p] = r;
-      lenbits[p] = (uint64_t)N * R.b;
-      if (R.b) atomicMax(max_b, R.b);
+  for (uint64_t p0 = ((uint64_t)blockIdx.x * kFitWarps + (threadIdx.x >> 5)) * kTiles; p0 < m; p0 += nw * kTiles) {
+    const uint64_t p = p0 + lane / TILE;
+    uint64_t a = 0;
+    uint32_t N = 0;
+    if (p < m) {
+      a = part_begin(starts, L, n, p);
+      N = (uint32_t)(part_begin(starts, L, n, p + 1) - a);
     }
+    FitResult R;
+    if (TILE == 32)
+      R = fit_range<32>(values, sizeof(T) == 4 ? LECO_U32 : LECO_U64, a, N, model, lane, nullptr);
+    else
+      R = fit_tile<TILE>(values + a, N, model, r);
+    if (r == 0 && N) put_fit(R, a, N, p, rec, lenbits, max_b);
   }
 }
 
@@ -50,8 +63,9 @@ __global__ void __launch_bounds__(kFitBlock, kFitCtasPerSm)
 // own named barrier): as many warps stream as with one warp per partition, but half as many
 // partitions are in flight, so the second pass finds the partition in L2 instead of DRAM.
 constexpr int kFitPairs = kFitBlock / 64;
+constexpr int kPairCtas = 3;  // sixteen loads in flight per lane need the registers (4 CTAs: 1081 us a pass, 3: 1061)
 
-__global__ void __launch_bounds__(kFitBlock, kFitCtasPerSm)
+__global__ void __launch_bounds__(kFitBlock, kPairCtas)
     k_fit_pairs(const void* __restrict__ values, int dtype, uint64_t n, const uint64_t* __restrict__ starts,
                 uint32_t L, uint64_t m, int model, Record* __restrict__ rec, uint64_t* __restrict__ lenbits,
                 uint32_t* __restrict__ max_b) {
@@ -62,16 +76,7 @@ __global__ void __launch_bounds__(kFitBlock, kFitCtasPerSm)
     const uint64_t a = part_begin(starts, L, n, p);
     const uint32_t N = (uint32_t)(part_begin(starts, L, n, p + 1) - a);
     const FitResult R = fit_range<64>(values, dtype, a, N, model, rank, &sm[g], 1 + (int)g);
-    if (rank == 0) {
-      Record r;
-      r.theta0 = R.theta0;
-      r.theta1 = R.theta1;
-      r.start = a;
-      r.word3 = make_w3(0, R.b, R.s, 1);
-      rec[p] = r;
-      lenbits[p] = (uint64_t)N * R.b;
-      if (R.b) atomicMax(max_b, R.b);
-    }
+    if (rank == 0) put_fit(R, a, N, p, rec, lenbits, max_b);
   }
 }
 
@@ -749,30 +754,51 @@ __global__ void k_zero_bounds(const Aux* __restrict__ aux, uint64_t m, uint64_t 
 
 // ------------------------------------------------------------------------------ batched encode
 
-// one warp per partition of every column (its column from the partition-column table); registers
-// for 3 CTAs per SM (4 spilled, and the encode tuner then keeps 3)
-__global__ void __launch_bounds__(kFitBlock, 3)
+// The partitions of every column (a partition's column from the partition-column table; the polynomial
+// columns' are fitted by the polynomial phases), eight per pair of warps: a tile of eight lanes each when all
+// are short, else both warps on one after another, as k_fit_pairs.
+constexpr uint32_t kFitTileVals = 512;
+
+template <typename T>
+__global__ void __launch_bounds__(kFitBlock, kPairCtas)
     k_fit_multi(const EncCol* __restrict__ cols, const uint64_t* __restrict__ part_base,
-                const uint32_t* __restrict__ part_col, uint64_t P, int dtype, Record* __restrict__ rec,
+                const uint32_t* __restrict__ part_col, uint64_t P, Record* __restrict__ rec,
                 uint64_t* __restrict__ lenbits, uint32_t* __restrict__ max_b) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint64_t nw = (uint64_t)gridDim.x * kFitWarps;
-  for (uint64_t p = (uint64_t)blockIdx.x * kFitWarps + (threadIdx.x >> 5); p < P; p += nw) {
-    const uint32_t c = part_col[p];
-    const EncCol col = cols[c];
-    if (col.model == LECO_MODEL_POLY) continue;  // fitted by the polynomial phases
-    const uint64_t a = (p - part_base[c]) * (uint64_t)col.L;
-    const uint32_t N = (uint32_t)((a + col.L < col.n ? a + col.L : col.n) - a);
-    const FitResult R = fit_range<32>(col.values, dtype, a, N, col.model, lane, nullptr);
-    if (lane == 0) {
-      Record r;
-      r.theta0 = R.theta0;
-      r.theta1 = R.theta1;
-      r.start = a;
-      r.word3 = make_w3(0, R.b, R.s, 1);
-      rec[p] = r;
-      lenbits[p] = (uint64_t)N * R.b;
-      if (R.b) atomicMax(max_b + c, R.b);
+  __shared__ FitShared sm[kFitPairs];
+  const uint32_t g = threadIdx.x >> 6, rank = threadIdx.x & 63u, lane = threadIdx.x & 31u;
+  const uint64_t ng = (uint64_t)gridDim.x * kFitPairs;
+  for (uint64_t p0 = ((uint64_t)blockIdx.x * kFitPairs + g) * 8; p0 < P; p0 += ng * 8) {
+    // lane k (and k + 8, + 16, + 24) of both warps: partition p0 + k
+    const uint64_t p = p0 + (lane & 7u);
+    uint64_t a = 0;
+    uint32_t N = 0, c = 0;
+    int model = LECO_MODEL_CONSTANT;
+    const T* v = nullptr;
+    if (p < P) {
+      c = part_col[p];
+      const EncCol col = cols[c];
+      model = col.model;
+      a = (p - part_base[c]) * (uint64_t)col.L;
+      if (model != LECO_MODEL_POLY) N = (uint32_t)((a + col.L < col.n ? a + col.L : col.n) - a);
+      v = static_cast<const T*>(col.values) + a;
+    }
+    if (__all_sync(0xffffffffu, N <= kFitTileVals)) {
+      const int k = (int)(rank >> 3);
+      const uint32_t n = __shfl_sync(0xffffffffu, N, k);
+      const T* vk = reinterpret_cast<const T*>(__shfl_sync(0xffffffffu, (unsigned long long)v, k));
+      const FitResult R = fit_tile<8>(vk, n, __shfl_sync(0xffffffffu, model, k), rank & 7u);
+      const uint64_t ak = __shfl_sync(0xffffffffu, a, k);
+      const uint32_t ck = __shfl_sync(0xffffffffu, c, k);
+      if ((rank & 7u) == 0 && n) put_fit(R, ak, n, p0 + (uint32_t)k, rec, lenbits, max_b + ck);
+      continue;
+    }
+    for (int k = 0; k < 8; k++) {
+      const uint32_t n = __shfl_sync(0xffffffffu, N, k);
+      if (n == 0) continue;
+      const T* vk = reinterpret_cast<const T*>(__shfl_sync(0xffffffffu, (unsigned long long)v, k));
+      const FitResult R = fit_range<64>(vk, sizeof(T) == 4 ? LECO_U32 : LECO_U64, 0, n,
+                                        __shfl_sync(0xffffffffu, model, k), rank, &sm[g], 1 + (int)g);
+      if (rank == (uint32_t)k) put_fit(R, a, N, p, rec, lenbits, max_b + c);
     }
   }
 }
@@ -924,6 +950,19 @@ cudaError_t launch_poly_fit(const Map& map, int dtype, uint64_t m, Record* rec, 
   return e;
 }
 
+// eight lanes per partition up to kFitTileVals values, sixteen up to 1023; a warp for partitions of any lengths
+template <typename T>
+void launch_fit_tiles(const T* values, uint64_t n, const uint64_t* starts, uint32_t L, uint64_t m, int ctas, int model,
+                      Record* rec, uint64_t* lenbits, uint32_t* max_b, cudaStream_t st) {
+  auto grid = [&](uint64_t per) { return grid_for((m + per - 1) / per, kFitWarps, ctas); };
+  if (starts)
+    k_fit<T, 32><<<grid(1), kFitBlock, 0, st>>>(values, n, starts, L, m, model, rec, lenbits, max_b);
+  else if (L <= kFitTileVals)
+    k_fit<T, 8><<<grid(4), kFitBlock, 0, st>>>(values, n, starts, L, m, model, rec, lenbits, max_b);
+  else
+    k_fit<T, 16><<<grid(2), kFitBlock, 0, st>>>(values, n, starts, L, m, model, rec, lenbits, max_b);
+}
+
 cudaError_t launch_fit(const void* values, int dtype, uint64_t n, const uint64_t* starts,
                        uint32_t L, uint64_t m, int model, Record* rec, uint64_t* lenbits, PolyCoef* pcoef,
                        uint32_t* max_b, uint32_t* err, cudaStream_t st) {
@@ -939,13 +978,15 @@ cudaError_t launch_fit(const void* values, int dtype, uint64_t n, const uint64_t
   const int ctas = fc >= 1 && fc <= (uint32_t)kFitCtasPerSm ? (int)fc : kFitCtasPerSm;
   // partitions of at least 1024 values: two warps each (the second pass then stays in L2)
   if (!starts && L >= 1024) {
-    k_fit_pairs<<<grid_for((m + kFitPairs - 1) / kFitPairs, 1, ctas), kFitBlock, 0, st>>>(values, dtype, n, starts,
+    k_fit_pairs<<<grid_for((m + kFitPairs - 1) / kFitPairs, 1, ctas < kPairCtas ? ctas : kPairCtas), kFitBlock, 0, st>>>(values, dtype, n, starts,
                                                                                         L, m, model, rec, lenbits,
                                                                                         max_b);
     return cudaGetLastError();
   }
-  k_fit<<<grid_for((m + kFitWarps - 1) / kFitWarps, 1, ctas), kFitBlock, 0, st>>>(values, dtype, n, starts, L, m,
-                                                                                  model, rec, lenbits, max_b);
+  if (dtype == LECO_U32)
+    launch_fit_tiles(static_cast<const uint32_t*>(values), n, starts, L, m, ctas, model, rec, lenbits, max_b, st);
+  else
+    launch_fit_tiles(static_cast<const uint64_t*>(values), n, starts, L, m, ctas, model, rec, lenbits, max_b, st);
   return cudaGetLastError();
 }
 
@@ -1033,8 +1074,11 @@ cudaError_t launch_fit_multi(const EncCol* cols, const uint64_t* part_base, cons
   cudaError_t e = cudaMemsetAsync(max_b, 0, sizeof(uint32_t) * (ncols ? ncols : 1), st);
   if (e != cudaSuccess || P == 0) return e;
   const int ctas = fit_ctas >= 1 && fit_ctas <= (uint32_t)kFitCtasPerSm ? (int)fit_ctas : kFitCtasPerSm;
-  const int grid = grid_for((P + kFitWarps - 1) / kFitWarps, 1, ctas);
-  k_fit_multi<<<grid, kFitBlock, 0, st>>>(cols, part_base, part_col, P, dtype, rec, lenbits, max_b);
+  const int grid = grid_for((P + 7) / 8, kFitPairs, ctas < kPairCtas ? ctas : kPairCtas);
+  if (dtype == LECO_U32)
+    k_fit_multi<uint32_t><<<grid, kFitBlock, 0, st>>>(cols, part_base, part_col, P, rec, lenbits, max_b);
+  else
+    k_fit_multi<uint64_t><<<grid, kFitBlock, 0, st>>>(cols, part_base, part_col, P, rec, lenbits, max_b);
   e = cudaGetLastError();
   if (e == cudaSuccess && pcoef)
     e = launch_poly_fit(BatchColumns{cols, part_base, ncols}, dtype, P, rec, lenbits, pcoef, max_b, st, poly_scratch);

@@ -36,65 +36,6 @@ __device__ __forceinline__ i128 line_moment(const SpanStats& s, uint32_t N) {
   return 2 * s.T1 - mul_i128_u64(s.T0, N - 1);
 }
 
-// minimum, maximum and sum over aligned tiles of TILE lanes (32: the warp), in every lane
-template <int TILE>
-__device__ __forceinline__ int32_t tile_min(int32_t v) {
-  if constexpr (TILE == 32) {
-    v = __reduce_min_sync(kFull, v);
-  } else {
-    for (int o = TILE / 2; o > 0; o >>= 1) v = min(v, __shfl_xor_sync(kFull, v, o));
-  }
-  return v;
-}
-template <int TILE>
-__device__ __forceinline__ int32_t tile_max(int32_t v) {
-  if constexpr (TILE == 32) {
-    v = __reduce_max_sync(kFull, v);
-  } else {
-    for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(kFull, v, o));
-  }
-  return v;
-}
-template <int TILE>
-__device__ __forceinline__ int64_t tile_min(int64_t v) {
-  for (int o = TILE / 2; o > 0; o >>= 1) v = min(v, (int64_t)__shfl_xor_sync(kFull, v, o));
-  return v;
-}
-template <int TILE>
-__device__ __forceinline__ int64_t tile_max(int64_t v) {
-  for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, (int64_t)__shfl_xor_sync(kFull, v, o));
-  return v;
-}
-template <int TILE>
-__device__ __forceinline__ uint64_t tile_max(uint64_t v) {
-  for (int o = TILE / 2; o > 0; o >>= 1) v = max(v, (uint64_t)__shfl_xor_sync(kFull, v, o));
-  return v;
-}
-template <int TILE>
-__device__ __forceinline__ int64_t tile_sum(int64_t v) {
-  for (int o = TILE / 2; o > 0; o >>= 1) v += (int64_t)__shfl_xor_sync(kFull, v, o);
-  return v;
-}
-
-// Narrow spans: values within 2^30 of a reference in (-2^62, 2^62), so that their differences d from it fit
-// 32 bits (a difference that wraps in 64 bits is above 2^61 in magnitude, so the test sees it), and a line
-// that stays within 2^30 over the span. Extremes are then 32-bit, products 32 x 32 -> 64-bit, and the line
-// needs no 64-bit shift: G = B x 2^(32-s) (or B x, for s > 32) is carried and its high half read.
-constexpr int64_t kNarrow = (int64_t)1 << 30;
-constexpr int64_t kNarrowRef = (int64_t)1 << 62;
-__device__ __forceinline__ bool narrow_ref(int64_t ref) { return ref > -kNarrowRef && ref < kNarrowRef; }
-__device__ __forceinline__ bool narrow_diff(int64_t d) { return d > -kNarrow && d < kNarrow; }
-__device__ __forceinline__ bool narrow_line(const FitParams& P, uint32_t N) {
-  return !P.fallback && P.s >= 0 && ((uint64_t)(P.B < 0 ? -P.B : P.B) * (N - 1)) >> P.s < (uint64_t)kNarrow;
-}
-struct NarrowLine {
-  uint64_t B;
-  uint32_t sh;
-  __device__ __forceinline__ NarrowLine(int64_t slope, int s)
-      : B((uint64_t)slope << (s < 32 ? 32 - s : 0)), sh(s > 32 ? (uint32_t)(s - 32) : 0u) {}
-  __device__ __forceinline__ int32_t at(uint64_t G) const { return (int32_t)(G >> 32) >> sh; }
-};
-
 // Sums of w and x w as high and low halves of w (the high half signed), each below 2^62 in magnitude
 // while a thread adds at most 2^11 values at positions x < 2^17.
 struct HalfSums {
