@@ -71,7 +71,7 @@ leco_status alloc_meta(leco_column* c, cudaStream_t st) {
   c->tiles = (TileDesc*)(b + 2 * rec_b + starts_b);
   c->status = (uint32_t*)(b + 2 * rec_b + starts_b + tiles_b);
   c->poly = poly_b ? (PolyAux*)(b + 2 * rec_b + starts_b + tiles_b + 256) : nullptr;
-  return from_cuda(cudaMemsetAsync(c->status, 0, 256, st));
+  return LECO_OK;  // the status word is cleared with the decode table's build
 }
 
 void release(leco_column* c, cudaStream_t st) {
@@ -108,7 +108,6 @@ leco_status encode_partitions(leco_column* c, const void* d_values, cudaStream_t
   const uint64_t* starts = c->kind == LECO_PART_VAR ? c->starts : nullptr;
   uint64_t hres[2] = {0, 0};
   uint64_t& total = hres[0];
-  uint32_t flags = 0;
   if (prefit)
     e = launch_lenbits(c->rec, starts, m, lenbits, d_maxb, st);
   else
@@ -117,12 +116,7 @@ leco_status encode_partitions(leco_column* c, const void* d_values, cudaStream_t
   if (e == cudaSuccess)
     e = launch_offsets(c->rec, lenbits, m, off_scr, offsets_scratch_elems(m), d_total, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hres, d_total, 16, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&flags, c->status, 4, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && (flags & kStatTimeout)) {
-    cudaFreeAsync(scr, st);
-    return LECO_ERR_TIMEOUT;  // a staging copy never landed: the fit is incomplete
-  }
   if (e == cudaSuccess && total >= (1ull << 48)) e = cudaErrorInvalidValue;
   if (e == cudaSuccess) {
     c->total_bits = total;
@@ -132,11 +126,12 @@ leco_status encode_partitions(leco_column* c, const void* d_values, cudaStream_t
     c->words_bytes = c->nwords * 8;
     e = dev_alloc((void**)&c->words, c->words_bytes, st);
   }
-  if (e == cudaSuccess) e = launch_build_aux(c->rec, pcoef, m, c->n, c->aux, c->poly, c->status, st);
+  if (e == cudaSuccess)
+    e = launch_build_aux(c->rec, pcoef, m, c->n, c->aux, c->poly, total, c->words, c->nwords, c->status, st);
   if (e == cudaSuccess) e = launch_tile_desc(view_of(c), c->tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack(d_values, c->dtype, starts ? 0u : c->L, c->tiles, c->rec, c->aux, pcoef, c->poly, m, c->n, total,
-                    c->words, c->nwords, st);
+    e = launch_pack(d_values, c->dtype, starts ? 0u : c->L, c->tiles, c->rec, c->aux, pcoef, c->poly, m, c->n,
+                    c->words, st);
   cudaFreeAsync(scr, st);
   if (e == cudaErrorInvalidValue) return LECO_ERR_INVALID_ARG;
   return from_cuda(e);
@@ -656,7 +651,7 @@ leco_status leco_deserialize(const void* host_buf, uint64_t bytes, leco_stream_t
     if (s == LECO_OK)
       s = from_cuda(cudaMemcpyAsync(d_pcoef, pcoef.data(), sizeof(PolyCoef) * pcoef.size(), cudaMemcpyHostToDevice, st));
   }
-  if (s == LECO_OK) s = from_cuda(launch_build_aux(c->rec, d_pcoef, c->m, c->n, c->aux, c->poly, c->status, st));
+  if (s == LECO_OK) s = from_cuda(launch_build_aux(c->rec, d_pcoef, c->m, c->n, c->aux, c->poly, 0, nullptr, 0, c->status, st));
   if (s == LECO_OK) s = from_cuda(launch_tile_desc(view_of(c), c->tiles, st));
   if (d_pcoef) cudaFreeAsync(d_pcoef, st);
   // the host vectors die at return: finish the copies first

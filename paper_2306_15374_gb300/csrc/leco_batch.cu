@@ -470,10 +470,7 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   if (e == cudaSuccess) e = launch_offsets_multi(p.rec, p.lenbits, d_part, p.part_col, ncols, P, p.offs, p.colbits, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(col_bits.data(), p.colbits, 8 * ncols, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(max_b.data(), p.maxb, 4 * ncols, cudaMemcpyDeviceToHost, st);
-  uint32_t fit_flags = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&fit_flags, p.status, 4, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess && (fit_flags & kStatTimeout)) e = cudaErrorTimeout;  // a staging copy never landed
   if (e == cudaSuccess) {
     word_base[0] = 0;
     for (uint32_t c = 0; c < ncols; c++) {
@@ -486,11 +483,11 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_word, word_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, st);
   const std::vector<ColumnView> views = enc_views(B, p, n, L);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_views, views.data(), sizeof(ColumnView) * ncols, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, d_ec, d_part, p.part_col, P, p.aux, p.poly, st);
+  if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, d_ec, d_part, p.part_col, d_word, p.colbits, ncols, P, p.aux, p.poly, words, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(d_views, d_tile, ncols, T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(d_ec, d_part, d_tile, p.part_col, d_word, p.colbits, ncols, P, T, W, dtype, cfg.item_values,
-                          p.rec, p.aux, p.pcoef, p.poly, words, st);
+    e = launch_pack_multi(d_ec, d_part, d_tile, d_word, ncols, T, dtype, cfg.item_values, p.rec, p.aux, p.pcoef, p.poly,
+                          words, st);
   if (e == cudaSuccess) e = make_batch_columns(B, p, words, word_base, col_bits, max_b, models, L, dev, st, meta, out);
   cudaFreeAsync(scr, st);
   cudaFreeAsync(d_ec, st);
@@ -560,11 +557,11 @@ cudaError_t enc_plan_launches(leco_batch_encode_plan* pl, cudaStream_t st) {
   if (e == cudaSuccess)
     e = launch_offsets_multi(p.rec, p.lenbits, d_part, p.part_col, B.ncols, B.P, p.offs, p.colbits, st);
   if (e == cudaSuccess) e = launch_word_bases(p.colbits, B.ncols, d_word, st);
-  if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, pl->d_ec, d_part, p.part_col, B.P, p.aux, p.poly, st);
+  if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, pl->d_ec, d_part, p.part_col, d_word, p.colbits, B.ncols, B.P, p.aux, p.poly, pl->words, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(pl->d_views, d_tile, B.ncols, B.T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(pl->d_ec, d_part, d_tile, p.part_col, d_word, p.colbits, B.ncols, B.P, B.T, pl->words_cap,
-                          B.dtype, pl->cfg.item_values, p.rec, p.aux, p.pcoef, p.poly, pl->words, st);
+    e = launch_pack_multi(pl->d_ec, d_part, d_tile, d_word, B.ncols, B.T, B.dtype, pl->cfg.item_values, p.rec, p.aux,
+                          p.pcoef, p.poly, pl->words, st);
   return e;
 }
 
@@ -716,14 +713,11 @@ extern "C" leco_status leco_batch_encode_plan_columns(leco_batch_encode_plan* pl
   cudaStream_t st = (cudaStream_t)stream;
   const EncPtrs p = enc_ptrs(B, plan->meta, plan->scr);
   std::vector<uint64_t> col_bits(ncols), word_base(ncols + 1);
-  std::vector<uint32_t> max_b(ncols), flags(ncols);
+  std::vector<uint32_t> max_b(ncols);
   cudaError_t e = cudaMemcpyAsync(col_bits.data(), p.colbits, 8 * ncols, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(max_b.data(), p.maxb, 4 * ncols, cudaMemcpyDeviceToHost, st);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(flags.data(), p.status, 4 * ncols, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return from_cuda(e);
-  for (uint32_t c = 0; c < ncols; c++)
-    if (flags[c] & kStatTimeout) return LECO_ERR_TIMEOUT;  // a staging copy never landed: streams incomplete
   word_base[0] = 0;
   for (uint32_t c = 0; c < ncols; c++) word_base[c + 1] = word_base[c] + stream_words(col_bits[c]);
   const uint64_t W = word_base[ncols];

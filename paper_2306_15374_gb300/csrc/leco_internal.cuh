@@ -297,15 +297,16 @@ uint64_t offsets_multi_scratch_elems(uint64_t P);
 cudaError_t launch_offsets_multi(Record* rec, const uint64_t* lenbits, const uint64_t* part_base,
                                  const uint32_t* part_col, uint32_t ncols, uint64_t P, uint64_t* scratch,
                                  uint64_t* col_bits, cudaStream_t st);
+// the decode tables, and zeroes in the words that packing OR-s into
 cudaError_t launch_aux_multi(const Record* rec, const PolyCoef* pcoef, const EncCol* cols, const uint64_t* part_base,
-                             const uint32_t* part_col, uint64_t P, Aux* aux, PolyAux* poly, cudaStream_t st);
+                             const uint32_t* part_col, const uint64_t* word_base, const uint64_t* col_bits,
+                             uint32_t ncols, uint64_t P, Aux* aux, PolyAux* poly, uint64_t* words, cudaStream_t st);
 // word_base[c] = sum of stream_words(col_bits[k]) over k < c, for c = 0 .. ncols, on the device (one
 // CTA): each column's packed stream placed right after the previous one
 cudaError_t launch_word_bases(const uint64_t* col_bits, uint32_t ncols, uint64_t* word_base, cudaStream_t st);
 // window: positions a warp packs (1024, 2048 or 4096); tiles: scan tiles of all columns
 cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* tile_base,
-                              const uint32_t* part_col, const uint64_t* word_base, const uint64_t* col_bits,
-                              uint32_t ncols, uint64_t P, uint64_t tiles, uint64_t W, int dtype, uint32_t window,
+                              const uint64_t* word_base, uint32_t ncols, uint64_t tiles, int dtype, uint32_t window,
                               const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                               uint64_t* words, cudaStream_t st);
 // poly: some column has a polynomial table (its tiles then get the exact polynomial bounds)
@@ -349,12 +350,14 @@ cudaError_t launch_fit(const void* values, int dtype, uint64_t n, const uint64_t
 cudaError_t launch_offsets(Record* rec, const uint64_t* lenbits, uint64_t m, uint64_t* scratch,
                            uint64_t scratch_elems, uint64_t* total_out, cudaStream_t st);
 uint64_t offsets_scratch_elems(uint64_t m);
+// words (nullptr: a stream that exists already): the words that packing OR-s into are zeroed; *status is cleared
 cudaError_t launch_build_aux(const Record* rec, const PolyCoef* pcoef, uint64_t m, uint64_t n, Aux* aux,
-                             PolyAux* poly, uint32_t* status, cudaStream_t st);
+                             PolyAux* poly, uint64_t total_bits, uint64_t* words, uint64_t nwords, uint32_t* status,
+                             cudaStream_t st);
 // L: the fixed partition length, or 0 with the column's tile descriptors for partitions of any lengths
 cudaError_t launch_pack(const void* values, int dtype, uint32_t L, const TileDesc* tiles, const Record* rec,
                         const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly, uint64_t m, uint64_t n,
-                        uint64_t total_bits, uint64_t* words, uint64_t nwords, cudaStream_t st);
+                        uint64_t* words, cudaStream_t st);
 
 // scans (k_scan.cu) and lookups (k_decode.cu)
 cudaError_t launch_tile_desc(const ColumnView& c, TileDesc* tiles, cudaStream_t st);
