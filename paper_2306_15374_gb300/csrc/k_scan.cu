@@ -15,6 +15,8 @@
 // Tile descriptors (word range, partitions, value bounds) are built once per column.
 #include <string.h>
 
+#include <atomic>
+
 #include "leco_internal.cuh"
 #include "tma.cuh"
 
@@ -826,18 +828,50 @@ __global__ void k_tile_desc_multi(const ColumnView* __restrict__ views, const ui
   }
 }
 
+// the jobs of a whole-column batch decode, one per scan tile of every column (tile_base[c] tiles before
+// column c)
+__global__ void k_batch_items(const ColumnView* __restrict__ views, void* const* __restrict__ outs,
+                              const uint64_t* __restrict__ tile_base, uint32_t ncols, uint64_t nitems,
+                              BatchItem* __restrict__ items) {
+  for (uint64_t g = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; g < nitems; g += (uint64_t)gridDim.x * blockDim.x) {
+    const uint32_t c = find_col(tile_base, ncols, g);
+    const uint64_t n = views[c].n;
+    BatchItem it;
+    it.col = c;
+    it.pad = 0;
+    it.tile = g - tile_base[c];
+    it.begin = it.tile * kScanTile;
+    it.end = min(it.begin + kScanTile, n);
+    it.out = static_cast<char*>(outs[c]) + it.begin * (views[c].dtype == LECO_U32 ? 4 : 8);
+    items[g] = it;
+  }
+}
+
 template <int MODE, int CW, bool MULTI, bool POLY, bool TAIL>
 cudaError_t launch_scan_cfg(const ScanArgs& g, const ColumnView* cols, const BatchItem* items,
                             uint64_t nitems, uint32_t stage_bytes, ScanConfig cfg, cudaStream_t st) {
   const uint32_t nst = cfg.stages < 2 ? 2u : (cfg.stages > (uint32_t)kMaxStages ? (uint32_t)kMaxStages : cfg.stages);
   const uint32_t smem = kCtrlBytes + nst * (stage_bytes + kAuxBytes);
   auto kern = k_tilescan<MODE, CW, MULTI, POLY, TAIL>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // CTAs per SM of this kernel at this stage size, asked once per device (the two driver calls cost more
+  // than the launch); the shared memory limit is raised to the device's own, once, so that no call can lower
+  // another's
+  static std::atomic<uint64_t> resident[64];  // (smem << 8 | CTAs), one size per device at a time
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  int nb = 0;
-  e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, (CW + 1) * 32, smem);
-  if (e != cudaSuccess) return e;
-  if (nb < 1) return cudaErrorInvalidConfiguration;
+  const uint64_t seen = dev < 64 ? resident[dev].load(std::memory_order_relaxed) : 0;
+  int nb = (int)(seen & 0xFFu);
+  if (nb == 0 || (seen >> 8) != smem) {
+    int most = 0;
+    e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess && smem > (uint32_t)most) return cudaErrorInvalidValue;
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, (CW + 1) * 32, smem);
+    if (e != cudaSuccess) return e;
+    if (nb < 1) return cudaErrorInvalidConfiguration;
+    if (dev < 64) resident[dev].store((uint64_t)smem << 8 | (uint64_t)nb, std::memory_order_relaxed);
+  }
   const uint64_t njobs = MULTI ? nitems : g.t_last - g.t_first + 1;
   const uint64_t cap = (uint64_t)sm_count() * nb;
   const unsigned grid = (unsigned)(njobs < cap ? njobs : cap);
@@ -955,6 +989,14 @@ cudaError_t launch_filter_sum_cfg(const ColumnView& c, uint64_t lo, uint64_t hi,
   g.flags = flags;
   g.res = out;
   return launch_scan<kFilter, false>(g, nullptr, nullptr, 0, c.stage_bytes, cfg, c.poly != nullptr, st);
+}
+
+cudaError_t launch_batch_items(const ColumnView* d_cols, void* const* d_outs, const uint64_t* d_tile_base,
+                               uint32_t ncols, uint64_t nitems, BatchItem* items, cudaStream_t st) {
+  if (nitems == 0) return cudaSuccess;
+  const uint64_t need = (nitems + 255) / 256, cap = (uint64_t)sm_count() * 8;
+  k_batch_items<<<(unsigned)(need < cap ? need : cap), 256, 0, st>>>(d_cols, d_outs, d_tile_base, ncols, nitems, items);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_batch_decode(const ColumnView* d_cols, const BatchItem* d_items, uint64_t nitems,

@@ -14,6 +14,7 @@ int tune_table_load(const char* path);
 }  // namespace leco
 
 struct leco_batch_plan {
+  void* table = nullptr;  // columns | outputs | first tile of each column | jobs | status word
   ColumnView* d_cols = nullptr;
   BatchItem* d_items = nullptr;
   uint32_t* d_status = nullptr;
@@ -34,10 +35,50 @@ void plan_release(leco_batch_plan* p) {
   if (p->exec) cudaGraphExecDestroy(p->exec);
   if (p->graph) cudaGraphDestroy(p->graph);
   if (p->capture) cudaStreamDestroy(p->capture);
-  if (p->d_cols) cudaFree(p->d_cols);
-  if (p->d_items) cudaFree(p->d_items);
-  if (p->d_status) cudaFree(p->d_status);
+  if (p->table) cudaFree(p->table);
   delete p;
+}
+
+// A plan's table on stream st: the columns go up in one copy, the jobs (one per scan tile) are written on the
+// device. pooled: from the library pool (freed by the caller in stream order), else a plain allocation.
+leco_status plan_build(leco_batch_plan* p, const leco_column* const* cols, void* const* d_outs, uint32_t ncols,
+                       bool pooled, cudaStream_t st) {
+  if (cudaGetDevice(&p->device) != cudaSuccess) return LECO_ERR_CUDA;
+  int dtype = LECO_U32;
+  auto a256 = [](uint64_t x) { return (x + 255) & ~255ull; };
+  const uint64_t outs_at = a256(sizeof(ColumnView) * ncols), base_at = outs_at + a256(sizeof(void*) * ncols);
+  std::vector<char> up(base_at + 8 * ((uint64_t)ncols + 1));
+  ColumnView* views = reinterpret_cast<ColumnView*>(up.data());
+  void** outs = reinterpret_cast<void**>(up.data() + outs_at);
+  uint64_t* tile_base = reinterpret_cast<uint64_t*>(up.data() + base_at);
+  uint64_t tiles = 0;
+  for (uint32_t c = 0; c < ncols; c++) {
+    const leco_column* col = cols[c];
+    if (!col || col->device != p->device || (col->n && !d_outs[c])) return LECO_ERR_INVALID_ARG;
+    views[c] = view_of(col);
+    outs[c] = d_outs[c];
+    tile_base[c] = tiles;
+    tiles += scan_tiles(col->n);
+    p->poly = p->poly || col->poly != nullptr;
+    p->stage_bytes = col->stage_bytes > p->stage_bytes ? col->stage_bytes : p->stage_bytes;
+    if (col->dtype == LECO_U64) dtype = LECO_U64;
+  }
+  tile_base[ncols] = tiles;
+  p->nitems = tiles;
+  p->cfg = scan_config_lookup(0, dtype, p->stage_bytes);
+  const uint64_t items_at = a256(up.size()), status_at = items_at + a256(sizeof(BatchItem) * tiles);
+  cudaError_t e = pooled ? dev_alloc(&p->table, status_at + 256, st) : cudaMalloc(&p->table, status_at + 256);
+  if (e != cudaSuccess) return from_cuda(e);
+  char* t = static_cast<char*>(p->table);
+  p->d_cols = reinterpret_cast<ColumnView*>(t);
+  p->d_items = reinterpret_cast<BatchItem*>(t + items_at);
+  p->d_status = reinterpret_cast<uint32_t*>(t + status_at);
+  e = cudaMemcpyAsync(t, up.data(), up.size(), cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(p->d_status, 0, 256, st);
+  if (e == cudaSuccess)
+    e = launch_batch_items(p->d_cols, reinterpret_cast<void* const*>(t + outs_at),
+                           reinterpret_cast<const uint64_t*>(t + base_at), ncols, tiles, p->d_items, st);
+  return from_cuda(e);
 }
 
 }  // namespace
@@ -115,55 +156,15 @@ leco_status leco_batch_plan_create(const leco_column* const* cols, void* const* 
                                    leco_batch_plan** out) {
   if (!out || (ncols && (!cols || !d_outs))) return LECO_ERR_INVALID_ARG;
   *out = nullptr;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return LECO_ERR_CUDA;
-  std::vector<ColumnView> views(ncols);
-  std::vector<BatchItem> items;
-  uint32_t stage_bytes = 64;
-  int dtype = LECO_U32;
-  bool any_poly = false;
-  for (uint32_t c = 0; c < ncols; c++) {
-    const leco_column* col = cols[c];
-    if (!col || col->device != dev || (col->n && !d_outs[c])) return LECO_ERR_INVALID_ARG;
-    views[c] = view_of(col);
-    any_poly = any_poly || col->poly != nullptr;
-    stage_bytes = col->stage_bytes > stage_bytes ? col->stage_bytes : stage_bytes;
-    if (col->dtype == LECO_U64) dtype = LECO_U64;
-    const uint64_t vb = col->dtype == LECO_U32 ? 4 : 8;
-    const uint64_t nt = scan_tiles(col->n);
-    for (uint64_t t = 0; t < nt; t++) {
-      BatchItem it;
-      it.col = c;
-      it.pad = 0;
-      it.tile = t;
-      it.begin = t * kScanTile;
-      it.end = it.begin + kScanTile < col->n ? it.begin + kScanTile : col->n;
-      it.out = static_cast<char*>(d_outs[c]) + it.begin * vb;
-      items.push_back(it);
-    }
-  }
   leco_batch_plan* p = new (std::nothrow) leco_batch_plan();
   if (!p) return LECO_ERR_OOM;
-  p->device = dev;
-  p->nitems = items.size();
-  p->stage_bytes = stage_bytes;
-  p->poly = any_poly;
-  p->cfg = scan_config_lookup(0, dtype, stage_bytes);
-  cudaError_t e = cudaMalloc((void**)&p->d_cols, sizeof(ColumnView) * (ncols ? ncols : 1));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_items, sizeof(BatchItem) * (items.empty() ? 1 : items.size()));
-  if (e == cudaSuccess) e = cudaMalloc((void**)&p->d_status, 256);
-  if (e == cudaSuccess) e = cudaMemset(p->d_status, 0, 256);
-  if (e == cudaSuccess && ncols)
-    e = cudaMemcpy(p->d_cols, views.data(), sizeof(ColumnView) * ncols, cudaMemcpyHostToDevice);
-  if (e == cudaSuccess && !items.empty())
-    e = cudaMemcpy(p->d_items, items.data(), sizeof(BatchItem) * items.size(), cudaMemcpyHostToDevice);
-  // the memset and the copies from pageable memory ran on the legacy stream, and a copy may return
-  // before its DMA lands: wait for them, so a run on any stream (non-blocking ones included) finds
-  // the tables in place
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
-  if (e != cudaSuccess) {
+  leco_status s = plan_build(p, cols, d_outs, ncols, false, cudaStreamLegacy);
+  // the copies from pageable memory, the job kernel and the status clear ran on the legacy stream: wait for
+  // them, so a run on any stream (non-blocking ones included) finds the tables in place
+  if (s == LECO_OK) s = from_cuda(cudaStreamSynchronize(cudaStreamLegacy));
+  if (s != LECO_OK) {
     plan_release(p);
-    return from_cuda(e);
+    return s;
   }
   *out = p;
   return LECO_OK;
@@ -273,13 +274,24 @@ void leco_batch_plan_free(leco_batch_plan* plan) {
 
 leco_status leco_batch_decode(const leco_column* const* cols, void* const* d_outs, uint32_t ncols,
                               leco_stream_t stream) {
-  leco_batch_plan* p = nullptr;
-  leco_status s = leco_batch_plan_create(cols, d_outs, ncols, &p);
-  if (s != LECO_OK) return s;
-  s = leco_batch_plan_run(p, stream);
-  const cudaError_t e = cudaStreamSynchronize((cudaStream_t)stream);
-  plan_release(p);
+  if (ncols && (!cols || !d_outs)) return LECO_ERR_INVALID_ARG;
+  // one run: the table from the library pool, filled on the legacy stream (behind the work of every
+  // blocking stream, as a plan's creation is), which `stream` then waits for
+  leco_batch_plan p;
+  cudaEvent_t ready = nullptr;
+  cudaStream_t st = (cudaStream_t)stream;
+  leco_status s = plan_build(&p, cols, d_outs, ncols, true, cudaStreamLegacy);
+  if (s == LECO_OK) {
+    cudaError_t e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ready, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ready, 0);
+    s = from_cuda(e);
+  }
+  if (s == LECO_OK) s = leco_batch_plan_run(&p, stream);
+  const cudaError_t e = cudaStreamSynchronize(st);
   if (s == LECO_OK && e != cudaSuccess) s = LECO_ERR_CUDA;
+  if (p.table) cudaFreeAsync(p.table, cudaStreamLegacy);
+  if (ready) cudaEventDestroy(ready);
   return s;
 }
 

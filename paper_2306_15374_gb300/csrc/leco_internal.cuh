@@ -372,6 +372,9 @@ cudaError_t launch_decode_cfg(const ColumnView& c, uint64_t begin, uint64_t coun
                               ScanConfig cfg, cudaStream_t st);
 cudaError_t launch_lookup_multi(const ColumnView* views, const uint32_t* col, const uint64_t* idx, uint64_t k,
                                 uint64_t* out, cudaStream_t st);
+// items[g]: scan tile g of the batch's columns, whole (d_tile_base: ncols + 1 entries, the last nitems)
+cudaError_t launch_batch_items(const ColumnView* d_cols, void* const* d_outs, const uint64_t* d_tile_base,
+                               uint32_t ncols, uint64_t nitems, BatchItem* items, cudaStream_t st);
 // poly: some column of the batch may hold polynomial partitions (a column with a polynomial table)
 cudaError_t launch_batch_decode(const ColumnView* d_cols, const BatchItem* d_items, uint64_t nitems,
                                 uint32_t stage_bytes, ScanConfig cfg, bool poly, uint32_t* status, cudaStream_t st);
