@@ -74,11 +74,11 @@ constexpr uint64_t kScanTile = 4096;
 
 struct TileDesc {
   uint64_t p0;      // first partition touching the tile
+  uint32_t np;      // partitions touching the tile (beside p0: a lookup reads both in one load)
+  uint32_t wbytes;  // bytes of the staged word range (multiple of 16)
   uint64_t g0;      // byte offset of the staged word range in the residual stream (16-aligned)
   uint64_t vmin;    // bounds == 1: every value of the tile lies in [vmin, vmax] (unsigned);
   uint64_t vmax;    // bounds == 2: in [0, vmax] or [vmin, 2^64 - 1] (vmax < vmin); 0: unknown
-  uint32_t np;      // partitions touching the tile
-  uint32_t wbytes;  // bytes of the staged word range (multiple of 16)
   uint32_t bounds;
   uint32_t pad;
 };
@@ -134,7 +134,7 @@ __device__ __forceinline__ uint64_t read_field(const uint64_t* __restrict__ word
   const uint64_t w = pos >> 6;
   const uint32_t o = (uint32_t)pos & 63u;
   const uint64_t lo = __ldg(words + w);
-  const uint64_t hi = __ldg(words + w + 1);
+  const uint64_t hi = o + b > 64 ? __ldg(words + w + 1) : 0;  // most narrow fields lie in one word
   // (hi << 1) << (63 - o) is hi << (64 - o) without the undefined shift by 64 when o == 0
   return ((lo >> o) | ((hi << 1) << (63 - o))) & low_mask(b);
 }
