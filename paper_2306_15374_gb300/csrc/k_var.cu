@@ -1007,29 +1007,33 @@ __device__ __forceinline__ void job_range(const T* __restrict__ p, const SpanJob
     const NarrowLine line(q.B, q.s);
     const uint32_t ref = x0 < x1 ? (uint32_t)__ldg(p) : 0u;
     int32_t l = INT32_MAX, h = INT32_MIN;
-    auto pass = [&](uint32_t xa, uint32_t xb, uint32_t step) {
-      uint64_t G = line.B * xa;
-      const uint64_t dG = line.B * (uint64_t)step;
-#pragma unroll 4
-      for (uint32_t x = xa; x < xb; x += step, G += dG) {
-        const int32_t e = (int32_t)((uint32_t)__ldg(p + x) - ref) - line.at(G);
-        l = min(l, e);
-        h = max(h, e);
-      }
+    // values xa + r, + TILE, ... < xb, eight loads in flight per lane
+    auto pass = [&](uint32_t xa, uint32_t xb) {
+      uint64_t G = line.B * (xa + r);
+      const uint64_t dG = line.B * (uint64_t)TILE;
+      for_runs<TILE, 8>(
+          p + xa, xb - xa, r, (T)0,
+          [&](T value) {
+            const int32_t e = (int32_t)((uint32_t)value - ref) - line.at(G);
+            l = min(l, e);
+            h = max(h, e);
+            G += dG;
+          },
+          []() { return true; });
     };
     if (CHECK && q.bmax < 31) {
       bool over = false;
       if (x1 - x0 >= 1024) {
         const uint32_t x = x0 + r * ((x1 - x0) >> 5);
-        pass(x, x + 1, 1);
+        l = h = (int32_t)((uint32_t)__ldg(p + x) - ref) - line.at(line.B * x);
         over = ((uint32_t)tile_max<TILE>(h) - (uint32_t)tile_min<TILE>(l)) >> q.bmax != 0;
       }
       for (uint32_t x = x0; x < x1 && !over; x += 1024) {
-        pass(x + r, min(x + 1024u, x1), TILE);
+        pass(x, min(x + 1024u, x1));
         if (x + 1024 < x1) over = __any_sync(kFull, l <= h && ((uint32_t)h - (uint32_t)l) >> q.bmax != 0);
       }
     } else {
-      pass(x0 + r, x1, TILE);
+      pass(x0, x1);
     }
     // 32-bit differences from the span's first value: whole again by its 64 bits
     const int64_t ref64 = x0 < x1 ? (int64_t)__ldg(p) : 0;
