@@ -78,10 +78,9 @@ def parse_args():
 KSCAN_SRCS = [os.path.join(ROOT, "paper_2306_15374_gb300", "csrc", f) for f in ("k_scan.cu", "leco_internal.cuh", "tma.cuh")]
 # DRAM read + write per decode launch from one ncu capture of this workload (mean of columns a, b, c;
 # see profiles/k_tilescan_decode_filter_fix200M.md), valid only for the kernel sources it was taken on
-# (keyed by their hash; re-keyed once since, when the shared header gained only host declarations of
-# the batched-encode launchers and the decode kernel's code stayed the same).
-DECODE_TRAFFIC = {"sha256": "1e091f3002cd25780c164ad5dc869ef8ca403b716143b0ec0422a72376811554",
-                  "bytes_per_launch": (1894286848 + 1973986048 + 1846223104) / 3}
+# (keyed by their hash).
+DECODE_TRAFFIC = {"sha256": "89f00e7413beb6f3eb0d3adc82aae7e2c0b3ba981762c990f227bec8c9b47259",
+                  "bytes_per_launch": (1893644544 + 1973048320 + 1845314816) / 3}
 
 
 def decode_traffic():
