@@ -441,7 +441,7 @@ __global__ void k_build_aux(const Record* __restrict__ rec, const PolyCoef* __re
 // or 80 registers were slower). Measured, former -> this: 200M sorted normal uint64 in partitions of 4096
 // 431 -> 351 us (5.7 TB/s), 250M 32-bit timestamps in variable partitions 1295 -> 531 us, 100M piecewise
 // values 2.39 -> 0.9 ms, 96 columns of 200M values in partitions of 256 .. 4096 492 -> 431 us, 20M 32-bit
-// values in partitions of 1000 83 -> 60 us.
+// values in partitions of 1000 83 -> 44 us.
 constexpr int kPackBlock = 256;
 constexpr int kPackWarps = kPackBlock / 32;
 constexpr int kPackCtas = 4;  // CTAs per SM the registers are held for
@@ -761,17 +761,21 @@ __device__ __forceinline__ void pack_window(const T* __restrict__ values, uint64
   }
 }
 
-// L: the fixed partition length, or 0: partitions of any lengths, found through the scan tiles
+// L: the fixed partition length, or 0: partitions of any lengths, found through the scan tiles. Every `period`
+// positions hold `per` windows, the last one shorter where they do not divide it.
 template <typename T, bool POLY>
 __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
-    k_pack(const T* __restrict__ values, uint64_t n, uint64_t m, uint32_t L, uint32_t window,
-           const TileDesc* __restrict__ tiles, const Record* __restrict__ rec, const Aux* __restrict__ aux,
-           const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly, uint32_t* __restrict__ words) {
+    k_pack(const T* __restrict__ values, uint64_t n, uint64_t m, uint32_t L, uint32_t window, uint32_t period,
+           uint32_t per, const TileDesc* __restrict__ tiles, const Record* __restrict__ rec,
+           const Aux* __restrict__ aux, const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly,
+           uint32_t* __restrict__ words) {
   __shared__ uint64_t zbuf[kPackWarps][kPackTile / 2];
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  const uint64_t nwin = (n + window - 1) / window, nw = (uint64_t)gridDim.x * kPackWarps;
+  const uint64_t nwin = (n + period - 1) / period * per, nw = (uint64_t)gridDim.x * kPackWarps;
   for (uint64_t k = (uint64_t)blockIdx.x * kPackWarps + wid; k < nwin; k += nw) {
-    const uint64_t pos = k * window, end = min(pos + window, n);
+    const uint64_t q = per == 1 ? k : k / per, from = q * period, pos = from + (k - q * per) * window;
+    const uint64_t end = min(min(pos + window, from + period), n);
+    if (pos >= end) continue;  // past the last partition's end
     uint64_t p;
     if (L) {
       p = pos / L;
@@ -1069,9 +1073,20 @@ cudaError_t launch_pack_t(const void* values, uint64_t n, uint64_t m, uint32_t L
   // (which cut most partitions) and 531 us with 4096; columns below 5M values come down to 256.
   uint32_t window = kPackWindow;
   while (window > kPackWindowMin && n / window < (uint64_t)sm_count() * 128) window /= 2;
-  const uint64_t nwin = (n + window - 1) / window;
+  // Fixed partitions: whole ones to a window, or a partition's windows from its start on, so that none is cut
+  // where it need not be. Whole encodes, windows at any position -> this: 20M values in partitions of 1000 / 1500
+  // / 2047 / 3000 159 / 180 / 160 / 151 -> 142 / 167 / 151 / 145 us, 150M of 1000 / 1500 563 / 760 -> 520 / 704.
+  uint32_t period = window, per = 1;
+  if (L && L <= window) {
+    period = window -= window % L;
+  } else if (L) {
+    period = (uint32_t)min((uint64_t)L, n);
+    per = (uint32_t)(((uint64_t)period + window - 1) / window);
+  }
+  const uint64_t nwin = (n + period - 1) / period * per;
   k_pack<T, POLY><<<grid_for(nwin, kPackWarps, 8), kPackBlock, 0, st>>>(
-      static_cast<const T*>(values), n, m, L, window, tiles, rec, aux, pcoef, poly, reinterpret_cast<uint32_t*>(words));
+      static_cast<const T*>(values), n, m, L, window, period, per, tiles, rec, aux, pcoef, poly,
+      reinterpret_cast<uint32_t*>(words));
   return cudaGetLastError();
 }
 

@@ -81,3 +81,11 @@ def test_batch_of_windows(lc):
     Ls, models = [1, 256, 1000, 4096, 64, 10_000], [0, 1, 2, 1, 2, 1]
     for col, v, L, model in zip(lc.leco_batch_encode([to_dev(v) for v in vals], models, Ls), vals, Ls, models):
         _check(lc, col, v, L, model)
+
+
+@pytest.mark.parametrize("L", [1, 255, 257, 511, 513, 1000, 1023, 1025, 1500, 2047, 2049, 1_000_003, 9_961_473, 1 << 24])
+def test_windows_of_whole_partitions(lc, L):
+    # windows of 256 and of 1024 positions, cut to whole partitions or a part of one
+    for n in (9_961_473, 20_000_003) if L == 1000 else (9_961_473,):
+        v = W.linear_noise(n, 1 << 20, 3, 700, seed=43)
+        _check(lc, lc.leco_encode(to_dev(v, 32), lc.fixed(L), 1), v, L, 1)
