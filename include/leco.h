@@ -182,9 +182,9 @@ leco_status leco_encode_with_starts(const void* d_values, uint64_t n, leco_dtype
  * the caller's own pool reserves the device's memory. All calls on a device share the array, so
  * calls whose GPU work overlaps (e.g. on different streams) race; nothing of it needs clearing
  * between calls. The call synchronizes `stream` twice: once to size the stream, and once at the
- * end, so that the buffers are complete when it returns. INVALID_ARG when words_cap < *nwords_out (nothing packed then) or for
- * LECO_MODEL_POLY (constant and linear only), CUDA on a runtime failure. No cudaMalloc, cudaFree
- * or allocating library routine is called. */
+ * end, so that the buffers are complete when it returns. INVALID_ARG when words_cap < *nwords_out
+ * (nothing packed then) or for LECO_MODEL_POLY (constant and linear only), CUDA on a runtime
+ * failure. No cudaMalloc, cudaFree or allocating library routine is called. */
 leco_status leco_encode_fixed_noalloc(const void* d_values, uint64_t n, leco_dtype dtype, uint32_t L,
                                       leco_model model, void* d_records, void* d_words,
                                       uint64_t words_cap, uint64_t* nwords_out,
