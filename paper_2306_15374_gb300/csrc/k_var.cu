@@ -605,7 +605,8 @@ int grid_for(uint64_t items, int per_block, int max_blocks_per_sm) {
 // only the pairs that can merge and those that changed.
 // Measured, 100M piecewise uint64 (45 rounds) and 250M 32-bit timestamps (62 rounds), against 16-byte sizes
 // and 48-byte moments moved every round, one kernel of 78 registers for fits of all lengths, and ten
-// launches and a host round trip per round to the end: whole passes 28.05 -> 20.46 ms and 18.37 -> 11.59 ms.
+// launches and a host round trip per round to the end: whole passes 28.05 -> 20.46 ms and 18.37 -> 11.59 ms
+// (17.7 and 10.3 ms with what the kernels below say of themselves).
 constexpr uint32_t kTinySpan = 256;    // size search: a thread per sampled partition up to this size
 constexpr uint32_t kLaneVals = 64;     // a lane fits spans up to this long on its own
 constexpr uint32_t kStatVals = 32;     // longer partitions carry their moments (at most kLaneVals; the table's stride)
@@ -1141,25 +1142,42 @@ __global__ void __launch_bounds__(256)
   // [i] belongs to pair base - 1 + i. A pair's gain fits 32 bits (at most 2^24 values of 64 bits); kLoses:
   // it does not merge. Gains tie in most pairs of the first rounds, so each pair's hash is taken once too.
   constexpr int32_t kLoses = INT32_MIN;
-  __shared__ uint64_t s_st[kMergeTile + 2], s_hash[kMergeTile + 2];
+  __shared__ uint64_t s_st[kMergeTile + 4], s_hash[kMergeTile + 2];
   __shared__ int32_t s_gain[kMergeTile + 2];
+  __shared__ uint8_t s_b[kMergeTile + 4];
   __shared__ uint32_t ws[8];
   const uint64_t base = (uint64_t)blockIdx.x * kMergeTile;
-  for (uint32_t i = threadIdx.x; i < kMergeTile + 2; i += 256) {
-    const int64_t p = (int64_t)(base + i) - 1;
-    int32_t g = kLoses;
-    uint64_t a = 0;
-    if (p >= 0 && (uint64_t)p + 1 < m) {
-      const uint32_t w = mb[p];
-      a = st[p];
-      if (w <= 64) {
-        const uint64_t mid = st[p + 1];
-        g = (int32_t)gain_of(mid - a, b[p], st[p + 2] - mid, b[p + 1], w);
-      }
+  // all of the tile's loads at once, whether or not a pair turns out to gain, against a
+  // chain of loads per pair: 1016 -> 778 us over the rounds of 100M piecewise values (the encode 18.1 -> 17.9 ms)
+  constexpr int kPer = (kMergeTile + 4 + 255) / 256;
+  uint64_t s0[kPer];
+  uint8_t b0[kPer], w0[kPer];
+#pragma unroll
+  for (int k = 0; k < kPer; k++) {
+    const uint32_t i = threadIdx.x + 256u * k;
+    const uint64_t p = base + i - 1;  // wraps below 0: past every bound
+    const bool in = i < kMergeTile + 4;
+    s0[k] = in && p <= m ? st[p] : 0;
+    b0[k] = in && p < m ? b[p] : 0;
+    w0[k] = in && p < m && p + 1 < m ? mb[p] : kNo;
+  }
+#pragma unroll
+  for (int k = 0; k < kPer; k++) {
+    const uint32_t i = threadIdx.x + 256u * k;
+    if (i < kMergeTile + 4) {
+      s_st[i] = s0[k];
+      s_b[i] = b0[k];
     }
-    s_gain[i] = g;
-    s_st[i] = a;
-    s_hash[i] = splitmix64(a);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int k = 0; k < kPer; k++) {
+    const uint32_t i = threadIdx.x + 256u * k;
+    if (i < kMergeTile + 2) {
+      const uint64_t mid = s_st[i + 1];
+      s_gain[i] = w0[k] <= 64 ? (int32_t)gain_of(mid - s0[k], b0[k], s_st[i + 2] - mid, s_b[i + 1], w0[k]) : kLoses;
+      s_hash[i] = splitmix64(s0[k]);
+    }
   }
   __syncthreads();
   uint32_t local = 0;
