@@ -85,10 +85,21 @@ uint64_t leco_batch_plan_jobs(const leco_batch_plan* plan);
  * Batching layer; the paper has no counterpart. */
 void leco_batch_plan_free(leco_batch_plan* plan);
 
-/* The §3.3 Decoder over many columns in one call: create + run + free (synchronizes `stream`
- * before freeing). Arguments and errors as leco_batch_plan_create and leco_batch_plan_run. */
+/* The §3.3 Decoder over many columns in one call: create + run + sync + free (synchronizes
+ * `stream`). Arguments and errors as leco_batch_plan_create and leco_batch_plan_run, and the
+ * device-side errors of leco_batch_plan_sync: LECO_ERR_TIMEOUT when a bounded wait inside the
+ * decode gave up (the outputs are then incomplete). */
 leco_status leco_batch_decode(const leco_column* const* cols, void* const* d_outs, uint32_t ncols,
                               leco_stream_t stream);
+
+/* Failure-detection self-test of leco_batch_decode: the same call with, behind its decode, a
+ * bounded wait that nothing completes, limited to limit_us microseconds (1 .. 1000000), which
+ * records its giving up where the decode's own waits record theirs. Returns LECO_ERR_TIMEOUT when
+ * that was reported (the expected outcome: the device stays usable and the outputs are whole), else
+ * as leco_batch_decode; INVALID_ARG for a limit out of range. A systems facility; the paper has no
+ * counterpart. */
+leco_status leco_selftest_batch_decode_timeout(const leco_column* const* cols, void* const* d_outs, uint32_t ncols,
+                                               uint32_t limit_us, leco_stream_t stream);
 
 /* Fixed-partition encode of ncols columns at once (§3.2.1 partitions, §3.1 fit, §3.3 packing):
  * column c has n[c] values of `dtype` at d_vals[c] (device), model models[c] (constant, linear or

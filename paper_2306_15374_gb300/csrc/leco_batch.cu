@@ -81,6 +81,41 @@ leco_status plan_build(leco_batch_plan* p, const leco_column* const* cols, void*
   return from_cuda(e);
 }
 
+// the first device-side error a batched decode recorded in its status word
+leco_status decode_status(uint32_t flags) {
+  if (flags & kStatTimeout) return LECO_ERR_TIMEOUT;
+  if (flags & kStatCorrupt) return LECO_ERR_CORRUPT;
+  if (flags & kStatIndexRange) return LECO_ERR_INDEX_RANGE;
+  return LECO_OK;
+}
+
+// One run of a plan that nobody keeps: the table from the library pool, filled on the legacy stream (behind
+// the work of every blocking stream, as a plan's creation is), which st then waits for. The status word
+// goes with the table, so it is read here. wait_ns: a bounded wait that nothing completes runs behind the decode
+// and records its giving up in the same word (the self-test).
+leco_status decode_once(const leco_column* const* cols, void* const* d_outs, uint32_t ncols, uint64_t wait_ns,
+                        cudaStream_t st) {
+  leco_batch_plan p;
+  cudaEvent_t ready = nullptr;
+  uint32_t flags = 0;
+  leco_status s = plan_build(&p, cols, d_outs, ncols, true, cudaStreamLegacy);
+  if (s == LECO_OK) {
+    cudaError_t e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
+    if (e == cudaSuccess) e = cudaEventRecord(ready, cudaStreamLegacy);
+    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ready, 0);
+    if (e == cudaSuccess)
+      e = launch_batch_decode(p.d_cols, p.d_items, p.nitems, p.stage_bytes, p.cfg, p.poly, p.d_status, st);
+    if (e == cudaSuccess && wait_ns) e = launch_wait_selftest(wait_ns, p.d_status, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(&flags, p.d_status, 4, cudaMemcpyDeviceToHost, st);
+    s = from_cuda(e);
+  }
+  const cudaError_t e = cudaStreamSynchronize(st);
+  if (s == LECO_OK) s = e == cudaSuccess ? decode_status(flags) : LECO_ERR_CUDA;
+  if (p.table) cudaFreeAsync(p.table, cudaStreamLegacy);
+  if (ready) cudaEventDestroy(ready);
+  return s;
+}
+
 }  // namespace
 
 extern "C" {
@@ -258,10 +293,7 @@ leco_status leco_batch_plan_sync(leco_batch_plan* plan, leco_stream_t stream) {
   if (flags && (cudaMemsetAsync(plan->d_status, 0, 4, (cudaStream_t)stream) != cudaSuccess ||
                 cudaStreamSynchronize((cudaStream_t)stream) != cudaSuccess))
     return LECO_ERR_CUDA;
-  if (flags & kStatTimeout) return LECO_ERR_TIMEOUT;
-  if (flags & kStatCorrupt) return LECO_ERR_CORRUPT;
-  if (flags & kStatIndexRange) return LECO_ERR_INDEX_RANGE;
-  return LECO_OK;
+  return decode_status(flags);
 }
 
 uint64_t leco_batch_plan_jobs(const leco_batch_plan* plan) { return plan ? plan->nitems : 0; }
@@ -275,24 +307,13 @@ void leco_batch_plan_free(leco_batch_plan* plan) {
 leco_status leco_batch_decode(const leco_column* const* cols, void* const* d_outs, uint32_t ncols,
                               leco_stream_t stream) {
   if (ncols && (!cols || !d_outs)) return LECO_ERR_INVALID_ARG;
-  // one run: the table from the library pool, filled on the legacy stream (behind the work of every
-  // blocking stream, as a plan's creation is), which `stream` then waits for
-  leco_batch_plan p;
-  cudaEvent_t ready = nullptr;
-  cudaStream_t st = (cudaStream_t)stream;
-  leco_status s = plan_build(&p, cols, d_outs, ncols, true, cudaStreamLegacy);
-  if (s == LECO_OK) {
-    cudaError_t e = cudaEventCreateWithFlags(&ready, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventRecord(ready, cudaStreamLegacy);
-    if (e == cudaSuccess) e = cudaStreamWaitEvent(st, ready, 0);
-    s = from_cuda(e);
-  }
-  if (s == LECO_OK) s = leco_batch_plan_run(&p, stream);
-  const cudaError_t e = cudaStreamSynchronize(st);
-  if (s == LECO_OK && e != cudaSuccess) s = LECO_ERR_CUDA;
-  if (p.table) cudaFreeAsync(p.table, cudaStreamLegacy);
-  if (ready) cudaEventDestroy(ready);
-  return s;
+  return decode_once(cols, d_outs, ncols, 0, (cudaStream_t)stream);
+}
+
+leco_status leco_selftest_batch_decode_timeout(const leco_column* const* cols, void* const* d_outs, uint32_t ncols,
+                                               uint32_t limit_us, leco_stream_t stream) {
+  if ((ncols && (!cols || !d_outs)) || limit_us < 1 || limit_us > 1000000) return LECO_ERR_INVALID_ARG;
+  return decode_once(cols, d_outs, ncols, (uint64_t)limit_us * 1000ull, (cudaStream_t)stream);
 }
 
 }  // extern "C"

@@ -146,6 +146,7 @@ def lib() -> ctypes.CDLL:
         "leco_batch_plan_tune": (i32, [vp, vp, ctypes.POINTER(ScanConfig)]),
         "leco_batch_plan_free": (None, [vp]),
         "leco_batch_decode": (i32, [ctypes.POINTER(vp), ctypes.POINTER(vp), u32, vp]),
+        "leco_selftest_batch_decode_timeout": (i32, [ctypes.POINTER(vp), ctypes.POINTER(vp), u32, u32, vp]),
         "leco_batch_encode": (i32, [ctypes.POINTER(vp), ctypes.POINTER(u64), ctypes.POINTER(i32),
                                     ctypes.POINTER(u32), u32, i32, vp, ctypes.POINTER(vp)]),
         "leco_tune_batch_encode": (i32, [ctypes.POINTER(vp), ctypes.POINTER(u64), ctypes.POINTER(i32),
@@ -545,6 +546,14 @@ def leco_batch_plan_free(plan: BatchPlan) -> None:
 def leco_batch_decode(cols, outs, stream=None) -> None:
     _outs_room(cols, outs, "leco_batch_decode")
     _check(lib().leco_batch_decode(_handles(cols), _ptrs(outs), len(cols), _stream(stream)), "leco_batch_decode")
+
+
+def leco_selftest_batch_decode_timeout(cols, outs, limit_us: int, stream=None) -> int:
+    """A batched decode with a bounded wait that gives up behind it; returns the status (LECO_ERR_TIMEOUT is
+    the expected one)."""
+    _outs_room(cols, outs, "leco_selftest_batch_decode_timeout")
+    return int(lib().leco_selftest_batch_decode_timeout(_handles(cols), _ptrs(outs), len(cols), int(limit_us),
+                                                        _stream(stream)))
 
 
 class Server:
