@@ -15,8 +15,7 @@
 // Tile descriptors (word range, partitions, value bounds) are built once per column.
 #include <string.h>
 
-#include <atomic>
-
+#include "launch_shape.cuh"
 #include "leco_internal.cuh"
 #include "tma.cuh"
 
@@ -883,25 +882,21 @@ cudaError_t launch_scan_cfg(const ScanArgs& g, const ColumnView* cols, const Bat
   const uint32_t nst = cfg.stages < 2 ? 2u : (cfg.stages > (uint32_t)kMaxStages ? (uint32_t)kMaxStages : cfg.stages);
   const uint32_t smem = kCtrlBytes + nst * (stage_bytes + kAuxBytes);
   auto kern = k_tilescan<MODE, CW, MULTI, POLY, TAIL>;
-  // CTAs per SM of this kernel at this stage size, asked once per device (the two driver calls cost more
-  // than the launch); the shared memory limit is raised to the device's own, once, so that no call can lower
-  // another's
-  static std::atomic<uint64_t> resident[64];  // (smem << 8 | CTAs), one size per device at a time
+  // the shared memory limit is raised to the device's own, so that no call can lower another's
+  static ResidentCache resident;
   int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return e;
-  const uint64_t seen = dev < 64 ? resident[dev].load(std::memory_order_relaxed) : 0;
-  int nb = (int)(seen & 0xFFu);
-  if (nb == 0 || (seen >> 8) != smem) {
-    int most = 0;
+  const int nb = resident.get(dev, smem, [&]() {
+    int most = 0, n = 0;
     e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    if (e == cudaSuccess && smem > (uint32_t)most) return cudaErrorInvalidValue;
+    if (e == cudaSuccess && smem > (uint32_t)most) e = cudaErrorInvalidValue;
     if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, kern, (CW + 1) * 32, smem);
-    if (e != cudaSuccess) return e;
-    if (nb < 1) return cudaErrorInvalidConfiguration;
-    if (dev < 64) resident[dev].store((uint64_t)smem << 8 | (uint64_t)nb, std::memory_order_relaxed);
-  }
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, (CW + 1) * 32, smem);
+    return n;
+  });
+  if (e != cudaSuccess) return e;
+  if (nb < 1) return cudaErrorInvalidConfiguration;
   const uint64_t njobs = MULTI ? nitems : g.t_last - g.t_first + 1;
   const uint64_t cap = (uint64_t)sm_count() * nb;
   const unsigned grid = (unsigned)(njobs < cap ? njobs : cap);

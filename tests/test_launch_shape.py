@@ -1,0 +1,70 @@
+"""Host-side launch shapes (csrc/launch_shape.cuh), compiled by themselves: no GPU needed."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2306_15374_gb300", "csrc")
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    cxx = shutil.which("g++")
+    if not cxx:
+        pytest.skip("no g++")
+
+    def go(name, body):
+        d = tmp_path_factory.mktemp(name)
+        src, exe = str(d / "t.cpp"), str(d / "t")
+        with open(src, "w") as f:
+            f.write('#include <stdio.h>\n#include <thread>\n#include <vector>\n#include "launch_shape.cuh"\n'
+                    "using namespace leco;\nint main() {\n" + body + "\nreturn 0;\n}\n")
+        subprocess.run([cxx, "-std=c++17", "-O1", "-pthread", "-Wall", "-Werror", "-I", CSRC, src, "-o", exe], check=True)
+        return [int(x) for x in subprocess.run([exe], check=True, capture_output=True, text=True).stdout.split()]
+
+    return go
+
+
+def test_every_size_is_asked_once(run):
+    """Columns of every width in turn (stages of 512 bytes a bit), two devices: one question per size and
+    device however often the sizes alternate."""
+    asks, wrong = run("cache", """
+  static ResidentCache cache;
+  int asks = 0, wrong = 0;
+  for (int round = 0; round < 50; round++)
+    for (uint32_t b = 0; b <= 64; b++)
+      for (int dev = 0; dev < 2; dev++) {
+        const uint32_t smem = 1536 + 2 * (512 * b + 64 + 2048);
+        const int want = 1 + (int)((b + dev) % 7);
+        wrong += cache.get(dev, smem, [&]() { asks++; return want; }) != want;
+      }
+  printf("%d %d", asks, wrong);""")
+    assert asks == 2 * 65 and wrong == 0
+
+
+def test_answers_are_the_size_asked_for(run):
+    """Sizes that share a slot, devices beyond the table, failures and threads: always the answer for the size."""
+    wrong, asks, failed = run("mixed", """
+  static ResidentCache cache;
+  int wrong = 0, asks = 0;
+  for (int round = 0; round < 3; round++)
+    for (uint32_t smem : {2048u, 2049u, 2048u + 256u * 1024u, 3000u}) {
+      for (int dev : {0, 63, 64, -1}) wrong += cache.get(dev, smem, [&]() { return (int)(smem % 251u) + 1; }) != (int)(smem % 251u) + 1;
+    }
+  for (int k = 0; k < 3; k++) cache.get(5, 4096, [&]() { asks++; return k < 2 ? 0 : 3; });
+  const int failed = cache.get(5, 4096, []() { return -1; });
+  std::vector<std::thread> ts;
+  std::vector<int> bad(4);
+  for (int t = 0; t < 4; t++)
+    ts.emplace_back([&bad, t]() {
+      for (int k = 0; k < 20000; k++) {
+        const uint32_t smem = 512u * (uint32_t)((k * 7 + t) % 400);
+        bad[t] += cache.get(1, smem, [&]() { return (int)(smem >> 9) % 255 + 1; }) != (int)(smem >> 9) % 255 + 1;
+      }
+    });
+  for (auto& t : ts) t.join();
+  for (int b : bad) wrong += b;
+  printf("%d %d %d", wrong, asks, failed);""")
+    assert wrong == 0 and asks == 3 and failed == 3
