@@ -15,7 +15,7 @@ constexpr int kBlock = 256;
 // that fits L2 is bound by that. So a lookup takes each thing it needs in one load: the first partition
 // and the partition count of its tile, four starts at a time, the whole decode-table entry, and the second
 // residual word only where the field crosses into it: 5M lookups in 100M 32-bit timestamps (variable
-// partitions) 133 -> 105 us against a binary search, two 16-byte entry loads and both words always.
+// partitions) 129 -> 98 us against a binary search, two 16-byte entry loads and both words always.
 
 struct Load32 {
   uint64_t x[4];
@@ -58,12 +58,14 @@ struct PartSearch {
   }
 };
 
+// fixed partitions: the one holding position i (< n)
+__device__ __forceinline__ uint64_t fixed_part(const ColumnView& c, uint64_t i) {
+  return c.n <= 0xFFFFFFFFull ? (uint32_t)i / c.L : i / c.L;
+}
+
 // partition holding position i (< n)
 __device__ __forceinline__ uint64_t find_part(const ColumnView& c, uint64_t i) {
-  if (!c.starts) {
-    if (c.n <= 0xFFFFFFFFull) return (uint32_t)i / c.L;
-    return i / c.L;
-  }
+  if (!c.starts) return fixed_part(c, i);
   PartSearch s;
   s.begin(c, i);
   for (uint32_t step = 0; s.open(); step++) s.take(load32(s.group(c)), i, step);
@@ -80,63 +82,69 @@ __device__ __forceinline__ Aux load_aux(const Aux* __restrict__ aux, uint64_t p)
   return a;
 }
 
-// kUnroll independent lookups per thread and iteration: their loads (index, decode-table entry,
-// residual words) are issued together, so each thread keeps several memory round trips in flight.
-constexpr int kUnroll = 4;
+// U independent lookups per thread and iteration: their loads (index, decode-table entry, residual words) are
+// issued together, so each thread keeps several memory round trips in flight. VAR (variable partitions) is a kernel
+// of its own, two lookups per thread in 64 registers (four CTAs per SM) where a fixed column takes four in 76 (three):
+// with the search behind a branch of one kernel both held 118 registers, two CTAs per SM, and fixed columns paid for
+// a search they never run. 10M lookups in 200M values of fixed partitions 213 -> 193 us, 5M in 20M values 76 -> 63 us;
+// variable partitions: 5M in 1M near-linear values 35 -> 29 us, 5M in 100M timestamps 98 -> 82 us, 10M in 100M piecewise
+// values 244 -> 176 us (three or four lookups per thread: 94 / 96 us on the timestamps, 215 / 242 us on the piecewise).
+constexpr int kUnroll = 4, kVarUnroll = 2;
 
-template <typename T>
+template <typename T, bool VAR>
 __global__ void __launch_bounds__(kBlock)
     k_random_access(const ColumnView c, const uint64_t* __restrict__ idx, uint64_t k,
                     T* __restrict__ out) {
+  constexpr int U = VAR ? kVarUnroll : kUnroll;
   const uint64_t stride = (uint64_t)gridDim.x * kBlock;
-  for (uint64_t base = (uint64_t)blockIdx.x * kBlock + threadIdx.x; base < k; base += stride * kUnroll) {
-    uint64_t i[kUnroll], p[kUnroll];
-    bool ok[kUnroll];
+  for (uint64_t base = (uint64_t)blockIdx.x * kBlock + threadIdx.x; base < k; base += stride * U) {
+    uint64_t i[U], p[U];
+    bool ok[U];
 #pragma unroll
-    for (int u = 0; u < kUnroll; u++) {
+    for (int u = 0; u < U; u++) {
       const uint64_t q = base + (uint64_t)u * stride;
       i[u] = q < k ? __ldg(idx + q) : 0;
       ok[u] = q < k && i[u] < c.n;
     }
-    if (c.starts) {  // the searches of the thread's lookups step together
-      PartSearch f[kUnroll];
+    if (VAR) {  // the searches of the thread's lookups step together
+      PartSearch f[U];
 #pragma unroll
-      for (int u = 0; u < kUnroll; u++) {
+      for (int u = 0; u < U; u++) {
         f[u].begin(c, ok[u] ? i[u] : 0);
         if (!ok[u]) f[u].hi = 0;
       }
       bool more = true;
       for (uint32_t step = 0; more; step++) {
         more = false;
-        Load32 s[kUnroll];
+        Load32 s[U];
 #pragma unroll
-        for (int u = 0; u < kUnroll; u++)
+        for (int u = 0; u < U; u++)
           if (f[u].hi > f[u].lo + 1) s[u] = load32(f[u].group(c));
 #pragma unroll
-        for (int u = 0; u < kUnroll; u++) {
+        for (int u = 0; u < U; u++) {
           if (f[u].hi <= f[u].lo + 1) continue;
           f[u].take(s[u], i[u], step);
           more = more || f[u].open();
         }
       }
 #pragma unroll
-      for (int u = 0; u < kUnroll; u++) p[u] = ok[u] ? f[u].p0 + f[u].lo : 0;
+      for (int u = 0; u < U; u++) p[u] = ok[u] ? f[u].p0 + f[u].lo : 0;
     } else {
 #pragma unroll
-      for (int u = 0; u < kUnroll; u++) p[u] = ok[u] ? find_part(c, i[u]) : 0;
+      for (int u = 0; u < U; u++) p[u] = ok[u] ? fixed_part(c, i[u]) : 0;
     }
-    Aux a[kUnroll];
+    Aux a[U];
 #pragma unroll
-    for (int u = 0; u < kUnroll; u++) a[u] = load_aux(c.aux, ok[u] ? p[u] : 0);
-    uint64_t z[kUnroll];
+    for (int u = 0; u < U; u++) a[u] = load_aux(c.aux, ok[u] ? p[u] : 0);
+    uint64_t z[U];
 #pragma unroll
-    for (int u = 0; u < kUnroll; u++) {
+    for (int u = 0; u < U; u++) {
       const uint64_t x = i[u] - a[u].start;
       const uint32_t b = w3_b(a[u].word3);
       z[u] = ok[u] ? read_field(c.words, w3_off(a[u].word3) + x * b, b) : 0;
     }
 #pragma unroll
-    for (int u = 0; u < kUnroll; u++) {
+    for (int u = 0; u < U; u++) {
       const uint64_t q = base + (uint64_t)u * stride;
       if (q >= k) continue;
       if (!ok[u]) {
@@ -184,11 +192,13 @@ int grid_for(uint64_t items, int per_block, int max_blocks_per_sm) {
 cudaError_t launch_random_access(const ColumnView& c, const uint64_t* idx, uint64_t k, void* out,
                                  cudaStream_t st) {
   if (k == 0) return cudaSuccess;
-  const int grid = grid_for((k + kUnroll - 1) / kUnroll, kBlock, 8);
+  const int u = c.starts ? kVarUnroll : kUnroll, grid = grid_for((k + u - 1) / u, kBlock, 8);
   if (c.dtype == LECO_U32)
-    k_random_access<uint32_t><<<grid, kBlock, 0, st>>>(c, idx, k, (uint32_t*)out);
+    (c.starts ? k_random_access<uint32_t, true> : k_random_access<uint32_t, false>)<<<grid, kBlock, 0, st>>>(
+        c, idx, k, (uint32_t*)out);
   else
-    k_random_access<uint64_t><<<grid, kBlock, 0, st>>>(c, idx, k, (uint64_t*)out);
+    (c.starts ? k_random_access<uint64_t, true> : k_random_access<uint64_t, false>)<<<grid, kBlock, 0, st>>>(
+        c, idx, k, (uint64_t*)out);
   return cudaGetLastError();
 }
 
