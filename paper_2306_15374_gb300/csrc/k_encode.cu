@@ -1,6 +1,7 @@
 // Encoder kernels (§3.1 Regressor, §3.3 Encoder): per-partition fit (fit.cuh), offset scan,
 // decode-table build and residual packing.
 #include "fit.cuh"
+#include "launch_shape.cuh"
 #include "leco_internal.cuh"
 
 namespace leco {
@@ -449,7 +450,6 @@ constexpr int kChunkLoads = 9;
 constexpr uint32_t kChunkVals = 32 * kChunkLoads;
 constexpr uint32_t kPackPiece = 1024;   // values packed at a time
 constexpr uint32_t kPackWindow = 4096;  // positions per warp of a large column
-constexpr uint32_t kPackWindowMin = 256;
 constexpr uint32_t kPackTile = 32 * 33;  // 32-bit entries of a warp's tile
 static_assert(kPackTile * 4 >= kChunkVals * 8, "a chunk's 64-bit residuals fit the tile");
 
@@ -798,19 +798,29 @@ __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
 // ------------------------------------------------------------------------------ batched encode
 
 // The partitions of every column (a partition's column from the partition-column table; the polynomial
-// columns' are fitted by the polynomial phases), eight per pair of warps: a tile of eight lanes each when all
-// are short, else both warps on one after another, as k_fit_pairs.
+// columns' are fitted by the polynomial phases), in groups of eight per pair of warps: a tile of eight lanes each
+// when all are short, else both warps on one after another, as k_fit_pairs. PARTS: the groups of long partitions
+// are dealt out in `parts` parts (fit_parts), where whole groups would leave pairs without work or some with far
+// more than others; a column of 5M values in partitions of 4096 kept 153 of the GPU's 1824 pairs busy.
+// This kernel's time, whole groups -> parts: that column 47 -> 12 us, 20 columns of 8M values in all in partitions of
+// 4096 53 -> 20 us, 16 of 16M 32-bit values in partitions of 1024 53 -> 47 us, 60 columns of 50M values in partitions
+// of 256, 1024 and 4096 231 -> 173 us. A path of a warp or of sixteen lanes per partition of 513 .. 1024 values
+// beside these cost the long ones more in registers (84 -> 96 us for 50M values in partitions of 4096).
 constexpr uint32_t kFitTileVals = 512;
 
-template <typename T>
+template <typename T, bool PARTS>
 __global__ void __launch_bounds__(kFitBlock, kPairCtas)
     k_fit_multi(const EncCol* __restrict__ cols, const uint64_t* __restrict__ part_base,
-                const uint32_t* __restrict__ part_col, uint64_t P, Record* __restrict__ rec,
+                const uint32_t* __restrict__ part_col, uint64_t P, uint32_t parts, Record* __restrict__ rec,
                 uint64_t* __restrict__ lenbits, uint32_t* __restrict__ max_b) {
   __shared__ FitShared sm[kFitPairs];
   const uint32_t g = threadIdx.x >> 6, rank = threadIdx.x & 63u, lane = threadIdx.x & 31u;
-  const uint64_t ng = (uint64_t)gridDim.x * kFitPairs;
-  for (uint64_t p0 = ((uint64_t)blockIdx.x * kFitPairs + g) * 8; p0 < P; p0 += ng * 8) {
+  const uint64_t ng = (uint64_t)gridDim.x * kFitPairs, groups = (P + 7) / 8;
+  const int per = PARTS ? 8 / (int)parts : 8;
+  for (uint64_t t = (uint64_t)blockIdx.x * kFitPairs + g; t < (PARTS ? groups * parts : groups); t += ng) {
+    // first parts of all groups, then the second ones: whole groups of short partitions go with the first
+    const uint64_t part = PARTS ? t / groups : 0, p0 = (t - part * groups) * 8;
+    const int k0 = (int)part * per;
     // lane k (and k + 8, + 16, + 24) of both warps: partition p0 + k
     const uint64_t p = p0 + (lane & 7u);
     uint64_t a = 0;
@@ -826,6 +836,7 @@ __global__ void __launch_bounds__(kFitBlock, kPairCtas)
       v = static_cast<const T*>(col.values) + a;
     }
     if (__all_sync(0xffffffffu, N <= kFitTileVals)) {
+      if (PARTS && part) continue;
       const int k = (int)(rank >> 3);
       const uint32_t n = __shfl_sync(0xffffffffu, N, k);
       const T* vk = reinterpret_cast<const T*>(__shfl_sync(0xffffffffu, (unsigned long long)v, k));
@@ -835,7 +846,7 @@ __global__ void __launch_bounds__(kFitBlock, kPairCtas)
       if ((rank & 7u) == 0 && n) put_fit(R, ak, n, p0 + (uint32_t)k, rec, lenbits, max_b + ck);
       continue;
     }
-    for (int k = 0; k < 8; k++) {
+    for (int k = k0; k < k0 + per; k++) {
       const uint32_t n = __shfl_sync(0xffffffffu, N, k);
       if (n == 0) continue;
       const T* vk = reinterpret_cast<const T*>(__shfl_sync(0xffffffffu, (unsigned long long)v, k));
@@ -879,23 +890,20 @@ __global__ void k_aux_multi(const Record* __restrict__ rec, const PolyCoef* __re
     for (uint64_t w = word_base[c] + (col_bits[c] >> 6); w < word_base[c + 1]; w++) words[w] = 0;
 }
 
-// k_pack over the columns of a batch: windows of every column, tile_base[c] scan tiles before column c
+// k_pack over the columns of a batch: win_base[c] windows before column c's
 template <typename T, bool POLY>
 __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
     k_pack_multi(const EncCol* __restrict__ cols, const uint64_t* __restrict__ part_base,
-                 const uint64_t* __restrict__ tile_base, const uint64_t* __restrict__ word_base, uint32_t ncols,
-                 uint64_t T_tiles, uint32_t window, const Record* __restrict__ rec, const Aux* __restrict__ aux,
+                 const uint64_t* __restrict__ win_base, const uint64_t* __restrict__ word_base, uint32_t ncols,
+                 uint64_t windows, uint32_t window, const Record* __restrict__ rec, const Aux* __restrict__ aux,
                  const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly, uint64_t* __restrict__ words) {
   __shared__ uint64_t zbuf[kPackWarps][kPackTile / 2];
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  const uint32_t per_tile = (uint32_t)kScanTile / window;
-  const uint64_t jobs = T_tiles * per_tile, nw = (uint64_t)gridDim.x * kPackWarps;
-  for (uint64_t k = (uint64_t)blockIdx.x * kPackWarps + wid; k < jobs; k += nw) {
-    const uint64_t g = k / per_tile;
-    const uint32_t c = find_col(tile_base, ncols, g);
+  const uint64_t nw = (uint64_t)gridDim.x * kPackWarps;
+  for (uint64_t k = (uint64_t)blockIdx.x * kPackWarps + wid; k < windows; k += nw) {
+    const uint32_t c = find_col(win_base, ncols, k);
     const EncCol col = cols[c];
-    const uint64_t pos = (k - tile_base[c] * per_tile) * window;
-    if (pos >= col.n) continue;  // the column's last tile is short
+    const uint64_t pos = (k - win_base[c]) * window;
     const uint64_t p0 = part_base[c];
     pack_window<T, POLY>(static_cast<const T*>(col.values), col.n, part_base[c + 1] - p0, pos, min(pos + window, col.n),
                          pos / col.L, rec + p0, aux + p0, POLY ? pcoef + p0 : nullptr, POLY ? poly + p0 : nullptr,
@@ -1068,11 +1076,9 @@ template <typename T, bool POLY>
 cudaError_t launch_pack_t(const void* values, uint64_t n, uint64_t m, uint32_t L, const TileDesc* tiles,
                           const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                           uint64_t* words, cudaStream_t st) {
-  // Windows as long as kPackWindow while each resident warp (32 per SM) still has four, so that the last
-  // wave weighs little: 250M timestamps of ~570-value partitions packed in 650 us with windows of 1024
-  // (which cut most partitions) and 531 us with 4096; columns below 5M values come down to 256.
-  uint32_t window = kPackWindow;
-  while (window > kPackWindowMin && n / window < (uint64_t)sm_count() * 128) window /= 2;
+  // 250M timestamps of ~570-value partitions packed in 650 us with windows of 1024 (which cut most partitions)
+  // and 531 us with 4096; columns below 5M values come down to 256
+  uint32_t window = pack_window(n, kPackWindow, kPackWindowMin, sm_count() * 128);
   // Fixed partitions: whole ones to a window, or a partition's windows from its start on, so that none is cut
   // where it need not be. Whole encodes, windows at any position -> this: 20M values in partitions of 1000 / 1500
   // / 2047 / 3000 159 / 180 / 160 / 151 -> 142 / 167 / 151 / 145 us, 150M of 1000 / 1500 563 / 760 -> 520 / 704.
@@ -1113,16 +1119,20 @@ uint64_t poly_fit_scratch_bytes(uint64_t m) {
 
 cudaError_t launch_fit_multi(const EncCol* cols, const uint64_t* part_base, const uint32_t* part_col, uint32_t ncols,
                              uint64_t P, int dtype, Record* rec, uint64_t* lenbits, PolyCoef* pcoef, uint32_t* max_b,
-                             uint32_t* err, uint32_t fit_ctas, cudaStream_t st, void* poly_scratch) {
-  (void)err;
+                             uint64_t values, uint32_t longest, uint32_t fit_ctas, cudaStream_t st,
+                             void* poly_scratch) {
   cudaError_t e = cudaMemsetAsync(max_b, 0, sizeof(uint32_t) * (ncols ? ncols : 1), st);
   if (e != cudaSuccess || P == 0) return e;
   const int ctas = fit_ctas >= 1 && fit_ctas <= (uint32_t)kFitCtasPerSm ? (int)fit_ctas : kFitCtasPerSm;
-  const int grid = grid_for((P + 7) / 8, kFitPairs, ctas < kPairCtas ? ctas : kPairCtas);
+  const int per_sm = ctas < kPairCtas ? ctas : kPairCtas;
+  const uint32_t parts = fit_parts(values, (uint64_t)sm_count() * per_sm * kFitPairs, longest, kFitTileVals);
+  const int grid = grid_for((P + 7) / 8 * parts, kFitPairs, per_sm);
   if (dtype == LECO_U32)
-    k_fit_multi<uint32_t><<<grid, kFitBlock, 0, st>>>(cols, part_base, part_col, P, rec, lenbits, max_b);
+    (parts > 1 ? k_fit_multi<uint32_t, true> : k_fit_multi<uint32_t, false>)<<<grid, kFitBlock, 0, st>>>(
+        cols, part_base, part_col, P, parts, rec, lenbits, max_b);
   else
-    k_fit_multi<uint64_t><<<grid, kFitBlock, 0, st>>>(cols, part_base, part_col, P, rec, lenbits, max_b);
+    (parts > 1 ? k_fit_multi<uint64_t, true> : k_fit_multi<uint64_t, false>)<<<grid, kFitBlock, 0, st>>>(
+        cols, part_base, part_col, P, parts, rec, lenbits, max_b);
   e = cudaGetLastError();
   if (e == cudaSuccess && pcoef)
     e = launch_poly_fit(BatchColumns{cols, part_base, ncols}, dtype, P, rec, lenbits, pcoef, max_b, st, poly_scratch);
@@ -1160,30 +1170,28 @@ cudaError_t launch_word_bases(const uint64_t* col_bits, uint32_t ncols, uint64_t
 }
 
 template <typename T, bool POLY>
-cudaError_t launch_pack_multi_t(const EncCol* cols, const uint64_t* part_base, const uint64_t* tile_base,
-                                const uint64_t* word_base, uint32_t ncols, uint64_t tiles, uint32_t window,
+cudaError_t launch_pack_multi_t(const EncCol* cols, const uint64_t* part_base, const uint64_t* win_base,
+                                const uint64_t* word_base, uint32_t ncols, uint64_t windows, uint32_t window,
                                 const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                                 uint64_t* words, cudaStream_t st) {
-  const uint64_t jobs = tiles * (kScanTile / window);
-  k_pack_multi<T, POLY><<<grid_for(jobs, kPackWarps, 8), kPackBlock, 0, st>>>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
-                                                     aux, pcoef, poly, words);
+  k_pack_multi<T, POLY><<<grid_for(windows, kPackWarps, 8), kPackBlock, 0, st>>>(
+      cols, part_base, win_base, word_base, ncols, windows, window, rec, aux, pcoef, poly, words);
   return cudaGetLastError();
 }
 
-cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* tile_base,
-                              const uint64_t* word_base, uint32_t ncols, uint64_t tiles, int dtype, uint32_t window,
+cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* win_base,
+                              const uint64_t* word_base, uint32_t ncols, uint64_t windows, int dtype, uint32_t window,
                               const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                               uint64_t* words, cudaStream_t st) {
-  if (tiles == 0) return cudaSuccess;
-  if (window < 1024 || window > kScanTile || kScanTile % window) window = (uint32_t)kScanTile;
+  if (windows == 0) return cudaSuccess;
   if (dtype == LECO_U32)
-    return pcoef ? launch_pack_multi_t<uint32_t, true>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
+    return pcoef ? launch_pack_multi_t<uint32_t, true>(cols, part_base, win_base, word_base, ncols, windows, window, rec,
                                                        aux, pcoef, poly, words, st)
-                 : launch_pack_multi_t<uint32_t, false>(cols, part_base, tile_base, word_base, ncols, tiles, window,
+                 : launch_pack_multi_t<uint32_t, false>(cols, part_base, win_base, word_base, ncols, windows, window,
                                                         rec, aux, nullptr, nullptr, words, st);
-  return pcoef ? launch_pack_multi_t<uint64_t, true>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
+  return pcoef ? launch_pack_multi_t<uint64_t, true>(cols, part_base, win_base, word_base, ncols, windows, window, rec,
                                                      aux, pcoef, poly, words, st)
-               : launch_pack_multi_t<uint64_t, false>(cols, part_base, tile_base, word_base, ncols, tiles, window, rec,
+               : launch_pack_multi_t<uint64_t, false>(cols, part_base, win_base, word_base, ncols, windows, window, rec,
                                                       aux, nullptr, nullptr, words, st);
 }
 

@@ -1,9 +1,11 @@
 // Batched decode plans and the scan autotuner (declared in include/leco_batch.h).
+#include <algorithm>
 #include <string.h>
 
 #include <vector>
 
 #include "column.cuh"
+#include "launch_shape.cuh"
 #include "leco_batch.h"
 
 using namespace leco;
@@ -342,11 +344,15 @@ struct EncBatch {
   bool any_poly = false;
   std::vector<EncCol> ec;
   std::vector<uint64_t> part_base, tile_base;
+  std::vector<uint64_t> bases;  // part_base | tile_base | first packer window of each column
+  uint32_t window = 0;          // positions per packer window
   uint64_t P = 0, T = 0;
+  uint64_t fit_values = 0;  // the constant and linear columns: values, longest partition
+  uint32_t longest = 0;
   uint64_t rec_b = 0, tiles_b = 0, stat_b = 0, poly_b = 0, pc_words = 0, pcol_words = 0, scr_words = 0;
 
   EncBatch(const void* const* d_vals, const uint64_t* n, const leco_model* models, const uint32_t* L, uint32_t k,
-           leco_dtype dt)
+           leco_dtype dt, uint32_t item_values)
       : ncols(k), dtype(dt), ec(k), part_base(k + 1), tile_base(k + 1) {
     for (uint32_t c = 0; c < ncols; c++) any_poly = any_poly || models[c] == LECO_MODEL_POLY;
     part_base[0] = tile_base[0] = 0;
@@ -354,9 +360,20 @@ struct EncBatch {
       ec[c] = EncCol{d_vals[c], n[c], L[c], (int32_t)models[c]};
       part_base[c + 1] = part_base[c] + (n[c] + L[c] - 1) / L[c];
       tile_base[c + 1] = tile_base[c] + scan_tiles(n[c]);
+      if (models[c] == LECO_MODEL_POLY) continue;
+      fit_values += n[c];
+      longest = std::max(longest, (uint32_t)std::min<uint64_t>(n[c], L[c]));
     }
     P = part_base[ncols];
     T = tile_base[ncols];
+    uint64_t values = 0;
+    for (uint32_t c = 0; c < ncols; c++) values += n[c];
+    if (item_values < 1024 || item_values > kScanTile || kScanTile % item_values) item_values = (uint32_t)kScanTile;
+    window = pack_window(values, item_values, kPackWindowMin, sm_count() * 32);
+    bases = part_base;
+    bases.insert(bases.end(), tile_base.begin(), tile_base.end());
+    bases.push_back(0);
+    for (uint32_t c = 0; c < ncols; c++) bases.push_back(bases.back() + (n[c] + window - 1) / window);
     auto a256 = [](uint64_t x) { return (x + 255) & ~255ull; };
     rec_b = a256(32 * (P ? P : 1));
     tiles_b = a256(sizeof(TileDesc) * (T ? T : 1));
@@ -469,12 +486,12 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   cudaStream_t st = (cudaStream_t)stream;
   int dev = 0;
   cudaGetDevice(&dev);
-  const EncBatch B(d_vals, n, models, L, ncols, dtype);
+  const EncBatch B(d_vals, n, models, L, ncols, dtype, cfg.item_values);
   const uint64_t P = B.P, T = B.T;
   char* meta = nullptr;
   uint64_t* scr = nullptr;
   EncCol* d_ec = nullptr;
-  uint64_t* d_bases = nullptr;  // part_base | tile_base | word_base
+  uint64_t* d_bases = nullptr;  // part_base | tile_base | win_base | word_base
   ColumnView* d_views = nullptr;
   uint64_t* words = nullptr;
   std::vector<uint64_t> col_bits(ncols), word_base(ncols + 1);
@@ -483,23 +500,22 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   cudaError_t e = dev_alloc((void**)&meta, B.meta_bytes(), st);
   if (e == cudaSuccess) e = dev_alloc((void**)&scr, 8 * B.scr_words, st);
   if (e == cudaSuccess) e = dev_alloc((void**)&d_ec, sizeof(EncCol) * ncols, st);
-  if (e == cudaSuccess) e = dev_alloc((void**)&d_bases, 8 * 3 * (uint64_t)(ncols + 1), st);
+  if (e == cudaSuccess) e = dev_alloc((void**)&d_bases, 8 * 4 * (uint64_t)(ncols + 1), st);
   if (e == cudaSuccess) e = dev_alloc((void**)&d_views, sizeof(ColumnView) * ncols, st);
   const EncPtrs p = enc_ptrs(B, meta, scr);
   uint64_t* d_part = d_bases;
   uint64_t* d_tile = d_bases + (ncols + 1);
-  uint64_t* d_word = d_bases + 2 * (ncols + 1);
+  uint64_t* d_win = d_bases + 2 * (ncols + 1);
+  uint64_t* d_word = d_bases + 3 * (ncols + 1);
   if (e == cudaSuccess) e = cudaMemsetAsync(p.status, 0, B.stat_b, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(d_ec, B.ec.data(), sizeof(EncCol) * ncols, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_part, B.part_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(d_tile, B.tile_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, st);
+    e = cudaMemcpyAsync(d_bases, B.bases.data(), 8 * B.bases.size(), cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) e = launch_part_col(d_part, ncols, P, p.part_col, st);
   // fit every partition of every column, then column-relative offsets and per-column totals
   if (e == cudaSuccess)
-    e = launch_fit_multi(d_ec, d_part, p.part_col, ncols, P, dtype, p.rec, p.lenbits, p.pcoef, p.maxb, p.status,
-                         cfg.fit_ctas, st);
+    e = launch_fit_multi(d_ec, d_part, p.part_col, ncols, P, dtype, p.rec, p.lenbits, p.pcoef, p.maxb,
+                         B.fit_values, B.longest, cfg.fit_ctas, st);
   if (e == cudaSuccess) e = launch_offsets_multi(p.rec, p.lenbits, d_part, p.part_col, ncols, P, p.offs, p.colbits, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(col_bits.data(), p.colbits, 8 * ncols, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(max_b.data(), p.maxb, 4 * ncols, cudaMemcpyDeviceToHost, st);
@@ -519,8 +535,8 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, d_ec, d_part, p.part_col, d_word, p.colbits, ncols, P, p.aux, p.poly, words, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(d_views, d_tile, ncols, T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(d_ec, d_part, d_tile, d_word, ncols, T, dtype, cfg.item_values, p.rec, p.aux, p.pcoef, p.poly,
-                          words, st);
+    e = launch_pack_multi(d_ec, d_part, d_win, d_word, ncols, B.bases.back(), dtype, B.window, p.rec, p.aux, p.pcoef,
+                          p.poly, words, st);
   if (e == cudaSuccess) e = make_batch_columns(B, p, words, word_base, col_bits, max_b, models, L, dev, st, meta, out);
   cudaFreeAsync(scr, st);
   cudaFreeAsync(d_ec, st);
@@ -552,7 +568,7 @@ struct leco_batch_encode_plan {
   uint64_t* scr = nullptr;
   void* poly_scr = nullptr;
   EncCol* d_ec = nullptr;
-  uint64_t* d_bases = nullptr;  // part_base | tile_base | word_base
+  uint64_t* d_bases = nullptr;  // part_base | tile_base | win_base | word_base
   ColumnView* d_views = nullptr;
   uint64_t* words = nullptr;
   uint64_t words_cap = 0;  // 64-bit words reserved for the packed streams
@@ -582,18 +598,19 @@ cudaError_t enc_plan_launches(leco_batch_encode_plan* pl, cudaStream_t st) {
   const EncPtrs p = enc_ptrs(B, pl->meta, pl->scr);
   uint64_t* d_part = pl->d_bases;
   uint64_t* d_tile = pl->d_bases + (B.ncols + 1);
-  uint64_t* d_word = pl->d_bases + 2 * (B.ncols + 1);
+  uint64_t* d_win = pl->d_bases + 2 * (B.ncols + 1);
+  uint64_t* d_word = pl->d_bases + 3 * (B.ncols + 1);
   cudaError_t e = cudaMemsetAsync(p.status, 0, B.stat_b, st);
   if (e == cudaSuccess)
     e = launch_fit_multi(pl->d_ec, d_part, p.part_col, B.ncols, B.P, B.dtype, p.rec, p.lenbits, p.pcoef, p.maxb,
-                         p.status, pl->cfg.fit_ctas, st, pl->poly_scr);
+                         B.fit_values, B.longest, pl->cfg.fit_ctas, st, pl->poly_scr);
   if (e == cudaSuccess)
     e = launch_offsets_multi(p.rec, p.lenbits, d_part, p.part_col, B.ncols, B.P, p.offs, p.colbits, st);
   if (e == cudaSuccess) e = launch_word_bases(p.colbits, B.ncols, d_word, st);
   if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, pl->d_ec, d_part, p.part_col, d_word, p.colbits, B.ncols, B.P, p.aux, p.poly, pl->words, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(pl->d_views, d_tile, B.ncols, B.T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(pl->d_ec, d_part, d_tile, d_word, B.ncols, B.T, B.dtype, pl->cfg.item_values, p.rec, p.aux,
+    e = launch_pack_multi(pl->d_ec, d_part, d_win, d_word, B.ncols, B.bases.back(), B.dtype, B.window, p.rec, p.aux,
                           p.pcoef, p.poly, pl->words, st);
   return e;
 }
@@ -667,7 +684,7 @@ extern "C" leco_status leco_batch_encode_plan_create(const void* const* d_vals, 
   if (!pl) return LECO_ERR_OOM;
   pl->device = dev;
   pl->cfg = encode_config_lookup(dtype);
-  pl->B = new (std::nothrow) EncBatch(d_vals, n, models, L, ncols, dtype);
+  pl->B = new (std::nothrow) EncBatch(d_vals, n, models, L, ncols, dtype, pl->cfg.item_values);
   if (!pl->B) {
     enc_plan_release(pl);
     return LECO_ERR_OOM;
@@ -694,7 +711,7 @@ extern "C" leco_status leco_batch_encode_plan_create(const void* const* d_vals, 
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->scr, 8 * B.scr_words);
   if (e == cudaSuccess && B.any_poly) e = cudaMalloc(&pl->poly_scr, poly_fit_scratch_bytes(B.P ? B.P : 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_ec, sizeof(EncCol) * ncols);
-  if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_bases, 8 * 3 * (uint64_t)(ncols + 1));
+  if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_bases, 8 * 4 * (uint64_t)(ncols + 1));
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->d_views, sizeof(ColumnView) * ncols);
   if (e == cudaSuccess) e = cudaMalloc((void**)&pl->words, 8 * cap);
   const EncPtrs p = enc_ptrs(B, pl->meta, pl->scr);
@@ -705,9 +722,7 @@ extern "C" leco_status leco_batch_encode_plan_create(const void* const* d_vals, 
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(pl->d_ec, B.ec.data(), sizeof(EncCol) * ncols, cudaMemcpyHostToDevice, cst);
   if (e == cudaSuccess)
-    e = cudaMemcpyAsync(pl->d_bases, B.part_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, cst);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(pl->d_bases + (ncols + 1), B.tile_base.data(), 8 * (ncols + 1), cudaMemcpyHostToDevice, cst);
+    e = cudaMemcpyAsync(pl->d_bases, B.bases.data(), 8 * B.bases.size(), cudaMemcpyHostToDevice, cst);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(pl->d_views, views.data(), sizeof(ColumnView) * ncols, cudaMemcpyHostToDevice, cst);
   // the partition -> column table depends on the shapes only: filled once, outside the graph
@@ -778,7 +793,7 @@ extern "C" uint64_t leco_batch_encode_plan_reserved_bytes(const leco_batch_encod
   const EncBatch& B = *plan->B;
   const uint64_t nc = B.ncols;
   return B.meta_bytes() + 8 * B.scr_words + (B.any_poly ? poly_fit_scratch_bytes(B.P ? B.P : 1) : 0) +
-         sizeof(EncCol) * nc + 8 * 3 * (nc + 1) + sizeof(ColumnView) * nc + 8 * plan->words_cap;
+         sizeof(EncCol) * nc + 8 * 4 * (nc + 1) + sizeof(ColumnView) * nc + 8 * plan->words_cap;
 }
 
 extern "C" void leco_batch_encode_plan_free(leco_batch_encode_plan* plan) {

@@ -288,11 +288,13 @@ struct EncCol {
 // part_col[p]: the column of global partition p (launch_part_col fills it once per batch)
 cudaError_t launch_part_col(const uint64_t* part_base, uint32_t ncols, uint64_t P, uint32_t* part_col, cudaStream_t st);
 // poly_scratch: poly_fit_scratch_bytes(P) caller-owned bytes for the polynomial phases, or nullptr
-// (then taken from the library pool for the call)
+// (then taken from the library pool for the call); values and longest: of
+// the constant and linear columns, in all and in their longest partition
 uint64_t poly_fit_scratch_bytes(uint64_t m);
 cudaError_t launch_fit_multi(const EncCol* cols, const uint64_t* part_base, const uint32_t* part_col, uint32_t ncols,
                              uint64_t P, int dtype, Record* rec, uint64_t* lenbits, PolyCoef* pcoef, uint32_t* max_b,
-                             uint32_t* err, uint32_t fit_ctas, cudaStream_t st, void* poly_scratch = nullptr);
+                             uint64_t values, uint32_t longest, uint32_t fit_ctas, cudaStream_t st,
+                             void* poly_scratch = nullptr);
 uint64_t offsets_multi_scratch_elems(uint64_t P);
 cudaError_t launch_offsets_multi(Record* rec, const uint64_t* lenbits, const uint64_t* part_base,
                                  const uint32_t* part_col, uint32_t ncols, uint64_t P, uint64_t* scratch,
@@ -304,9 +306,9 @@ cudaError_t launch_aux_multi(const Record* rec, const PolyCoef* pcoef, const Enc
 // word_base[c] = sum of stream_words(col_bits[k]) over k < c, for c = 0 .. ncols, on the device (one
 // CTA): each column's packed stream placed right after the previous one
 cudaError_t launch_word_bases(const uint64_t* col_bits, uint32_t ncols, uint64_t* word_base, cudaStream_t st);
-// window: positions a warp packs (1024, 2048 or 4096); tiles: scan tiles of all columns
-cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* tile_base,
-                              const uint64_t* word_base, uint32_t ncols, uint64_t tiles, int dtype, uint32_t window,
+// window: positions a warp packs at a time; windows: of all columns, win_base[c] of them before column c's
+cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* win_base,
+                              const uint64_t* word_base, uint32_t ncols, uint64_t windows, int dtype, uint32_t window,
                               const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                               uint64_t* words, cudaStream_t st);
 // poly: some column has a polynomial table (its tiles then get the exact polynomial bounds)

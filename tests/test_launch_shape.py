@@ -68,3 +68,25 @@ def test_answers_are_the_size_asked_for(run):
   for (int b : bad) wrong += b;
   printf("%d %d %d", wrong, asks, failed);""")
     assert wrong == 0 and asks == 3 and failed == 3
+
+
+def test_small_columns_get_windows_for_many_warps(run):
+    """A few thousand values are packed by as many warps as windows of 256 positions give; a large column or batch
+    keeps the long ones."""
+    got = run("window", """
+  for (uint64_t n : {0ull, 1ull, 3000ull, 1245183ull, 5000000ull, 20000000ull, 79691776ull, 200000000ull})
+    printf("%u %u %u ", pack_window(n, 4096, 256, 152 * 128), pack_window(n, 4096, 256, 152 * 32), pack_window(n, 1024, 256, 152 * 32));""")
+    assert got[0::3] == [256, 256, 256, 256, 256, 1024, 4096, 4096]
+    assert got[1::3] == [256, 256, 256, 256, 1024, 4096, 4096, 4096]
+    assert got[2::3] == [256, 256, 256, 256, 1024, 1024, 1024, 1024]
+
+
+def test_long_partitions_are_dealt_out(run):
+    """Groups of eight partitions stay together where they are short or where the longest is half a pair's
+    share; otherwise as many parts as that takes, a partition at the least."""
+    pairs = 152 * 3 * 4
+    got = run("parts", f"""
+  struct {{ uint64_t values; uint32_t longest; }} cases[] = {{{{0, 0}}, {{200000000, 512}}, {{5000, 513}}, {{5000000, 4096}},
+      {{16000000, 1024}}, {{50000000, 4096}}, {{100000000, 2048}}, {{100000000, 1000}}, {{200000000, 4096}}, {{1ull << 40, 1u << 24}}}};
+  for (auto c : cases) printf("%u ", fit_parts(c.values, {pairs}, c.longest, 512));""")
+    assert got == [1, 1, 8, 8, 2, 4, 1, 1, 1, 1]
