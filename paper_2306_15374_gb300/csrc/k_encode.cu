@@ -1,5 +1,7 @@
 // Encoder kernels (§3.1 Regressor, §3.3 Encoder): per-partition fit (fit.cuh), offset scan,
 // decode-table build and residual packing.
+#include <type_traits>
+
 #include "fit.cuh"
 #include "launch_shape.cuh"
 #include "leco_internal.cuh"
@@ -434,8 +436,9 @@ __global__ void k_build_aux(const Record* __restrict__ rec, const PolyCoef* __re
 // The values' residuals go to a shared tile of 32 rows of K = 8, 16 or 32 consecutive values; lane r takes
 // row r into registers, strings its bits together from their place in the piece's words on (no division,
 // two values at a time up to 16 bits), passes the open last word to the next lane and leaves the others in
-// the tile, from where they go out coalesced. Widths above 32 bits and binary64 partitions assemble each word from
-// the fields it holds instead (pack_words, 79 instructions per value against 43).
+// the tile, from where they go out coalesced. Widths above 32 bits take 64-bit entries and rows of 8 (20M values of 63
+// bits in partitions of 4096 116 -> 75 us, of 40 bits 88 -> 63 us, against each word assembled from the fields it
+// holds); pieces of up to 128 such values, wide polynomial and binary64 partitions still assemble words (pack_words).
 // The former packer staged a partition, or a run of short ones, per CTA by a bulk copy, three to seven
 // CTAs per SM each waiting for its own, and recomputed every field of partitions beyond 4096 values
 // from memory. Bound: memory and the latency of a piece's chain (64 registers hold 32 warps per SM; 48, 40
@@ -541,8 +544,9 @@ __device__ __forceinline__ void pack_words(const PackPart<T>& q, const Aux& a, c
 }
 
 // values [x0, x0 + V) of a partition of width b <= 32 on a line (or, PL, a polynomial), V <= 32 K, K b >= 32:
-// lane r packs the K consecutive values of row r
-template <int K, typename T, bool PL>
+// lane r packs the K consecutive values of row r. WIDE: widths above 32 bits, K = 8; a value goes in as its low 32
+// bits and the rest.
+template <int K, typename T, bool PL, bool WIDE = false>
 __device__ __forceinline__ void pack_rows(const PackPart<T>& q, const Aux& a, const PolyAux* __restrict__ poly,
                                           uint32_t x0, uint32_t V, uint32_t* tile, uint32_t lane) {
   const uint32_t b = q.b;
@@ -566,13 +570,18 @@ __device__ __forceinline__ void pack_rows(const PackPart<T>& q, const Aux& a, co
     if (lane * b < o && lane < x0) {
       const uint32_t x = x0 - 1u - lane;
       const uint64_t pred = PL ? (uint64_t)predict_aux(a, nullptr, poly, q.p, x) : (uint64_t)((int64_t)(q.A + q.B * x) >> q.sh);
-      const uint32_t z = zz32((uint64_t)__ldg(q.v + x) - pred);
+      const uint64_t r = (uint64_t)__ldg(q.v + x) - pred;
       const int32_t s = (int32_t)o - (int32_t)((lane + 1u) * b);
-      c = s >= 0 ? z << s : z >> (-s);
+      if (WIDE)
+        c = (uint32_t)(zz_encode((int64_t)r) >> (-s));  // o < 32 < b
+      else
+        c = s >= 0 ? zz32(r) << s : zz32(r) >> (-s);
     }
     prev = __reduce_or_sync(0xffffffffu, c);
   }
-  uint32_t* put = tile + lane + (K == 32 ? 0u : lane / (uint32_t)K);
+  using Z = typename std::conditional<WIDE, uint64_t, uint32_t>::type;
+  Z* zs = reinterpret_cast<Z*>(tile);
+  Z* put = zs + lane + (K == 32 ? 0u : lane / (uint32_t)K);
 #pragma unroll
   for (int k = 0; k < K; k += 8) {
     const int cur = (k >> 3) & 1;
@@ -590,7 +599,8 @@ __device__ __forceinline__ void pack_rows(const PackPart<T>& q, const Aux& a, co
         pred = (uint64_t)((int64_t)F >> q.sh);
         F += dF;
       }
-      put[(32 + 32 / K) * (k + u)] = zz32((uint64_t)val[cur][u] - pred);  // value x at x + x / K
+      const uint64_t r = (uint64_t)val[cur][u] - pred;
+      put[(32 + 32 / K) * (k + u)] = WIDE ? (Z)zz_encode((int64_t)r) : (Z)zz32(r);  // value x at x + x / K
     }
   }
   __syncwarp();
@@ -624,9 +634,9 @@ __device__ __forceinline__ void pack_rows(const PackPart<T>& q, const Aux& a, co
     }
     open = acc;
   } else {
-    uint32_t z[K];
+    Z z[K];
 #pragma unroll
-    for (int i = 0; i < K; i++) z[i] = tile[lane * (K + 1) + i];
+    for (int i = 0; i < K; i++) z[i] = zs[lane * (K + 1) + i];
     __syncwarp();
     uint32_t w = wf, fill = at & 31u, acc = 0;
     auto emit = [&](uint32_t x, uint32_t width) {
@@ -638,13 +648,19 @@ __device__ __forceinline__ void pack_rows(const PackPart<T>& q, const Aux& a, co
       fill = (fill + width) & 31u;
       w += full ? 1u : 0u;
     };
-    if (b <= 16) {
+    if (WIDE) {
+#pragma unroll
+      for (int i = 0; i < K; i++) {
+        emit((uint32_t)z[i], 32u);
+        emit((uint32_t)((uint64_t)z[i] >> 32), b - 32u);
+      }
+    } else if (b <= 16) {
       const uint32_t pw = 1u << b;
 #pragma unroll
-      for (int i = 0; i < K; i += 2) emit(z[i] + z[i + 1] * pw, 2u * b);
+      for (int i = 0; i < K; i += 2) emit((uint32_t)z[i] + (uint32_t)z[i + 1] * pw, 2u * b);
     } else {
 #pragma unroll
-      for (int i = 0; i < K; i++) emit(z[i], b);
+      for (int i = 0; i < K; i++) emit((uint32_t)z[i], b);
     }
     open = acc;
   }
@@ -678,7 +694,7 @@ __device__ __forceinline__ void pack_rows(const PackPart<T>& q, const Aux& a, co
 }
 
 // values [xa, xb) of a partition of N values (its first value at v[0], entry a, index p)
-template <typename T, bool POLY>
+template <typename T, bool POLY, bool WIDE>
 __device__ __forceinline__ void pack_piece(const T* __restrict__ v, uint32_t N, uint32_t xa, uint32_t xb, const Aux& a,
                                            const Record* __restrict__ rec, const PolyAux* __restrict__ poly, uint64_t p,
                                            uint32_t* __restrict__ words, uint64_t* zbuf, uint32_t lane) {
@@ -697,8 +713,12 @@ __device__ __forceinline__ void pack_piece(const T* __restrict__ v, uint32_t N, 
   q.sh = sr > 0 ? (uint32_t)sr & 63u : 0u;
   q.p = p;
   const bool line = w3_exact(a.word3) != 0, pl = POLY && w3_poly(a.word3) != 0;
+  uint32_t* tile = reinterpret_cast<uint32_t*>(zbuf);
+  if (WIDE && q.b > 32 && line && xb - xa > 128) {  // shorter pieces leave most of the 32 rows empty
+    for (uint32_t x = xa; x < xb; x += 256) pack_rows<8, T, false, true>(q, a, poly, x, min(256u, xb - x), tile, lane);
+    return;
+  }
   if (q.b <= 32 && (line || pl)) {
-    uint32_t* tile = reinterpret_cast<uint32_t*>(zbuf);
     for (uint32_t x = xa; x < xb; x += kPackPiece) {
       const uint32_t V = min(kPackPiece, xb - x);
       if (pl)
@@ -732,7 +752,7 @@ __device__ __forceinline__ void pack_block(const PolyCoef& pc, uint64_t off0, ui
 }
 
 // positions [pos, end) of a column, partition p holding pos
-template <typename T, bool POLY>
+template <typename T, bool POLY, bool WIDE>
 __device__ __forceinline__ void pack_window(const T* __restrict__ values, uint64_t n, uint64_t m, uint64_t pos,
                                             uint64_t end, uint64_t p, const Record* __restrict__ rec,
                                             const Aux* __restrict__ aux, const PolyCoef* __restrict__ pcoef,
@@ -754,16 +774,18 @@ __device__ __forceinline__ void pack_window(const T* __restrict__ values, uint64
       const uint64_t e = __shfl_sync(0xffffffffu, mine.start, k + 1);
       const uint32_t xa = (uint32_t)(pos - a.start);
       if (POLY && xa == 0 && w3_poly(a.word3)) pack_block(pcoef[p], w3_off(a.word3) - kPolyBlockBits, words, lane);
-      pack_piece<T, POLY>(values + a.start, (uint32_t)(e - a.start), xa, (uint32_t)(min(e, end) - a.start), a, rec, poly,
+      pack_piece<T, POLY, WIDE>(values + a.start, (uint32_t)(e - a.start), xa, (uint32_t)(min(e, end) - a.start), a, rec, poly,
                           p, words, zbuf, lane);
       pos = e;
     }
   }
 }
 
-// L: the fixed partition length, or 0: partitions of any lengths, found through the scan tiles. Every `period`
+// WIDE: some partition of the column is wider than 32 bits (a kernel of its own, since the others would be 2 - 4 %
+// slower beside those rows). L: the fixed partition length, or 0: partitions of any lengths, found through the scan
+// tiles. Every `period`
 // positions hold `per` windows, the last one shorter where they do not divide it.
-template <typename T, bool POLY>
+template <typename T, bool POLY, bool WIDE>
 __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
     k_pack(const T* __restrict__ values, uint64_t n, uint64_t m, uint32_t L, uint32_t window, uint32_t period,
            uint32_t per, const TileDesc* __restrict__ tiles, const Record* __restrict__ rec,
@@ -791,7 +813,7 @@ __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
           hi = mid;
       }
     }
-    pack_window<T, POLY>(values, n, m, pos, end, p, rec, aux, pcoef, poly, words, zbuf[wid], lane);
+    pack_window<T, POLY, WIDE>(values, n, m, pos, end, p, rec, aux, pcoef, poly, words, zbuf[wid], lane);
   }
 }
 
@@ -905,7 +927,7 @@ __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
     const EncCol col = cols[c];
     const uint64_t pos = (k - win_base[c]) * window;
     const uint64_t p0 = part_base[c];
-    pack_window<T, POLY>(static_cast<const T*>(col.values), col.n, part_base[c + 1] - p0, pos, min(pos + window, col.n),
+    pack_window<T, POLY, true>(static_cast<const T*>(col.values), col.n, part_base[c + 1] - p0, pos, min(pos + window, col.n),
                          pos / col.L, rec + p0, aux + p0, POLY ? pcoef + p0 : nullptr, POLY ? poly + p0 : nullptr,
                          reinterpret_cast<uint32_t*>(words + word_base[c]), zbuf[wid], lane);
   }
@@ -1075,7 +1097,7 @@ cudaError_t launch_build_aux(const Record* rec, const PolyCoef* pcoef, uint64_t 
 template <typename T, bool POLY>
 cudaError_t launch_pack_t(const void* values, uint64_t n, uint64_t m, uint32_t L, const TileDesc* tiles,
                           const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
-                          uint64_t* words, cudaStream_t st) {
+                          uint32_t max_b, uint64_t* words, cudaStream_t st) {
   // 250M timestamps of ~570-value partitions packed in 650 us with windows of 1024 (which cut most partitions)
   // and 531 us with 4096; columns below 5M values come down to 256
   uint32_t window = pack_window(n, kPackWindow, kPackWindowMin, sm_count() * 128);
@@ -1090,7 +1112,8 @@ cudaError_t launch_pack_t(const void* values, uint64_t n, uint64_t m, uint32_t L
     per = (uint32_t)(((uint64_t)period + window - 1) / window);
   }
   const uint64_t nwin = (n + period - 1) / period * per;
-  k_pack<T, POLY><<<grid_for(nwin, kPackWarps, 8), kPackBlock, 0, st>>>(
+  auto kern = max_b > 32 ? k_pack<T, POLY, true> : k_pack<T, POLY, POLY>;
+  kern<<<grid_for(nwin, kPackWarps, 8), kPackBlock, 0, st>>>(
       static_cast<const T*>(values), n, m, L, window, period, per, tiles, rec, aux, pcoef, poly,
       reinterpret_cast<uint32_t*>(words));
   return cudaGetLastError();
@@ -1098,13 +1121,13 @@ cudaError_t launch_pack_t(const void* values, uint64_t n, uint64_t m, uint32_t L
 
 cudaError_t launch_pack(const void* values, int dtype, uint32_t L, const TileDesc* tiles, const Record* rec,
                         const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly, uint64_t m, uint64_t n,
-                        uint64_t* words, cudaStream_t st) {
+                        uint32_t max_b, uint64_t* words, cudaStream_t st) {
   if (m == 0) return cudaSuccess;
   if (dtype == LECO_U32)
-    return pcoef ? launch_pack_t<uint32_t, true>(values, n, m, L, tiles, rec, aux, pcoef, poly, words, st)
-                 : launch_pack_t<uint32_t, false>(values, n, m, L, tiles, rec, aux, nullptr, nullptr, words, st);
-  return pcoef ? launch_pack_t<uint64_t, true>(values, n, m, L, tiles, rec, aux, pcoef, poly, words, st)
-               : launch_pack_t<uint64_t, false>(values, n, m, L, tiles, rec, aux, nullptr, nullptr, words, st);
+    return pcoef ? launch_pack_t<uint32_t, true>(values, n, m, L, tiles, rec, aux, pcoef, poly, max_b, words, st)
+                 : launch_pack_t<uint32_t, false>(values, n, m, L, tiles, rec, aux, nullptr, nullptr, max_b, words, st);
+  return pcoef ? launch_pack_t<uint64_t, true>(values, n, m, L, tiles, rec, aux, pcoef, poly, max_b, words, st)
+               : launch_pack_t<uint64_t, false>(values, n, m, L, tiles, rec, aux, nullptr, nullptr, max_b, words, st);
 }
 
 cudaError_t launch_part_col(const uint64_t* part_base, uint32_t ncols, uint64_t P, uint32_t* part_col, cudaStream_t st) {

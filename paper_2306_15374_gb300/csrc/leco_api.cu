@@ -131,7 +131,7 @@ leco_status encode_partitions(leco_column* c, const void* d_values, cudaStream_t
   if (e == cudaSuccess) e = launch_tile_desc(view_of(c), c->tiles, st);
   if (e == cudaSuccess)
     e = launch_pack(d_values, c->dtype, starts ? 0u : c->L, c->tiles, c->rec, c->aux, pcoef, c->poly, m, c->n,
-                    c->words, st);
+                    c->max_b, c->words, st);
   cudaFreeAsync(scr, st);
   if (e == cudaErrorInvalidValue) return LECO_ERR_INVALID_ARG;
   return from_cuda(e);

@@ -356,10 +356,11 @@ uint64_t offsets_scratch_elems(uint64_t m);
 cudaError_t launch_build_aux(const Record* rec, const PolyCoef* pcoef, uint64_t m, uint64_t n, Aux* aux,
                              PolyAux* poly, uint64_t total_bits, uint64_t* words, uint64_t nwords, uint32_t* status,
                              cudaStream_t st);
-// L: the fixed partition length, or 0 with the column's tile descriptors for partitions of any lengths
+// L: the fixed partition length, or 0 with the column's tile descriptors for partitions of any lengths; max_b: the
+// widest partition
 cudaError_t launch_pack(const void* values, int dtype, uint32_t L, const TileDesc* tiles, const Record* rec,
                         const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly, uint64_t m, uint64_t n,
-                        uint64_t* words, cudaStream_t st);
+                        uint32_t max_b, uint64_t* words, cudaStream_t st);
 
 // scans (k_scan.cu) and lookups (k_decode.cu)
 cudaError_t launch_tile_desc(const ColumnView& c, TileDesc* tiles, cudaStream_t st);

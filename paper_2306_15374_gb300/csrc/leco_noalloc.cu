@@ -70,8 +70,9 @@ extern "C" leco_status leco_encode_fixed_noalloc(const void* d_values, uint64_t 
   cudaError_t e = launch_fit(d_values, dtype, n, nullptr, L, m, model, rec, lenbits, nullptr,
                              reinterpret_cast<uint32_t*>(res + 1), nullptr, st);
   if (e == cudaSuccess) e = launch_offsets(rec, lenbits, m, off_scr, offsets_scratch_elems(m), res, st);
-  uint64_t total = 0;
-  if (e == cudaSuccess) e = cudaMemcpyAsync(&total, res, 8, cudaMemcpyDeviceToHost, st);
+  uint64_t hres[2] = {0, 0};
+  const uint64_t& total = hres[0];
+  if (e == cudaSuccess) e = cudaMemcpyAsync(hres, res, 16, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return e == cudaErrorMemoryAllocation ? LECO_ERR_OOM : LECO_ERR_CUDA;
   if (total >= (1ull << 48)) return LECO_ERR_INVALID_ARG;
@@ -81,7 +82,7 @@ extern "C" leco_status leco_encode_fixed_noalloc(const void* d_values, uint64_t 
   e = launch_build_aux(rec, nullptr, m, n, aux, nullptr, total, static_cast<uint64_t*>(d_words), nwords, nullptr, st);
   if (e == cudaSuccess)
     e = launch_pack(d_values, dtype, L, nullptr, rec, aux, nullptr, nullptr, m, n,
-                    static_cast<uint64_t*>(d_words), st);
+                    (uint32_t)hres[1], static_cast<uint64_t*>(d_words), st);
   // the buffers are complete when the call returns (and the shared scratch free for the next call)
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   return e == cudaSuccess ? LECO_OK : LECO_ERR_CUDA;
