@@ -1,5 +1,6 @@
-"""The packer's rows of 64-bit entries for widths above 32 bits, at the lengths where they take over. Records and
-words equal the oracle's."""
+"""The encoder's paths for short partitions (a lane packs each, a tile of eight lanes fits each) and for widths
+above 32 bits (rows of 64-bit entries), at the lengths where one path takes over from another. Records and words
+equal the oracle's."""
 import numpy as np
 import pytest
 
@@ -40,6 +41,19 @@ def _check(lc, lens, v, bits, model):
     rec_b, words_b, _ = lc.leco_column_export(col)
     rec, words = oracle.encode(v, starts, model)
     assert rec_b == rec.tobytes() and words_b == words.tobytes()
+
+
+@pytest.mark.parametrize("bits,top", [(64, 62), (32, 31)])
+@pytest.mark.parametrize("model", [0, 1])
+def test_many_short_partitions(lc, model, bits, top):
+    """Enough partitions for four at a time per warp: groups of short ones, groups with a long one (256, 257, 3000
+    values), a last group of one to three."""
+    g = W.rng(120)
+    for tail in (0, 1, 2, 3):
+        lens = g.integers(1, 12, size=160_000 + tail)
+        at = g.integers(0, len(lens), size=300)
+        lens[at] = g.choice([255, 256, 257, 3000], size=300)
+        _check(lc, lens, _column(lens, top, 121 + tail, bits), bits, model)
 
 
 @pytest.mark.parametrize("bits", [33, 34, 47, 62, 63, 64])
