@@ -786,13 +786,59 @@ __device__ __forceinline__ void pack_block(const PolyCoef& pc, uint64_t off0, ui
   if (o) atomicOr(w + 1, h >> (32u - o));
 }
 
+// A whole partition on a line by one lane: its bits strung together from the place of its first one, whole words
+// stored, the shared ones at its ends OR-ed into. For short ones (lane_part_of, and at most kLaneBits bits: beyond
+// them the words of 32 lanes are too far apart); a warp spends about 600 instructions on each.
+template <typename T>
+__device__ __forceinline__ void pack_lane(const T* __restrict__ v, uint32_t N, const Aux& a, uint32_t* __restrict__ words) {
+  const uint32_t b = w3_b(a.word3);
+  if (b == 0) return;
+  const uint64_t off = w3_off(a.word3);
+  const int32_t sr = w3_s(a.word3);
+  const uint32_t sh = sr > 0 ? (uint32_t)sr & 63u : 0u;
+  uint32_t* out = words + (off >> 5);
+  uint32_t fill = (uint32_t)off & 31u, acc = 0;
+  bool shared = fill != 0;  // the first word holds another partition's bits too
+  auto emit = [&](uint32_t x, uint32_t width) {
+    const uint64_t t = ((uint64_t)x << fill) | acc;
+    acc = (uint32_t)t;
+    fill += width;
+    if (fill >= 32u) {
+      if (shared)
+        atomicOr(out, acc);
+      else
+        *out = acc;
+      shared = false;
+      out++;
+      acc = (uint32_t)(t >> 32);
+      fill -= 32u;
+    }
+  };
+  uint64_t F = (uint64_t)a.A;
+  for (uint32_t x = 0; x < N; x += 4) {
+    T val[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) val[k] = x + k < N ? __ldg(v + x + k) : (T)0;
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+      if (x + k < N) {
+        const uint64_t z = zz_encode((int64_t)((uint64_t)val[k] - (uint64_t)((int64_t)F >> sh)));
+        F += (uint64_t)a.B;
+        emit((uint32_t)z, min(b, 32u));
+        if (b > 32) emit((uint32_t)(z >> 32), b - 32u);
+      }
+    }
+  }
+  if (fill) atomicOr(out, acc);
+}
+
 // positions [pos, end) of a column, partition p holding pos
-template <typename T, bool POLY, bool WIDE>
+template <typename T, bool POLY, bool SHORT, bool WIDE>
 __device__ __forceinline__ void pack_window(const T* __restrict__ values, uint64_t n, uint64_t m, uint64_t pos,
                                             uint64_t end, uint64_t p, const Record* __restrict__ rec,
                                             const Aux* __restrict__ aux, const PolyCoef* __restrict__ pcoef,
                                             const PolyAux* __restrict__ poly, uint32_t* __restrict__ words,
-                                            uint64_t* zbuf, uint32_t lane) {
+                                            uint64_t* zbuf, uint32_t lane, uint32_t lane_part) {
   // the lanes fetch 32 entries at a time (one memory round trip for a run of short partitions)
   while (pos < end) {
     Aux mine;
@@ -800,7 +846,25 @@ __device__ __forceinline__ void pack_window(const T* __restrict__ values, uint64
     mine.word3 = 0;
     mine.start = n;
     if (p + lane < m) mine = aux[p + lane];
+    uint32_t lanes = 0;  // short partitions that lie inside the window whole: a lane each, all at once
+    if (SHORT) {
+      const uint64_t next = __shfl_down_sync(0xffffffffu, mine.start, 1);
+      lanes = __ballot_sync(0xffffffffu, lane < 31 && mine.start >= pos && mine.start < next && next <= end &&
+                                             next - mine.start <= lane_part && w3_exact(mine.word3) &&
+                                             (next - mine.start) * w3_b(mine.word3) <= kLaneBits);
+      if (__popc(lanes) < 2)
+        lanes = 0;
+      else if ((lanes >> lane) & 1u)
+        pack_lane(values + mine.start, (uint32_t)(next - mine.start), mine, words);
+    }
     for (uint32_t k = 0; k < 31 && pos < end; k++, p++) {
+      if (SHORT && ((lanes >> k) & 1u)) {  // on to the next partition that is left
+        const uint32_t run = (uint32_t)__ffs((int)~(lanes >> k)) - 1u;
+        pos = __shfl_sync(0xffffffffu, mine.start, k + run);
+        k += run - 1u;
+        p += run - 1u;
+        continue;
+      }
       Aux a;
       a.A = __shfl_sync(0xffffffffu, mine.A, k);
       a.B = __shfl_sync(0xffffffffu, mine.B, k);
@@ -820,12 +884,12 @@ __device__ __forceinline__ void pack_window(const T* __restrict__ values, uint64
 // slower beside those rows). L: the fixed partition length, or 0: partitions of any lengths, found through the scan
 // tiles. Every `period`
 // positions hold `per` windows, the last one shorter where they do not divide it.
-template <typename T, bool POLY, bool WIDE>
+template <typename T, bool POLY, bool SHORT, bool WIDE>
 __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
     k_pack(const T* __restrict__ values, uint64_t n, uint64_t m, uint32_t L, uint32_t window, uint32_t period,
            uint32_t per, const TileDesc* __restrict__ tiles, const Record* __restrict__ rec,
            const Aux* __restrict__ aux, const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly,
-           uint32_t* __restrict__ words) {
+           uint32_t* __restrict__ words, uint32_t lane_part) {
   __shared__ uint64_t zbuf[kPackWarps][kPackTile / 2];
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   const uint64_t nwin = (n + period - 1) / period * per, nw = (uint64_t)gridDim.x * kPackWarps;
@@ -848,7 +912,8 @@ __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
           hi = mid;
       }
     }
-    pack_window<T, POLY, WIDE>(values, n, m, pos, end, p, rec, aux, pcoef, poly, words, zbuf[wid], lane);
+    pack_window<T, POLY, SHORT, WIDE>(values, n, m, pos, end, p, rec, aux, pcoef, poly, words, zbuf[wid], lane,
+                                  lane_part);
   }
 }
 
@@ -948,12 +1013,13 @@ __global__ void k_aux_multi(const Record* __restrict__ rec, const PolyCoef* __re
 }
 
 // k_pack over the columns of a batch: win_base[c] windows before column c's
-template <typename T, bool POLY>
+template <typename T, bool POLY, bool SHORT>
 __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
     k_pack_multi(const EncCol* __restrict__ cols, const uint64_t* __restrict__ part_base,
                  const uint64_t* __restrict__ win_base, const uint64_t* __restrict__ word_base, uint32_t ncols,
                  uint64_t windows, uint32_t window, const Record* __restrict__ rec, const Aux* __restrict__ aux,
-                 const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly, uint64_t* __restrict__ words) {
+                 const PolyCoef* __restrict__ pcoef, const PolyAux* __restrict__ poly, uint64_t* __restrict__ words,
+                 uint32_t lane_part) {
   __shared__ uint64_t zbuf[kPackWarps][kPackTile / 2];
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
   const uint64_t nw = (uint64_t)gridDim.x * kPackWarps;
@@ -962,9 +1028,9 @@ __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
     const EncCol col = cols[c];
     const uint64_t pos = (k - win_base[c]) * window;
     const uint64_t p0 = part_base[c];
-    pack_window<T, POLY, true>(static_cast<const T*>(col.values), col.n, part_base[c + 1] - p0, pos, min(pos + window, col.n),
+    pack_window<T, POLY, SHORT, true>(static_cast<const T*>(col.values), col.n, part_base[c + 1] - p0, pos, min(pos + window, col.n),
                          pos / col.L, rec + p0, aux + p0, POLY ? pcoef + p0 : nullptr, POLY ? poly + p0 : nullptr,
-                         reinterpret_cast<uint32_t*>(words + word_base[c]), zbuf[wid], lane);
+                         reinterpret_cast<uint32_t*>(words + word_base[c]), zbuf[wid], lane, lane_part);
   }
 }
 
@@ -1150,10 +1216,13 @@ cudaError_t launch_pack_t(const void* values, uint64_t n, uint64_t m, uint32_t L
     per = (uint32_t)(((uint64_t)period + window - 1) / window);
   }
   const uint64_t nwin = (n + period - 1) / period * per;
-  auto kern = max_b > 32 ? k_pack<T, POLY, true> : k_pack<T, POLY, POLY>;
+  const uint32_t lane_part = POLY ? 0u : lane_part_of(n / m, window, max_b);
+  const bool wide = max_b > 32;
+  auto kern = lane_part ? (wide ? k_pack<T, POLY, !POLY, true> : k_pack<T, POLY, !POLY, POLY>)
+                        : (wide ? k_pack<T, POLY, false, true> : k_pack<T, POLY, false, POLY>);
   kern<<<grid_for(nwin, kPackWarps, 8), kPackBlock, 0, st>>>(
       static_cast<const T*>(values), n, m, L, window, period, per, tiles, rec, aux, pcoef, poly,
-      reinterpret_cast<uint32_t*>(words));
+      reinterpret_cast<uint32_t*>(words), lane_part);
   return cudaGetLastError();
 }
 
@@ -1232,27 +1301,29 @@ cudaError_t launch_word_bases(const uint64_t* col_bits, uint32_t ncols, uint64_t
 
 template <typename T, bool POLY>
 cudaError_t launch_pack_multi_t(const EncCol* cols, const uint64_t* part_base, const uint64_t* win_base,
-                                const uint64_t* word_base, uint32_t ncols, uint64_t windows, uint32_t window,
+                                const uint64_t* word_base, uint32_t ncols, uint64_t windows, uint32_t window, uint32_t lane_part,
                                 const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                                 uint64_t* words, cudaStream_t st) {
-  k_pack_multi<T, POLY><<<grid_for(windows, kPackWarps, 8), kPackBlock, 0, st>>>(
-      cols, part_base, win_base, word_base, ncols, windows, window, rec, aux, pcoef, poly, words);
+  auto kern = lane_part ? k_pack_multi<T, POLY, !POLY> : k_pack_multi<T, POLY, false>;
+  kern<<<grid_for(windows, kPackWarps, 8), kPackBlock, 0, st>>>(
+      cols, part_base, win_base, word_base, ncols, windows, window, rec, aux, pcoef, poly, words, lane_part);
   return cudaGetLastError();
 }
 
 cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* win_base,
-                              const uint64_t* word_base, uint32_t ncols, uint64_t windows, int dtype, uint32_t window,
+                              const uint64_t* word_base, uint32_t ncols, uint64_t windows, int dtype, uint32_t window, uint64_t mean,
                               const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                               uint64_t* words, cudaStream_t st) {
   if (windows == 0) return cudaSuccess;
+  const uint32_t lp = pcoef ? 0u : lane_part_of(mean, window, 0);
   if (dtype == LECO_U32)
-    return pcoef ? launch_pack_multi_t<uint32_t, true>(cols, part_base, win_base, word_base, ncols, windows, window, rec,
+    return pcoef ? launch_pack_multi_t<uint32_t, true>(cols, part_base, win_base, word_base, ncols, windows, window, lp, rec,
                                                        aux, pcoef, poly, words, st)
-                 : launch_pack_multi_t<uint32_t, false>(cols, part_base, win_base, word_base, ncols, windows, window,
+                 : launch_pack_multi_t<uint32_t, false>(cols, part_base, win_base, word_base, ncols, windows, window, lp,
                                                         rec, aux, nullptr, nullptr, words, st);
-  return pcoef ? launch_pack_multi_t<uint64_t, true>(cols, part_base, win_base, word_base, ncols, windows, window, rec,
+  return pcoef ? launch_pack_multi_t<uint64_t, true>(cols, part_base, win_base, word_base, ncols, windows, window, lp, rec,
                                                      aux, pcoef, poly, words, st)
-               : launch_pack_multi_t<uint64_t, false>(cols, part_base, win_base, word_base, ncols, windows, window, rec,
+               : launch_pack_multi_t<uint64_t, false>(cols, part_base, win_base, word_base, ncols, windows, window, lp, rec,
                                                       aux, nullptr, nullptr, words, st);
 }
 

@@ -346,6 +346,7 @@ struct EncBatch {
   std::vector<uint64_t> part_base, tile_base;
   std::vector<uint64_t> bases;  // part_base | tile_base | first packer window of each column
   uint32_t window = 0;          // positions per packer window
+  uint64_t mean = 0;            // values per partition
   uint64_t P = 0, T = 0;
   uint64_t fit_values = 0;  // the constant and linear columns: values, longest partition
   uint32_t longest = 0;
@@ -370,6 +371,7 @@ struct EncBatch {
     for (uint32_t c = 0; c < ncols; c++) values += n[c];
     if (item_values < 1024 || item_values > kScanTile || kScanTile % item_values) item_values = (uint32_t)kScanTile;
     window = pack_window(values, item_values, kPackWindowMin, sm_count() * 32);
+    mean = P ? values / P : 0;
     bases = part_base;
     bases.insert(bases.end(), tile_base.begin(), tile_base.end());
     bases.push_back(0);
@@ -535,8 +537,8 @@ leco_status batch_encode_cfg(const void* const* d_vals, const uint64_t* n, const
   if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, d_ec, d_part, p.part_col, d_word, p.colbits, ncols, P, p.aux, p.poly, words, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(d_views, d_tile, ncols, T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(d_ec, d_part, d_win, d_word, ncols, B.bases.back(), dtype, B.window, p.rec, p.aux, p.pcoef,
-                          p.poly, words, st);
+    e = launch_pack_multi(d_ec, d_part, d_win, d_word, ncols, B.bases.back(), dtype, B.window, B.mean, p.rec, p.aux,
+                          p.pcoef, p.poly, words, st);
   if (e == cudaSuccess) e = make_batch_columns(B, p, words, word_base, col_bits, max_b, models, L, dev, st, meta, out);
   cudaFreeAsync(scr, st);
   cudaFreeAsync(d_ec, st);
@@ -610,8 +612,8 @@ cudaError_t enc_plan_launches(leco_batch_encode_plan* pl, cudaStream_t st) {
   if (e == cudaSuccess) e = launch_aux_multi(p.rec, p.pcoef, pl->d_ec, d_part, p.part_col, d_word, p.colbits, B.ncols, B.P, p.aux, p.poly, pl->words, st);
   if (e == cudaSuccess) e = launch_tile_desc_multi(pl->d_views, d_tile, B.ncols, B.T, B.any_poly, p.tiles, st);
   if (e == cudaSuccess)
-    e = launch_pack_multi(pl->d_ec, d_part, d_win, d_word, B.ncols, B.bases.back(), B.dtype, B.window, p.rec, p.aux,
-                          p.pcoef, p.poly, pl->words, st);
+    e = launch_pack_multi(pl->d_ec, d_part, d_win, d_word, B.ncols, B.bases.back(), B.dtype, B.window, B.mean, p.rec,
+                          p.aux, p.pcoef, p.poly, pl->words, st);
   return e;
 }
 

@@ -306,10 +306,11 @@ cudaError_t launch_aux_multi(const Record* rec, const PolyCoef* pcoef, const Enc
 // word_base[c] = sum of stream_words(col_bits[k]) over k < c, for c = 0 .. ncols, on the device (one
 // CTA): each column's packed stream placed right after the previous one
 cudaError_t launch_word_bases(const uint64_t* col_bits, uint32_t ncols, uint64_t* word_base, cudaStream_t st);
-// window: positions a warp packs at a time; windows: of all columns, win_base[c] of them before column c's
+// window: positions a warp packs at a time; windows: of all columns, win_base[c] of them before column c's;
+// mean: values per partition
 cudaError_t launch_pack_multi(const EncCol* cols, const uint64_t* part_base, const uint64_t* win_base,
                               const uint64_t* word_base, uint32_t ncols, uint64_t windows, int dtype, uint32_t window,
-                              const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
+                              uint64_t mean, const Record* rec, const Aux* aux, const PolyCoef* pcoef, const PolyAux* poly,
                               uint64_t* words, cudaStream_t st);
 // poly: some column has a polynomial table (its tiles then get the exact polynomial bounds)
 cudaError_t launch_tile_desc_multi(const ColumnView* views, const uint64_t* tile_base, uint32_t ncols, uint64_t T,

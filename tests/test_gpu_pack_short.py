@@ -43,6 +43,20 @@ def _check(lc, lens, v, bits, model):
     assert rec_b == rec.tobytes() and words_b == words.tobytes()
 
 
+@pytest.mark.parametrize("bits,top", [(64, 63), (64, 20), (32, 31)])
+@pytest.mark.parametrize("model", [0, 1])
+@pytest.mark.parametrize("edge", [(1, 2, 3, 4), (31, 32, 33, 34), (63, 64, 65, 66), (126, 127, 128, 129, 130)])
+def test_edges_of_the_lane_path(lc, edge, model, bits, top):
+    """Lengths about the limits, with a long partition now and then so that windows cut some, over means below 96,
+    up to 224 and above; 64 values of 33 bits and more go beyond a lane's bits."""
+    g = W.rng(100 + len(edge))
+    for every, count in ((0, 3000), (40, 2000), (9, 600)):
+        lens = g.choice(edge, size=count)
+        if every:
+            lens[::every] = g.integers(900, 5000, size=len(lens[::every]))
+        _check(lc, lens, _column(lens, top, 110 + every, bits), bits, model)
+
+
 @pytest.mark.parametrize("bits,top", [(64, 62), (32, 31)])
 @pytest.mark.parametrize("model", [0, 1])
 def test_many_short_partitions(lc, model, bits, top):
@@ -74,4 +88,14 @@ def test_32_bit_values_with_wide_residuals(lc):
         col = lc.leco_encode(to_dev(v, 32), lc.fixed(L), 1)
         rec_b, words_b, _ = lc.leco_column_export(col)
         rec, words = oracle.encode_fixed(v, L, 1)
+        assert rec_b == rec.tobytes() and words_b == words.tobytes()
+
+
+def test_short_partitions_in_a_batch(lc):
+    shapes = [(50_001, 1, 0), (40_000, 4, 1), (30_011, 33, 1), (3000, 128, 0), (20_000, 129, 1), (700, 3000, 1)]
+    vals = [W.random_u64(n, 150 + k, bits=5 + 11 * k) for k, (n, _, _) in enumerate(shapes)]
+    cols = lc.leco_batch_encode([to_dev(v) for v in vals], [m for _, _, m in shapes], [L for _, L, _ in shapes])
+    for col, v, (_, L, model) in zip(cols, vals, shapes):
+        rec_b, words_b, _ = lc.leco_column_export(col)
+        rec, words = oracle.encode_fixed(v, L, model)
         assert rec_b == rec.tobytes() and words_b == words.tobytes()

@@ -90,3 +90,11 @@ def test_long_partitions_are_dealt_out(run):
       {{16000000, 1024}}, {{50000000, 4096}}, {{100000000, 2048}}, {{100000000, 1000}}, {{200000000, 4096}}, {{1ull << 40, 1u << 24}}}};
   for (auto c : cases) printf("%u ", fit_parts(c.values, {pairs}, c.longest, 512));""")
     assert got == [1, 1, 8, 8, 2, 4, 1, 1, 1, 1]
+
+
+def test_lanes_by_mean_and_window(run):
+    got = run("lanes", """
+  for (uint64_t mean : {0ull, 1ull, 96ull, 97ull, 224ull, 225ull, 1ull << 24})
+    printf("%u %u ", lane_part_of(mean, 4096, 13), lane_part_of(mean, 256, 0));""")
+    assert got == [128, 32] * 3 + [32, 32] * 2 + [0, 0] * 2
+    assert run("wide", 'printf("%u %u", lane_part_of(48, 4096, 64), lane_part_of(49, 4096, 64));') == [128, 0]
