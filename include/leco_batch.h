@@ -117,9 +117,9 @@ leco_status leco_batch_encode(const void* const* d_vals, const uint64_t* n, cons
 
 /* Shape of the batched encode (a systems knob; the paper has no counterpart): values per pack item
  * (1024, 2048 or 4096: the window of consecutive positions of one column that a warp of the packer
- * takes at a time) and fit CTAs per SM (2, 3 or 4: fewer keep more of each
- * partition in L2 between the fit's two passes, more hide the exact solve's latency); ms is the
- * measured time of the chosen shape (leco_tune_batch_encode only). */
+ * takes at a time, fewer in a small batch) and fit CTAs per SM (2 keeps more of each partition in L2
+ * between the fit's two passes; 3 hides more of the exact solve's latency; a table that says 4 means
+ * the same); ms is the measured time of the chosen shape (leco_tune_batch_encode only). */
 typedef struct {
   uint32_t item_values;
   uint32_t fit_ctas;

@@ -1132,22 +1132,18 @@ void launch_fit_tiles(const T* values, uint64_t n, const uint64_t* starts, uint3
 
 cudaError_t launch_fit(const void* values, int dtype, uint64_t n, const uint64_t* starts,
                        uint32_t L, uint64_t m, int model, Record* rec, uint64_t* lenbits, PolyCoef* pcoef,
-                       uint32_t* max_b, uint32_t* err, cudaStream_t st) {
-  (void)err;  // the fit waits on nothing
+                       uint32_t* max_b, cudaStream_t st) {
   if (model == LECO_MODEL_POLY && !pcoef) return cudaErrorInvalidValue;
   cudaError_t e = cudaMemsetAsync(max_b, 0, sizeof(uint32_t), st);
   if (e != cudaSuccess || m == 0) return e;
   if (model == LECO_MODEL_POLY) return launch_poly_fit(OneColumn{values, n, starts, L}, dtype, m, rec, lenbits, pcoef,
                                                         max_b, st);
-  // fit CTAs per SM: the encode shape of the tuning table for this value width (fewer keep more of
-  // each partition in L2 between the two passes)
   const uint32_t fc = encode_config_lookup(dtype).fit_ctas;
-  const int ctas = fc >= 1 && fc <= (uint32_t)kFitCtasPerSm ? (int)fc : kFitCtasPerSm;
+  const int ctas = fit_ctas_of(fc, kFitCtasPerSm);
   // partitions of at least 1024 values: two warps each (the second pass then stays in L2)
   if (!starts && L >= 1024) {
-    k_fit_pairs<<<grid_for((m + kFitPairs - 1) / kFitPairs, 1, ctas < kPairCtas ? ctas : kPairCtas), kFitBlock, 0, st>>>(values, dtype, n, starts,
-                                                                                        L, m, model, rec, lenbits,
-                                                                                        max_b);
+    k_fit_pairs<<<grid_for((m + kFitPairs - 1) / kFitPairs, 1, fit_ctas_of(fc, kPairCtas)), kFitBlock, 0, st>>>(
+        values, dtype, n, starts, L, m, model, rec, lenbits, max_b);
     return cudaGetLastError();
   }
   if (dtype == LECO_U32)
@@ -1253,8 +1249,7 @@ cudaError_t launch_fit_multi(const EncCol* cols, const uint64_t* part_base, cons
                              void* poly_scratch) {
   cudaError_t e = cudaMemsetAsync(max_b, 0, sizeof(uint32_t) * (ncols ? ncols : 1), st);
   if (e != cudaSuccess || P == 0) return e;
-  const int ctas = fit_ctas >= 1 && fit_ctas <= (uint32_t)kFitCtasPerSm ? (int)fit_ctas : kFitCtasPerSm;
-  const int per_sm = ctas < kPairCtas ? ctas : kPairCtas;
+  const int per_sm = fit_ctas_of(fit_ctas, kPairCtas);
   const uint32_t parts = fit_parts(values, (uint64_t)sm_count() * per_sm * kFitPairs, longest, kFitTileVals);
   const int grid = grid_for((P + 7) / 8 * parts, kFitPairs, per_sm);
   if (dtype == LECO_U32)

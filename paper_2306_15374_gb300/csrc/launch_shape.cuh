@@ -68,4 +68,10 @@ inline uint32_t fit_parts(uint64_t values, uint64_t pairs, uint32_t longest, uin
   return parts;
 }
 
+// CTAs per SM of a fit, at most `most` (what its registers allow): 2 where the tuning table asks for it (fewer keep
+// more of each partition in L2 for the second pass), else as many as there can be. The batched fit holds three, so that
+// 3 and 4 are the same to it, and the tuner tries only what differs.
+constexpr uint32_t kFitCtasTried[] = {2, 3};
+inline int fit_ctas_of(uint32_t asked, int most) { return asked == 2 && most > 2 ? 2 : most; }
+
 }  // namespace leco

@@ -111,8 +111,7 @@ leco_status encode_partitions(leco_column* c, const void* d_values, cudaStream_t
   if (prefit)
     e = launch_lenbits(c->rec, starts, m, lenbits, d_maxb, st);
   else
-    e = launch_fit(d_values, c->dtype, c->n, starts, c->L, m, c->model, c->rec, lenbits, pcoef, d_maxb, c->status,
-                   st);
+    e = launch_fit(d_values, c->dtype, c->n, starts, c->L, m, c->model, c->rec, lenbits, pcoef, d_maxb, st);
   if (e == cudaSuccess)
     e = launch_offsets(c->rec, lenbits, m, off_scr, offsets_scratch_elems(m), d_total, st);
   if (e == cudaSuccess) e = cudaMemcpyAsync(hres, d_total, 16, cudaMemcpyDeviceToHost, st);

@@ -638,12 +638,12 @@ extern "C" leco_status leco_tune_batch_encode(const void* const* d_vals, const u
     return LECO_ERR_CUDA;
   }
   leco_status s = LECO_OK;
-  EncodeConfig win{4096, 4};
+  EncodeConfig win{4096, 3};
   float win_ms = -1.f;
-  const uint32_t items[3] = {1024, 2048, 4096}, ctas[3] = {2, 3, 4};
+  const uint32_t items[3] = {1024, 2048, 4096};
   for (int rep = 0; rep < 2 && s == LECO_OK; rep++) {  // the first pass warms pools and modules
     for (uint32_t iv : items)
-      for (uint32_t fc : ctas) {
+      for (uint32_t fc : kFitCtasTried) {
         if (s != LECO_OK) break;
         const EncodeConfig cfg{iv, fc};
         if (cudaEventRecord(e0, st) != cudaSuccess) s = LECO_ERR_CUDA;

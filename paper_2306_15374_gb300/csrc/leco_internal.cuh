@@ -330,8 +330,8 @@ __device__ __forceinline__ uint32_t find_col(const uint64_t* __restrict__ base, 
 }
 
 // Shape of the batched encode: values per pack item (a warp's window of positions: 1024, 2048 or 4096)
-// and fit CTAs per SM (2, 3 or 4; fewer keep more of each partition in L2 for
-// the fit's second pass). Tuned per value width by leco_tune_batch_encode.
+// and fit CTAs per SM (2: more of each partition stays in L2 for the fit's second pass; 3 or 4: as many as there
+// can be). Tuned per value width by leco_tune_batch_encode.
 struct EncodeConfig {
   uint32_t item_values;
   uint32_t fit_ctas;
@@ -349,7 +349,7 @@ void scan_config_store(int op, int dtype, uint32_t stage_bytes, ScanConfig cfg);
 // polynomial decode table; both nullptr for constant and linear columns.
 cudaError_t launch_fit(const void* values, int dtype, uint64_t n, const uint64_t* starts,
                        uint32_t L, uint64_t m, int model, Record* rec, uint64_t* lenbits, PolyCoef* pcoef,
-                       uint32_t* max_b, uint32_t* err, cudaStream_t st);
+                       uint32_t* max_b, cudaStream_t st);
 cudaError_t launch_offsets(Record* rec, const uint64_t* lenbits, uint64_t m, uint64_t* scratch,
                            uint64_t scratch_elems, uint64_t* total_out, cudaStream_t st);
 uint64_t offsets_scratch_elems(uint64_t m);

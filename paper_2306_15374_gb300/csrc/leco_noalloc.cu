@@ -68,7 +68,7 @@ extern "C" leco_status leco_encode_fixed_noalloc(const void* d_values, uint64_t 
   Record* rec = static_cast<Record*>(d_records);
   // every scratch word this call reads is written first by this call (launch_fit zeroes max b)
   cudaError_t e = launch_fit(d_values, dtype, n, nullptr, L, m, model, rec, lenbits, nullptr,
-                             reinterpret_cast<uint32_t*>(res + 1), nullptr, st);
+                             reinterpret_cast<uint32_t*>(res + 1), st);
   if (e == cudaSuccess) e = launch_offsets(rec, lenbits, m, off_scr, offsets_scratch_elems(m), res, st);
   uint64_t hres[2] = {0, 0};
   const uint64_t& total = hres[0];

@@ -47,7 +47,7 @@ EncodeConfig encode_config_lookup(int dtype) {
   std::lock_guard<std::mutex> lock(g_mu);
   auto it = g_enc.find(dtype);
   if (it != g_enc.end()) return it->second;
-  return EncodeConfig{4096, 4};  // untuned default: the largest items, four fit CTAs per SM
+  return EncodeConfig{4096, 3};  // untuned default: the largest items, as many fit CTAs as there can be
 }
 
 void encode_config_store(int dtype, EncodeConfig cfg) {

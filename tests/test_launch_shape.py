@@ -98,3 +98,13 @@ def test_lanes_by_mean_and_window(run):
     printf("%u %u ", lane_part_of(mean, 4096, 13), lane_part_of(mean, 256, 0));""")
     assert got == [128, 32] * 3 + [32, 32] * 2 + [0, 0] * 2
     assert run("wide", 'printf("%u %u", lane_part_of(48, 4096, 64), lane_part_of(49, 4096, 64));') == [128, 0]
+
+
+def test_tried_fit_shapes_differ(run):
+    """The tuner times no two shapes that start the same launch, and an older table's 4 is its 3."""
+    got = run("ctas", """
+  for (int most : {3, 4})
+    for (uint32_t asked : {0u, 1u, 2u, 3u, 4u, 5u}) printf("%d ", fit_ctas_of(asked, most));
+  for (uint32_t c : kFitCtasTried) printf("%d ", fit_ctas_of(c, 3));""")
+    assert got[:6] == [3, 3, 2, 3, 3, 3] and got[6:12] == [4, 4, 2, 4, 4, 4]
+    assert len(set(got[12:])) == len(got[12:]) == 2
