@@ -236,7 +236,7 @@ leco_status leco_search_partition_size(const void* d_values, uint64_t n, leco_dt
                                        uint32_t* best_L, uint64_t* best_bits, uint64_t* evals);
 
 /* Failure-detection self-test: one kernel waits on a shared-memory barrier that nothing completes,
- * with the same bounded wait the scan and pack kernels use, limited to limit_us microseconds
+ * with the same bounded wait the scan kernels use, limited to limit_us microseconds
  * (1 .. 1000000). Returns LECO_ERR_TIMEOUT when the wait gave up and reported it (the expected
  * outcome: the device stays usable), LECO_OK if the barrier completed, INVALID_ARG or CUDA on
  * errors. Synchronizes `stream`. A systems facility; the paper has no counterpart. */

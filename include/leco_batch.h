@@ -156,17 +156,15 @@ leco_status leco_batch_encode_plan_create(const void* const* d_vals, const uint6
 
 /* One launch of the plan's graph on `stream`: every column is encoded (§3.1 fit, §3.3 packing)
  * into the plan's blocks, replacing the previous run's result. Runs that overlap on the device race
- * on those blocks. Errors: INVALID_ARG (NULL plan), CUDA; a bounded wait that gave up surfaces at
- * leco_batch_encode_plan_columns. */
+ * on those blocks. Errors: INVALID_ARG (NULL plan), CUDA. */
 leco_status leco_batch_encode_plan_run(leco_batch_encode_plan* plan, leco_stream_t stream);
 
 /* Synchronize `stream` (the stream of the last run), then copy the last run's result out into
  * ncols new columns, out[c] identical to leco_batch_encode's out[c] for the same values: one block
  * of the records, decode table and tile descriptors and one of the packed streams at their exact
  * size, shared by the columns and released when the last of them is freed. The plan is unchanged
- * and may run again. Errors: INVALID_ARG (also before the plan's first run), OOM, TIMEOUT (a
- * bounded wait inside the run gave up; the streams are incomplete and no column is returned),
- * CUDA. Batching layer; the paper has no counterpart. */
+ * and may run again. Errors: INVALID_ARG (also before the plan's first run), OOM, CUDA. Batching
+ * layer; the paper has no counterpart. */
 leco_status leco_batch_encode_plan_columns(leco_batch_encode_plan* plan, leco_stream_t stream, leco_column** out);
 
 /* Device bytes the plan holds (its tables, scratch and reserved words); 0 for NULL. The paper has no

@@ -3,7 +3,7 @@
 // Fit of one partition of N values (w = the value as two's complement int64):
 //  1. exact least-squares slope q = 6S/D, S = sum (2x - (N-1)) (w_x - w_0), D = N (N^2 - 1)
 //     (integer moments reduced across the group in int128; q = 0 for the constant model; the
-//     divisions are exact 128-by-64 long divisions where the divisor allows, see floordiv_i128);
+//     quotients are exact, by the reciprocal of D, see solve_params);
 //  2. magnitude bound U = max|w| + (wmax - wmin) + (ceil|q| + 1) N + 4; bitlen(U) > 62 falls back
 //     to the constant model on the grid 2^11 (residuals taken mod 2^64);
 //  3. grid exponent s = min(52, 52 - bitlen(U)), slope B = round(q 2^s) (half up);
@@ -20,19 +20,13 @@
 namespace leco {
 namespace {
 
-
-
 // (u1 2^64 + u0) / v for u1 < v (so the quotient fits 64 bits), with the remainder: schoolbook
 // long division in base 2^32 after normalising v (Knuth's algorithm D with two quotient digits, in
 // the form of Warren's "divlu", Hacker's Delight §9-4). Each digit is estimated from the top two
 // dividend digits over the top divisor digit and corrected at most twice.
-__host__ __device__ __forceinline__ uint64_t divlu(uint64_t u1, uint64_t u0, uint64_t v, uint64_t* rem) {
+__device__ __forceinline__ uint64_t divlu(uint64_t u1, uint64_t u0, uint64_t v, uint64_t* rem) {
   const uint64_t base = 1ull << 32;
-#ifdef __CUDA_ARCH__
   const int sh = __clzll((long long)v);  // v > 0
-#else
-  const int sh = __builtin_clzll(v);
-#endif
   v <<= sh;
   const uint64_t vn1 = v >> 32, vn0 = v & 0xFFFFFFFFull;
   const uint64_t un32 = sh ? (u1 << sh) | (u0 >> (64 - sh)) : u1;
@@ -56,11 +50,11 @@ __host__ __device__ __forceinline__ uint64_t divlu(uint64_t u1, uint64_t u0, uin
   return q1 * base + q0;
 }
 
-// floor(num / den) for den > 0, exactly. Divisors below 2^64 (every fit of a partition up to 2^21
-// values) take one native 64-bit division when |num| < 2^64 (the common case of short partitions),
-// else two native 64-bit divisions and one 128-by-64 long division; wider divisors use the generic
+// floor(num / den) for den > 0, exactly: what the reciprocals below do not serve (grids coarser than 1,
+// partitions beyond 2^21 values, the Gram norms). Divisors below 2^64 take one native 64-bit division when
+// |num| < 2^64, else two native 64-bit divisions and one 128-by-64 long division; wider divisors use the generic
 // 128-bit routine, whose bit-serial latency would otherwise stall a whole CTA per fitted partition.
-__host__ __device__ __forceinline__ i128 floordiv_i128(i128 num, i128 den) {
+__device__ __forceinline__ i128 floordiv_i128(i128 num, i128 den) {
   if ((den >> 64) == 0 && num != ((i128)1 << 127)) {
     const uint64_t d = (uint64_t)den;
     const bool neg = num < 0;
@@ -81,7 +75,7 @@ __host__ __device__ __forceinline__ i128 floordiv_i128(i128 num, i128 den) {
   return t;
 }
 
-__host__ __device__ __forceinline__ i128 round_half_up_i128(i128 num, i128 den) {  // den > 0
+__device__ __forceinline__ i128 round_half_up_i128(i128 num, i128 den) {  // den > 0
   return floordiv_i128(2 * num + den, 2 * den);
 }
 
@@ -127,26 +121,12 @@ constexpr RecipTable make_recip_table() {
 
 static __device__ const RecipTable kRecip = make_recip_table();
 
-__host__ __device__ __forceinline__ uint64_t mulhi_u64(uint64_t a, uint64_t b) {
-#ifdef __CUDA_ARCH__
-  return __umul64hi(a, b);
-#else
-  return (uint64_t)(((u128)a * b) >> 64);
-#endif
-}
-
-__host__ __device__ __forceinline__ int clz_u64(uint64_t x) {  // x > 0
-#ifdef __CUDA_ARCH__
-  return __clzll((long long)x);
-#else
-  return __builtin_clzll(x);
-#endif
-}
+__device__ __forceinline__ int clz64(uint64_t x) { return __clzll((long long)x); }  // x > 0
 
 // floor((u1 2^64 + u0) / d) for a normalised d with reciprocal v and u1 < d (Moeller & Granlund,
 // algorithm 4)
-__host__ __device__ __forceinline__ uint64_t div_recip(uint64_t u1, uint64_t u0, uint64_t d, uint64_t v) {
-  uint64_t q0 = v * u1, q1 = mulhi_u64(v, u1);
+__device__ __forceinline__ uint64_t div_recip(uint64_t u1, uint64_t u0, uint64_t d, uint64_t v) {
+  uint64_t q0 = v * u1, q1 = __umul64hi(v, u1);
   q0 += u0;
   q1 += u1 + (q0 < u0 ? 1ull : 0ull) + 1ull;
   uint64_t r = u0 - q1 * d;
@@ -157,13 +137,13 @@ __host__ __device__ __forceinline__ uint64_t div_recip(uint64_t u1, uint64_t u0,
   return r >= d ? q1 + 1 : q1;
 }
 
-__host__ __device__ __forceinline__ uint64_t recip_of(uint64_t dn) {  // as the table's entries
+__device__ __forceinline__ uint64_t recip_of(uint64_t dn) {  // as the table's entries
   uint64_t rem;
   return divlu(~dn, ~0ull, dn, &rem);  // (2^128 - 1) - 2^64 dn over dn
 }
 
 // the constant model on the grid 2^11, for partitions whose magnitude bound exceeds 62 bits (step 2)
-__host__ __device__ __forceinline__ FitParams fallback_params(int64_t mx, int64_t mn) {
+__device__ __forceinline__ FitParams fallback_params(int64_t mx, int64_t mn) {
   const uint64_t half = (uint64_t)mx - (uint64_t)mn;  // mx - mn < 2^64
   // mn + ceil((mx - mn) / 2) rounded down to a multiple of 2^11
   const int64_t t = (int64_t)((uint64_t)mn + (half >> 1) + (half & 1ull));
@@ -182,22 +162,18 @@ constexpr uint32_t kFastLen = 1u << 21;  // D(N) < 2^63: the divisions below tak
 // dividend and the magnitude bound are plain words. False when the grid is coarser than 1 (s < 0), which
 // also holds whenever the bound asks for the fallback; solve_params then takes the general way. The merge
 // rounds solve a line per pair: 100M piecewise values 18.95 -> 18.6 ms, k_fit_spans 7.25 -> 7.0 ms.
-__host__ __device__ __forceinline__ bool solve_short(int64_t S, int64_t mx, int64_t mn, uint32_t N, FitParams* P) {
+__device__ __forceinline__ bool solve_short(int64_t S, int64_t mx, int64_t mn, uint32_t N, FitParams* P) {
   const uint64_t amx = (uint64_t)(mx < 0 ? -mx : mx), amn = (uint64_t)(mn < 0 ? -mn : mn);
   const uint64_t base = (amx > amn ? amx : amn) + ((uint64_t)mx - (uint64_t)mn) + 4;
   const bool neg = S < 0;
   const uint64_t a6 = (uint64_t)(neg ? -S : S) * 6;
   const uint64_t d = (uint64_t)N * (N * N - 1);
-  const int sh = clz_u64(d);  // 28 .. 61
+  const int sh = clz64(d);  // 28 .. 61
   const uint64_t dn = d << sh;
-#ifdef __CUDA_ARCH__
   const uint64_t v = kRecip.v[N];
-#else
-  const uint64_t v = recip_of(dn);
-#endif
   const uint64_t t = a6 + (d - 1);
   const uint64_t Q = div_recip(t >> (64 - sh), t << sh, dn, v);
-  const int s = clz_u64(base + (Q + 1) * N) - 12;
+  const int s = clz64(base + (Q + 1) * N) - 12;
   if (s < 0) return false;
   // (2 |6S| 2^s + D or D - 1) / 2D, both sides normalised
   const int k = s + sh;
@@ -218,7 +194,7 @@ __host__ __device__ __forceinline__ bool solve_short(int64_t S, int64_t mx, int6
 // 128-by-64-bit step by the reciprocal of D; a quotient that would not fit puts the bound above
 // 62 bits. Against three 64-bit divisions and 128-bit bounds: partition + encode of 100M piecewise
 // values 35.15 -> 34.50 ms, of 250M 32-bit timestamps 19.82 -> 19.60 ms.
-__host__ __device__ FitParams solve_params(i128 S, int64_t mx, int64_t mn, uint32_t N, bool lin) {
+__device__ FitParams solve_params(i128 S, int64_t mx, int64_t mn, uint32_t N, bool lin) {
   const int64_t lim = (int64_t)1 << 62;
   if (lin && N >= 2 && N <= kRecipLen && S > -((i128)1 << 58) && S < ((i128)1 << 58) && mx < lim && mn > -lim) {
     FitParams P;
@@ -244,13 +220,9 @@ __host__ __device__ FitParams solve_params(i128 S, int64_t mx, int64_t mn, uint3
     } else if (fast) {
       const uint64_t d = (uint64_t)N * ((uint64_t)N * N - 1);
       D = (i128)d;
-      sh = clz_u64(d);  // >= 1
+      sh = clz64(d);  // >= 1
       dn = d << sh;
-#ifdef __CUDA_ARCH__
       v = N <= kRecipLen ? kRecip.v[N] : recip_of(dn);
-#else
-      v = recip_of(dn);
-#endif
       const u128 t = a6 + (d - 1);
       if ((uint64_t)(t >> 64) == 0) {
         Q = div_recip((uint64_t)t >> (64 - sh), (uint64_t)t << sh, dn, v);
@@ -269,10 +241,10 @@ __host__ __device__ FitParams solve_params(i128 S, int64_t mx, int64_t mn, uint3
     if (Q >> 62) return fallback_params(mx, mn);
   }
   // U = base + (Q + 1) N
-  if (mulhi_u64(Q + 1, N)) return fallback_params(mx, mn);
+  if (__umul64hi(Q + 1, N)) return fallback_params(mx, mn);
   const uint64_t g = (Q + 1) * N;
   if ((g >> 62) || ((base + g) >> 62)) return fallback_params(mx, mn);
-  const int eU = 64 - clz_u64(base + g);  // base >= 4
+  const int eU = 64 - clz64(base + g);  // base >= 4
   const int s = 52 - eU;                  // -10 .. 49
   int64_t B = 0;
   if (lin && N == 2) {  // q = S exactly: B = S 2^s, or round(S / 2^-s) half up by a shift
@@ -314,7 +286,7 @@ __device__ __forceinline__ uint32_t finish_width(const FitParams& P, int64_t lo,
   // (2k - 1 and 2k for an even range 2k, 2k + 1 and 2k for an odd one)
   if (s >= 0) return (uint32_t)bitlen_u64((uint64_t)hi - (uint64_t)lo);
   const i128 t = (i128)lo + (((i128)hi - (i128)lo + 1) >> 1);
-  const i128 shift = s >= 0 ? t : (t >> (-s)) * ((i128)1 << (-s));
+  const i128 shift = (t >> (-s)) * ((i128)1 << (-s));
   const int64_t lo2 = (int64_t)((i128)lo - shift), hi2 = (int64_t)((i128)hi - shift);
   return (uint32_t)bitlen_u64(max(zz_encode(lo2), zz_encode(hi2)));
 }
@@ -948,7 +920,7 @@ __device__ __forceinline__ int64_t poly_value_at(const uint32_t* v32, const uint
 
 // phase 1 of a narrow partition of at least kPolyMinLen values by one warp (the result in every lane). The
 // Gram polynomials sum to zero over the partition, so S_j = sum p_j(x) d_x with d_x = w_x - w_0 in 32 bits. A
-// lane's positions x = lane + 32 (4096 c / 32 + k), k < 128, give power sums M_i = sum k^i d (k^3 < 2^21,
+// lane's positions x = c + lane + 32 k, k < 128, give power sums M_i = sum k^i d (k^3 < 2^21,
 // d < 2^30, 128 terms: below 2^58), three 32 x 32 -> 64-bit products per value; with x' = X + 64 k, the lane then
 // expands p_1 = x', p_2 = 3 x'^2 - (N^2 - 1) and p_3 = 5 x'^3 - (3 N^2 - 7) x' in k once per 128 values, in 128 bits.
 // 50M values in partitions of 4096: 262 -> 109 us against three 128-bit products per value.
@@ -1060,8 +1032,10 @@ __device__ PolyPlan poly_plan(const PolyMom& M, uint32_t N) {
 // stepped in 32.32 fixed point (F's forward differences over 32 positions, each truncated to 2^-32) and only the
 // extremes of (w - w_0) - y are kept, 16 instructions per polynomial and value where the exact 128-bit steps take
 // 40. After k steps the truncations add up to less than (C(k,3) + C(k,2) + k + 1) 2^-32; an extreme
-// closer than that to an integer leaves the partition to the exact pass (k < 512: up to 1 in 200 at 16384
-// values, 1 in 6000 at 4096). 50M values in partitions of 4096: 319 -> 183 us.
+// closer than that to an integer leaves the partition to the exact pass. With four extremes (k <= 512) that is up to
+// one partition in 48 at 16384 values and one in 3000 at 4096, and every one whose residuals are whole numbers
+// (values on an integer polynomial without noise), which takes both passes. 50M values in partitions of 4096:
+// 319 -> 183 us.
 template <typename T>
 __device__ __forceinline__ bool poly_ranges_narrow(const T* __restrict__ v, uint32_t N, uint32_t lane, int64_t ref,
                                                    const PolyPlan* __restrict__ plan, PolyRange& R) {

@@ -1872,11 +1872,6 @@ cudaError_t var_partition(const void* values, int dtype, uint64_t n, double tau,
   return var_partition_fit(values, dtype, n, tau, cap, model, seeded, starts_out, m_out, nullptr, st);
 }
 
-cudaError_t var_partition(const void* values, int dtype, uint64_t n, double tau, uint32_t cap,
-                          int model, uint64_t* starts_out, uint64_t* m_out, cudaStream_t st) {
-  return var_partition_fit(values, dtype, n, tau, cap, model, false, starts_out, m_out, nullptr, st);
-}
-
 namespace {
 // lenbits[p] = len_p * b_p and the widest b, from records whose fits are done (variable partitions)
 __global__ void k_lenbits(const Record* __restrict__ rec, const uint64_t* __restrict__ starts, uint64_t m,
