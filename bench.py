@@ -79,8 +79,8 @@ KSCAN_SRCS = [os.path.join(ROOT, "paper_2306_15374_gb300", "csrc", f) for f in (
 # DRAM read + write per decode launch from one ncu capture of this workload (mean of columns a, b, c;
 # see profiles/k_tilescan_decode_filter_fix200M.md), valid only for the kernel sources it was taken on
 # (keyed by their hash).
-DECODE_TRAFFIC = {"sha256": "89f00e7413beb6f3eb0d3adc82aae7e2c0b3ba981762c990f227bec8c9b47259",
-                  "bytes_per_launch": (1893644544 + 1973048320 + 1845314816) / 3}
+DECODE_TRAFFIC = {"sha256": "db5f0089f9dd93c1904c3bd9bd3a5498b367e3d813df23c2a47d9475913319a0",
+                  "bytes_per_launch": (1894198528 + 1973354880 + 1845761024) / 3}
 
 
 def decode_traffic():
