@@ -924,13 +924,16 @@ __global__ void __launch_bounds__(kPackBlock, POLY ? 2 : kPackCtas)
 // when all are short, else both warps on one after another, as k_fit_pairs. PARTS: the groups of long partitions
 // are dealt out in `parts` parts (fit_parts), where whole groups would leave pairs without work or some with far
 // more than others; a column of 5M values in partitions of 4096 kept 153 of the GPU's 1824 pairs busy.
-// This kernel's time, whole groups -> parts: that column 47 -> 12 us, 20 columns of 8M values in all in partitions of
-// 4096 53 -> 20 us, 16 of 16M 32-bit values in partitions of 1024 53 -> 47 us, 60 columns of 50M values in partitions
-// of 256, 1024 and 4096 231 -> 173 us. A path of a warp or of sixteen lanes per partition of 513 .. 1024 values
-// beside these cost the long ones more in registers (84 -> 96 us for 50M values in partitions of 4096).
-constexpr uint32_t kFitTileVals = 512;
+// MID: no partition is longer than kFitMidVals; sixteen lanes each, four at a time, where some are above kFitTileVals.
+// A kernel of its own: beside the long ones' path these tiles cost it more in registers (84 -> 96 us for 50M values in
+// partitions of 4096).
+// This kernel's time, whole groups of long partitions -> parts: that column 47 -> 12 us, 20 columns of 8M values in
+// all in partitions of 4096 53 -> 20 us, 60 columns of 50M values in partitions of 256, 1024 and 4096 231 -> 173 us.
+// Both warps on one after another -> tiles of sixteen: 20 columns of 20M values in partitions of 600 105 -> 49 us (a
+// warp each, formerly: 93), of 100M 32-bit values in partitions of 1000 246 -> 145 us.
+constexpr uint32_t kFitTileVals = 512, kFitMidVals = 1024;
 
-template <typename T, bool PARTS>
+template <typename T, bool PARTS, bool MID>
 __global__ void __launch_bounds__(kFitBlock, kPairCtas)
     k_fit_multi(const EncCol* __restrict__ cols, const uint64_t* __restrict__ part_base,
                 const uint32_t* __restrict__ part_col, uint64_t P, uint32_t parts, Record* __restrict__ rec,
@@ -957,15 +960,23 @@ __global__ void __launch_bounds__(kFitBlock, kPairCtas)
       if (model != LECO_MODEL_POLY) N = (uint32_t)((a + col.L < col.n ? a + col.L : col.n) - a);
       v = static_cast<const T*>(col.values) + a;
     }
-    if (__all_sync(0xffffffffu, N <= kFitTileVals)) {
-      if (PARTS && part) continue;
-      const int k = (int)(rank >> 3);
+    // partitions from, from + 1, ... of the group, a tile of lanes each
+    auto tiles = [&](auto width, int from) {
+      constexpr int TILE = decltype(width)::value;
+      const int k = from + (int)rank / TILE;
       const uint32_t n = __shfl_sync(0xffffffffu, N, k);
       const T* vk = reinterpret_cast<const T*>(__shfl_sync(0xffffffffu, (unsigned long long)v, k));
-      const FitResult R = fit_tile<8>(vk, n, __shfl_sync(0xffffffffu, model, k), rank & 7u);
+      const FitResult R = fit_tile<TILE>(vk, n, __shfl_sync(0xffffffffu, model, k), rank % TILE);
       const uint64_t ak = __shfl_sync(0xffffffffu, a, k);
       const uint32_t ck = __shfl_sync(0xffffffffu, c, k);
-      if ((rank & 7u) == 0 && n) put_fit(R, ak, n, p0 + (uint32_t)k, rec, lenbits, max_b + ck);
+      if (rank % TILE == 0 && n) put_fit(R, ak, n, p0 + (uint32_t)k, rec, lenbits, max_b + ck);
+    };
+    if (__all_sync(0xffffffffu, N <= kFitTileVals)) {
+      if (k0 == 0) tiles(std::integral_constant<int, 8>(), 0);
+      continue;
+    }
+    if constexpr (MID) {
+      for (int k = k0; k < k0 + per; k += 4) tiles(std::integral_constant<int, 16>(), k);
       continue;
     }
     for (int k = k0; k < k0 + per; k++) {
@@ -1250,14 +1261,19 @@ cudaError_t launch_fit_multi(const EncCol* cols, const uint64_t* part_base, cons
   cudaError_t e = cudaMemsetAsync(max_b, 0, sizeof(uint32_t) * (ncols ? ncols : 1), st);
   if (e != cudaSuccess || P == 0) return e;
   const int per_sm = fit_ctas_of(fit_ctas, kPairCtas);
-  const uint32_t parts = fit_parts(values, (uint64_t)sm_count() * per_sm * kFitPairs, longest, kFitTileVals);
+  uint32_t parts = fit_parts(values, (uint64_t)sm_count() * per_sm * kFitPairs, longest, kFitTileVals);
+  const bool mid = longest > kFitTileVals && longest <= kFitMidVals;
+  if (mid && parts > 2) parts = 2;  // four at a time
   const int grid = grid_for((P + 7) / 8 * parts, kFitPairs, per_sm);
+  auto launch = [&](auto value) {
+    using T = decltype(value);
+    auto kern = mid ? k_fit_multi<T, true, true> : parts > 1 ? k_fit_multi<T, true, false> : k_fit_multi<T, false, false>;
+    kern<<<grid, kFitBlock, 0, st>>>(cols, part_base, part_col, P, parts, rec, lenbits, max_b);
+  };
   if (dtype == LECO_U32)
-    (parts > 1 ? k_fit_multi<uint32_t, true> : k_fit_multi<uint32_t, false>)<<<grid, kFitBlock, 0, st>>>(
-        cols, part_base, part_col, P, parts, rec, lenbits, max_b);
+    launch(uint32_t());
   else
-    (parts > 1 ? k_fit_multi<uint64_t, true> : k_fit_multi<uint64_t, false>)<<<grid, kFitBlock, 0, st>>>(
-        cols, part_base, part_col, P, parts, rec, lenbits, max_b);
+    launch(uint64_t());
   e = cudaGetLastError();
   if (e == cudaSuccess && pcoef)
     e = launch_poly_fit(BatchColumns{cols, part_base, ncols}, dtype, P, rec, lenbits, pcoef, max_b, st, poly_scratch);

@@ -31,8 +31,11 @@ CASES = {
     "lengths mixed inside a group": ([(3000, 4096, 1), (700, 64, 0), (1, 1, 1), (0, 8, 1), (5000, 5000, 0), (2600, 513, 1)], 64),
     "models mixed inside a group": ([(2000, 600, 1), (1500, 600, 2), (1300, 700, 0), (400, 100, 2), (900, 900, 1)], 64),
     "32-bit": ([(30_007, 1024, 0), (300, 64, 1), (4097, 2047, 1)], 32),
-    "parts of four": ([(10_001 * 520, 520, 1), (10_000, 500, 0)], 32),
-    "parts of two": ([(20_001 * 520, 520, 0), (10_000, 100, 1)], 32),
+    "up to 1024": ([(5_000, 513, 1), (9_001, 1024, 0), (700, 64, 1), (1, 1, 0), (2500, 600, 2), (3_333, 1023, 1)], 64),
+    "up to 1024, many": ([(12_000_000, 700, 1), (50_000, 1024, 0)], 32),
+    "one above 1024": ([(5_000, 513, 1), (4_100, 1025, 0)], 64),
+    "parts of four": ([(9_000 * 2048, 2048, 1), (10_000, 500, 0)], 32),
+    "parts of two": ([(17_000 * 2048, 2048, 0), (10_000, 100, 1)], 32),
     "small": ([(3000, 64, 1)] * 4, 64),
 }
 
